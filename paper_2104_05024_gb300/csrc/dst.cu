@@ -7,11 +7,12 @@
 //
 // Work arrays are padded to N^d with index 0 of every axis holding the zero
 // Dirichlet value, so every line of the DST-I of length N-1 is a length-N row
-// starting at an aligned address.  Each 1-D DST-I of length N-1 runs in shared
-// memory as: sine pre-fold into a real sequence of length N, complex Stockham
-// FFT of length N/2 (radix 8/4/2/3 butterflies in registers), split into the
-// real DFT, and a prefix sum for the odd outputs.  A block owns a tile of W
-// independent lines laid out [transform index][line] so that every butterfly
+// starting at an aligned address.  Each 1-D DST-I of length N-1 runs as: sine
+// pre-fold into a real sequence of length N, complex FFT of length N/2, split
+// into the real DFT, and a prefix sum for the odd outputs: float64 lines in
+// 64-bit block fixed point (dst_fix.cuh), float32 lines in registers
+// (dst_reg.cuh), lines shorter than 32 by a Stockham FFT in shared memory.  A
+// block owns a tile of W independent lines laid out [transform index][line] so that every butterfly
 // stage is vectorised across the lines (consecutive threads touch consecutive
 // words).  Passes:
 //   x forward  : assembles r = alpha*src + corrections (irregular nodes) while
@@ -31,6 +32,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "dst_fix.cuh"
 #include "dst_reg.cuh"
 #include "ffloat.cuh"
 #include "internal.cuh"
@@ -66,13 +68,21 @@ struct Tile {
   static constexpr int N = N_, W = W_, RS = RS_;
   static constexpr int L = N / 2;
   static constexpr int G = NT / W;
-  // tile, scan totals, twiddles e^{i pi j/N} (2N complex), sines (register path)
-  static constexpr size_t smem_elems = (size_t)N * RS + (size_t)G * W + 4 * N + N;
+  // fixed-point DST of float64 lines, register DST of float32 lines; shorter
+  // lines take the Stockham path in shared memory
+  static constexpr bool FIX = sizeof(T) == 8 && N >= 32;
+  static constexpr bool REG = sizeof(T) == 4 && N >= 32 && N <= 512;
+  // tables and scratch: those of the fixed-point path, or scan totals,
+  // twiddles e^{i pi j/N} (2N complex) and sines (register path)
+  static constexpr size_t mem_elems = FIX ? fixdst::table_words<N>() : (size_t)G * W + 4 * N + N;
+  static constexpr size_t smem_elems = (size_t)N * RS + mem_elems;
+  // resident blocks per SM the registers are budgeted for
+  static constexpr int BLOCKS = FIX ? (N <= 256 ? 2 : 1) : 1;
 };
 
 template <typename T, int N>
 struct WSel {
-  static constexpr int W = sizeof(T) == 8 ? (N >= 384 ? 16 : (N < 32 ? N : 32)) : (N < 32 ? N : 32);
+  static constexpr int W = N < 32 ? N : 32;
 };
 
 template <typename T, int N>
@@ -322,26 +332,44 @@ __device__ __forceinline__ void copy_async(T* dst_smem, const T* src) {
 }
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// float32 tiles of 32 <= N <= 512 lines take the register-resident DST
-template <typename T, int N>
-constexpr bool kRegDst = sizeof(T) == 4 && N >= 32 && N <= 512;
-
 // sines sin(pi j / N) for the register path's pre-fold (imaginary parts of tw)
-template <typename T, int N>
-__device__ __forceinline__ void load_sines(T* sinv, const T* tw_g) {
-  if constexpr (kRegDst<T, N>)
-    for (int i = threadIdx.x; i < N; i += NT) sinv[i] = tw_g[2 * i + 1];
+template <typename C>
+__device__ __forceinline__ void load_sines(typename C::T* sinv, const typename C::T* tw_g) {
+  if constexpr (C::REG)
+    for (int i = threadIdx.x; i < C::N; i += NT) sinv[i] = tw_g[2 * i + 1];
 }
 
-// the DST-I of every column of the tile, rows 1..N-1 (post: map of the
-// outputs, register path only)
-template <typename C, class Post = regdst::Identity>
-__device__ __forceinline__ void dst_tile(typename C::T* s, const typename C::T* tw, const typename C::T* sinv,
-                                         typename C::T* tot, const Post& post = Post()) {
-  if constexpr (kRegDst<typename C::T, C::N>) {
-    regdst::dst1_tile_reg<regdst::Geo<C::N, C::RS>>(s, sinv, reinterpret_cast<const regdst::cf2*>(tw), tot, post);
+// a tile's tables to shared memory mem[C::mem_elems] (before the first barrier)
+template <typename C>
+__device__ __forceinline__ void load_tables(typename C::T* mem, const typename C::T* tw_g) {
+  if constexpr (C::FIX) {
+    fixdst::load_tables<C::N>(reinterpret_cast<fixdst::ll*>(mem), tw_g);
   } else {
-    dst1_tile<C>(s, tw, tot);
+    typename C::T* tw = mem + C::G * C::W;
+    load_twiddles<typename C::T, C::N>(tw, tw_g);
+    load_sines<C>(tw + 4 * C::N, tw_g);
+  }
+}
+
+struct NoPost {
+  template <typename T>
+  __device__ __forceinline__ T operator()(int, T v) const {
+    return v;
+  }
+};
+
+// the DST-I of every column of the tile, rows 1..N-1; post maps the outputs
+// (not on the Stockham path)
+template <typename C, class Post = NoPost>
+__device__ __forceinline__ void dst_tile(typename C::T* s, typename C::T* mem, const Post& post = Post()) {
+  if constexpr (C::FIX) {
+    fixdst::dst1_tile_fix<fixdst::Geo<C::N, C::RS>>(s, reinterpret_cast<fixdst::ll*>(mem), post);
+  } else if constexpr (C::REG) {
+    const typename C::T* tw = mem + C::G * C::W;
+    regdst::dst1_tile_reg<regdst::Geo<C::N, C::RS>>(s, tw + 4 * C::N, reinterpret_cast<const regdst::cf2*>(tw), mem,
+                                                    post);
+  } else {
+    dst1_tile<C>(s, mem + C::G * C::W, mem);
   }
 }
 
@@ -359,11 +387,28 @@ struct DivPost {
   }
 };
 
+// the same in float64: the factor from the table built for this lambda, or
+// divided here (handles without a table)
+struct FactorPost {
+  const double* r;  // table entry of this column's mode 0, row stride n (nullptr: none)
+  int n;
+  const double* mu;
+  double base;      // mu1[p] + mu1[q] - lambda
+  double scale;
+  bool zero;        // boundary column p = 0
+  bool on;
+  __device__ __forceinline__ double operator()(int j, double v) const {
+    if (!on) return v;
+    if (r != nullptr) return v * r[(size_t)j * n];
+    return zero || j == 0 ? 0.0 : v * (scale / (mu[j] + base));
+  }
+};
+
 // ------------------------------------------------------------- x forward
 // Tile: W consecutive lines y0..y0+W-1 of plane z; assembles
 // r = alpha*src + corrections on the fly.
 template <typename T, int N, int DIM>
-__global__ void __launch_bounds__(NT) k_xfwd(T* __restrict__ a, const double* __restrict__ src, double alpha,
+__global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xfwd(T* __restrict__ a, const double* __restrict__ src, double alpha,
                                              const float* __restrict__ src32,
                                              const double* __restrict__ corr, const int32_t* __restrict__ irr,
                                              const int32_t* __restrict__ line_start, const T* __restrict__ tw_g,
@@ -372,11 +417,8 @@ __global__ void __launch_bounds__(NT) k_xfwd(T* __restrict__ a, const double* __
   constexpr int W = C::W, RS = C::RS, n1 = N - 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
-  T* tot = s + N * RS;
-  T* tw = tot + C::G * W;
-  T* sinv = tw + 4 * N;
-  load_twiddles<T, N>(tw, tw_g);
-  load_sines<T, N>(sinv, tw_g);
+  T* mem = s + N * RS;
+  load_tables<C>(mem, tw_g);
   pdl_wait();
   if (skip != nullptr && *skip != 0) return;
   const int y0 = blockIdx.x * W;
@@ -423,7 +465,7 @@ __global__ void __launch_bounds__(NT) k_xfwd(T* __restrict__ a, const double* __
     }
   }
   __syncthreads();
-  dst_tile<C>(s, tw, sinv, tot);
+  dst_tile<C>(s, mem);
   pdl_launch_next();
   const size_t plane = (size_t)z * N * N;
   for (int idx = threadIdx.x; idx < N * W; idx += NT) {
@@ -434,7 +476,7 @@ __global__ void __launch_bounds__(NT) k_xfwd(T* __restrict__ a, const double* __
 
 // ------------------------------------------------------------- x inverse
 template <typename T, int N, int DIM>
-__global__ void __launch_bounds__(NT) k_xinv(T* __restrict__ a, bool keep, double* __restrict__ out,
+__global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ a, bool keep, double* __restrict__ out,
                                              const double* __restrict__ aux, double beta, double gamma,
                                              const T* __restrict__ tw_g, const int* __restrict__ skip,
                                              const float* __restrict__ aux32 = nullptr) {
@@ -442,11 +484,8 @@ __global__ void __launch_bounds__(NT) k_xinv(T* __restrict__ a, bool keep, doubl
   constexpr int W = C::W, RS = C::RS, n1 = N - 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
-  T* tot = s + N * RS;
-  T* tw = tot + C::G * W;
-  T* sinv = tw + 4 * N;
-  load_twiddles<T, N>(tw, tw_g);
-  load_sines<T, N>(sinv, tw_g);
+  T* mem = s + N * RS;
+  load_tables<C>(mem, tw_g);
   pdl_wait();
   if (skip != nullptr && *skip != 0) return;
   const int y0 = blockIdx.x * W;
@@ -458,7 +497,7 @@ __global__ void __launch_bounds__(NT) k_xinv(T* __restrict__ a, bool keep, doubl
   }
   copy_async_wait();
   __syncthreads();
-  dst_tile<C>(s, tw, sinv, tot);
+  dst_tile<C>(s, mem);
   pdl_launch_next();
   if (out == nullptr) {
     if (keep)
@@ -494,19 +533,16 @@ __global__ void __launch_bounds__(NT) k_xinv(T* __restrict__ a, bool keep, doubl
 // plane q = blockIdx.y + qoff.  SOLVE = forward DST, spectral multiply,
 // inverse DST.
 template <typename T, int N, bool SOLVE, int DIM>
-__global__ void __launch_bounds__(NT) k_strided(T* __restrict__ a, size_t row_stride, size_t plane_stride, int qoff,
+__global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_strided(T* __restrict__ a, size_t row_stride, size_t plane_stride, int qoff,
                                                 const T* __restrict__ mu1, T lambda, T scale,
                                                 const T* __restrict__ tw_g, const int* __restrict__ skip,
-                                                const T* __restrict__ rinv = nullptr) {
+                                                const T* __restrict__ rinv, int reps) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
-  T* tot = s + N * RS;
-  T* tw = tot + C::G * W;
-  T* sinv = tw + 4 * N;
-  load_twiddles<T, N>(tw, tw_g);
-  load_sines<T, N>(sinv, tw_g);
+  T* mem = s + N * RS;
+  load_tables<C>(mem, tw_g);
   pdl_wait();
   if (skip != nullptr && *skip != 0) return;
   const int x0 = blockIdx.x * W;
@@ -519,16 +555,31 @@ __global__ void __launch_bounds__(NT) k_strided(T* __restrict__ a, size_t row_st
   copy_async_wait();
   __syncthreads();
   const T muq = DIM == 3 ? mu1[q] : (T)0;
-  if constexpr (kRegDst<T, N>) {
+  if constexpr (C::REG) {
     if (SOLVE) {
       const int p = x0 + (int)(threadIdx.x & 31);
       // mu1 is read from global memory here (L1-resident, N values)
       const DivPost post{mu1, mu1[p] + muq - lambda, scale, p == 0};
-      dst_tile<C>(s, tw, sinv, tot, post);
+      dst_tile<C>(s, mem, post);
     }
-    dst_tile<C>(s, tw, sinv, tot);
+    dst_tile<C>(s, mem);
+  } else if constexpr (C::FIX) {
+    // forward DST with its outputs multiplied by the mode factors as they
+    // are written, then the inverse DST by the same (single inlined) body
+    if constexpr (SOLVE) {
+      const int p = x0 + (int)(threadIdx.x & 31);
+      FactorPost post{rinv != nullptr ? rinv + ((size_t)q * N * N + p) : nullptr, N, mu1, mu1[p] + muq - lambda, scale,
+                      p == 0, true};
+#pragma unroll 1
+      for (int rep = 0; rep < reps; ++rep) {
+        dst_tile<C>(s, mem, post);
+        post.on = false;
+      }
+    } else {
+      dst_tile<C>(s, mem);
+    }
   } else {
-    dst1_tile<C>(s, tw, tot);
+    dst_tile<C>(s, mem);
     if (SOLVE) {
       // the mode factor scale / mu_p from the table built for this lambda
       // (same expression, so the same value), else divided here
@@ -541,7 +592,7 @@ __global__ void __launch_bounds__(NT) k_strided(T* __restrict__ a, size_t row_st
         s[k * RS + c] = v;
       }
       __syncthreads();
-      dst1_tile<C>(s, tw, tot);
+      dst_tile<C>(s, mem);
     }
   }
   pdl_launch_next();
@@ -735,7 +786,7 @@ namespace cg = cooperative_groups;
 template <int N>
 constexpr size_t xy_smem_bytes() {
   using C = Cfg<float, N>;
-  return (2 * (size_t)N * C::RS + (size_t)C::G * C::W + 5 * (size_t)N) * sizeof(float);
+  return (2 * (size_t)N * C::RS + C::mem_elems) * sizeof(float);
 }
 
 // dst[(32 q + lane) RS + j] = src_q[(y0 + j) RS + lane] for every block q of
@@ -775,15 +826,12 @@ __global__ void __launch_bounds__(NT) k_xy_fwd(float* __restrict__ a, const doub
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* sA = reinterpret_cast<float*>(smem_raw);
   float* sB = sA + N * RS;
-  float* tot = sB + N * RS;
-  float* tw = tot + C::G * W;
-  float* sinv = tw + 4 * N;
+  float* mem = sB + N * RS;
   cg::cluster_group cluster = cg::this_cluster();
   // the flag is set before this launch by the stream's previous kernels, so
   // every block of a cluster sees the same value
   const bool skipped = skip != nullptr && *skip != 0;
-  load_twiddles<float, N>(tw, tw_g);
-  load_sines<float, N>(sinv, tw_g);
+  load_tables<C>(mem, tw_g);
   if (skipped) return;
   const int r = (int)cluster.block_rank();
   const int y0 = r * W;
@@ -817,11 +865,11 @@ __global__ void __launch_bounds__(NT) k_xy_fwd(float* __restrict__ a, const doub
     }
   }
   __syncthreads();
-  dst_tile<C>(sA, tw, sinv, tot);
+  dst_tile<C>(sA, mem);
   cluster.sync();
   xy_exchange<N>(cluster, sA, sB, y0);
   cluster.sync();
-  dst_tile<C>(sB, tw, sinv, tot);
+  dst_tile<C>(sB, mem);
   const size_t plane = (size_t)z * N * N;
   for (int idx = threadIdx.x; idx < N * W; idx += NT) {
     const int c = idx % W, y = idx / W;
@@ -840,13 +888,10 @@ __global__ void __launch_bounds__(NT) k_xy_inv(float* __restrict__ a, bool keep,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* sA = reinterpret_cast<float*>(smem_raw);
   float* sB = sA + N * RS;
-  float* tot = sB + N * RS;
-  float* tw = tot + C::G * W;
-  float* sinv = tw + 4 * N;
+  float* mem = sB + N * RS;
   cg::cluster_group cluster = cg::this_cluster();
   const bool skipped = skip != nullptr && *skip != 0;
-  load_twiddles<float, N>(tw, tw_g);
-  load_sines<float, N>(sinv, tw_g);
+  load_tables<C>(mem, tw_g);
   if (skipped) return;
   const int r = (int)cluster.block_rank();
   const int y0 = r * W;
@@ -858,11 +903,11 @@ __global__ void __launch_bounds__(NT) k_xy_inv(float* __restrict__ a, bool keep,
   }
   copy_async_wait();
   __syncthreads();
-  dst_tile<C>(sB, tw, sinv, tot);
+  dst_tile<C>(sB, mem);
   cluster.sync();
   xy_exchange<N>(cluster, sB, sA, y0);
   cluster.sync();
-  dst_tile<C>(sA, tw, sinv, tot);
+  dst_tile<C>(sA, mem);
   if (out == nullptr) {
     if (keep)
       for (int idx = threadIdx.x; idx < N * W; idx += NT) {
@@ -918,6 +963,16 @@ int prep(K kernel, size_t smem) {
   return KFBI_OK;
 }
 
+// a transform pass, chained to its predecessor by programmatic dependent
+// launch; not for handles whose tables the stream has just written (the
+// allocation-free box solve: no mode-factor table either)
+template <typename K, typename... Args>
+cudaError_t launch_pass(kfbi_handle* h, K kernel, dim3 grid, size_t smem, Args... args) {
+  if (h->rinv_ok) return launch_pdl(kernel, grid, dim3(NT), smem, h->stream, args...);
+  kernel<<<grid, NT, smem, h->stream>>>(args...);
+  return cudaGetLastError();
+}
+
 // one strided 3-D pass (mode 0: along y, mode 1: along z); float32 grids of
 // 32 <= N <= 256 go through the TMA-fed persistent kernel
 template <typename T, int N>
@@ -952,29 +1007,18 @@ int launch_strided3(kfbi_handle* h, int mode, bool solve, T* work, const T* mu1,
   const size_t smem = C::smem_elems * sizeof(T);
   const size_t NN = (size_t)N * N;
   dim3 grid(N / C::W, N - 1);
-  if constexpr (sizeof(T) == 4) {
-    cudaError_t e;
-    if (solve) {
-      if ((rc = prep(k_strided<T, N, true, 3>, smem))) return rc;
-      e = launch_pdl(k_strided<T, N, true, 3>, grid, dim3(NT), smem, st, work, (size_t)(mode == 0 ? N : NN),
-                     (size_t)(mode == 0 ? NN : N), 1, mu1, lam, scale, tw, (const int*)h->skip, rinv);
-    } else {
-      if ((rc = prep(k_strided<T, N, false, 3>, smem))) return rc;
-      e = launch_pdl(k_strided<T, N, false, 3>, grid, dim3(NT), smem, st, work, (size_t)(mode == 0 ? N : NN),
-                     (size_t)(mode == 0 ? NN : N), 1, mu1, lam, scale, tw, (const int*)h->skip, (const T*)nullptr);
-    }
-    return e == cudaSuccess ? KFBI_OK : launch_failed("strided pass");
-  }
+  const size_t rs = mode == 0 ? (size_t)N : NN, ps = mode == 0 ? NN : (size_t)N;
+  cudaError_t e;
   if (solve) {
     if ((rc = prep(k_strided<T, N, true, 3>, smem))) return rc;
-    k_strided<T, N, true, 3><<<grid, NT, smem, st>>>(work, mode == 0 ? N : NN, mode == 0 ? NN : N, 1, mu1, lam,
-                                                     scale, tw, h->skip, rinv);
+    e = launch_pass(h, k_strided<T, N, true, 3>, grid, smem, work, rs, ps, 1, mu1, lam, scale, tw, (const int*)h->skip,
+                    rinv, 2);
   } else {
     if ((rc = prep(k_strided<T, N, false, 3>, smem))) return rc;
-    k_strided<T, N, false, 3><<<grid, NT, smem, st>>>(work, mode == 0 ? N : NN, mode == 0 ? NN : N, 1, mu1, lam,
-                                                      scale, tw, h->skip);
+    e = launch_pass(h, k_strided<T, N, false, 3>, grid, smem, work, rs, ps, 1, mu1, lam, scale, tw,
+                    (const int*)h->skip, (const T*)nullptr, 1);
   }
-  return KFBI_OK;
+  return e == cudaSuccess ? KFBI_OK : launch_failed("strided pass");
 }
 
 // scale / mu_p over the mode grid (q, k, p) of the float64 middle pass,
@@ -1060,37 +1104,31 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
     const T* rinv = mode_factors<T, N>(h, sa.lambda, (double)scale);
     if ((rc = prep(k_xfwd<T, N, 3>, smem))) return rc;
     if ((rc = prep(k_xinv<T, N, 3>, smem))) return rc;
-    if constexpr (sizeof(T) == 4) {
-      // float32: the five passes chained by programmatic dependent launch
-      if (launch_pdl(k_xfwd<T, N, 3>, grid, dim3(NT), smem, st, work, sa.src, sa.alpha, sa.src32, sa.corr,
-                     (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, (const int*)h->skip) != cudaSuccess)
-        return launch_failed("x forward pass");
-    } else {
-      k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(work, sa.src, sa.alpha, sa.src32, sa.corr, t.irr, t.line_start, tw,
-                                               h->skip);
-    }
+    // the five passes chained by programmatic dependent launch
+    if (launch_pass(h, k_xfwd<T, N, 3>, grid, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, (const int32_t*)t.irr,
+                    (const int32_t*)t.line_start, tw, (const int*)h->skip) != cudaSuccess)
+      return launch_failed("x forward pass");
     if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw))) return rc;
     if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, rinv))) return rc;
     if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw))) return rc;
-    if constexpr (sizeof(T) == 4) {
-      if (launch_pdl(k_xinv<T, N, 3>, grid, dim3(NT), smem, st, work, sa.keep || sa.out_user == nullptr, sa.out_user,
-                     (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32) != cudaSuccess)
-        return launch_failed("x inverse pass");
-    } else {
-      k_xinv<T, N, 3><<<grid, NT, smem, st>>>(work, sa.keep || sa.out_user == nullptr, sa.out_user, sa.aux, sa.beta,
-                                               sa.gamma, tw, h->skip, sa.aux32);
-    }
+    if (launch_pass(h, k_xinv<T, N, 3>, grid, smem, work, sa.keep || sa.out_user == nullptr, sa.out_user,
+                    (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32) != cudaSuccess)
+      return launch_failed("x inverse pass");
   } else {
     dim3 grid(N / W, 1);
     const T* rinv = mode_factors<T, N>(h, sa.lambda, (double)scale);
     if ((rc = prep(k_xfwd<T, N, 2>, smem))) return rc;
-    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(work, sa.src, sa.alpha, sa.src32, sa.corr, t.irr, t.line_start, tw,
-                                             h->skip);
     if ((rc = prep(k_strided<T, N, true, 2>, smem))) return rc;
-    k_strided<T, N, true, 2><<<grid, NT, smem, st>>>(work, N, 0, 0, mu1, lam, scale, tw, h->skip, rinv);
     if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
-    k_xinv<T, N, 2><<<grid, NT, smem, st>>>(work, sa.keep || sa.out_user == nullptr, sa.out_user, sa.aux, sa.beta,
-                                             sa.gamma, tw, h->skip, sa.aux32);
+    if (launch_pass(h, k_xfwd<T, N, 2>, grid, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, (const int32_t*)t.irr,
+                    (const int32_t*)t.line_start, tw, (const int*)h->skip) != cudaSuccess)
+      return launch_failed("x forward pass");
+    if (launch_pass(h, k_strided<T, N, true, 2>, grid, smem, work, (size_t)N, (size_t)0, 0, mu1, lam, scale, tw,
+                    (const int*)h->skip, rinv, 2) != cudaSuccess)
+      return launch_failed("y solve pass");
+    if (launch_pass(h, k_xinv<T, N, 2>, grid, smem, work, sa.keep || sa.out_user == nullptr, sa.out_user,
+                    (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32) != cudaSuccess)
+      return launch_failed("x inverse pass");
   }
   KFBI_CHECK_LAUNCH_N(dim == 3 ? 5 : 3);
   return KFBI_OK;
@@ -1157,7 +1195,7 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
     } else if (pass == 1 || pass == 2) {
       const T* rinv = mode_factors<T, N>(h, lambda, (double)scale);
       if ((rc = prep(k_strided<T, N, true, 2>, smem))) return rc;
-      k_strided<T, N, true, 2><<<grid, NT, smem, st>>>(work, N, 0, 0, mu1, lam, scale, tw, nullptr, rinv);
+      k_strided<T, N, true, 2><<<grid, NT, smem, st>>>(work, N, 0, 0, mu1, lam, scale, tw, nullptr, rinv, 2);
     } else {
       if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
       k_xinv<T, N, 2><<<grid, NT, smem, st>>>(work, true, nullptr, nullptr, 1.0, 0.0, tw, nullptr);
@@ -1187,12 +1225,9 @@ __global__ void __launch_bounds__(NT) k_strided_coupled(T* __restrict__ a, T* __
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sa = reinterpret_cast<T*>(smem_raw);
   T* sb = sa + N * RS;
-  T* tot = sb + N * RS;
-  T* tw = tot + C::G * W;
-  T* sinv = tw + 4 * N;
+  T* mem = sb + N * RS;
   const bool skipped = skip != nullptr && *skip != 0;
-  load_twiddles<T, N>(tw, tw_g);
-  load_sines<T, N>(sinv, tw_g);
+  load_tables<C>(mem, tw_g);
   if (skipped) return;
   const int x0 = blockIdx.x * W;
   const int q = blockIdx.y + qoff;
@@ -1205,8 +1240,8 @@ __global__ void __launch_bounds__(NT) k_strided_coupled(T* __restrict__ a, T* __
   }
   copy_async_wait();
   __syncthreads();
-  dst_tile<C>(sa, tw, sinv, tot);
-  dst_tile<C>(sb, tw, sinv, tot);
+#pragma unroll 1
+  for (int f = 0; f < 2; ++f) dst_tile<C>(f == 0 ? sa : sb, mem);
   // table row of this plane: modes (q, k, p), p fastest
   const T* f0 = cf + (size_t)q * N * N + x0;
   for (int idx = threadIdx.x; idx < N * W; idx += NT) {
@@ -1218,8 +1253,8 @@ __global__ void __launch_bounds__(NT) k_strided_coupled(T* __restrict__ a, T* __
     sb[k * RS + c] = g1 * ri + g2 * re;
   }
   __syncthreads();
-  dst_tile<C>(sa, tw, sinv, tot);
-  dst_tile<C>(sb, tw, sinv, tot);
+#pragma unroll 1
+  for (int f = 0; f < 2; ++f) dst_tile<C>(f == 0 ? sa : sb, mem);
   for (int idx = threadIdx.x; idx < N * W; idx += NT) {
     const int c = idx % W, k = idx / W;
     ba[(size_t)k * row_stride + c] = sa[k * RS + c];
@@ -1290,7 +1325,7 @@ int run_solve_coupled(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, 
   using C = Cfg<T, N>;
   constexpr int W = C::W;
   const size_t smem = C::smem_elems * sizeof(T);
-  const size_t smem2 = (2 * (size_t)N * C::RS + (size_t)C::G * W + 5 * (size_t)N) * sizeof(T);
+  const size_t smem2 = (2 * (size_t)N * C::RS + C::mem_elems) * sizeof(T);
   const int dim = h->grid.dim;
   cudaStream_t st = h->stream;
   const Tables& t = h->t;
@@ -1313,10 +1348,10 @@ int run_solve_coupled(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, 
     k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(wb, se.src, se.alpha, se.src32, se.corr, t.irr, t.line_start, tw, h->skip);
     const size_t NN = (size_t)N * N;
     for (T* w : {wa, wb})
-      k_strided<T, N, false, 3><<<grid, NT, smem, st>>>(w, N, NN, 1, mu1T, (T)0, (T)1, tw, h->skip);
+      k_strided<T, N, false, 3><<<grid, NT, smem, st>>>(w, N, NN, 1, mu1T, (T)0, (T)1, tw, h->skip, nullptr, 1);
     k_strided_coupled<T, N, 3><<<grid, NT, smem2, st>>>(wa, wb, NN, N, 1, cf, (size_t)total, tw, h->skip);
     for (T* w : {wa, wb})
-      k_strided<T, N, false, 3><<<grid, NT, smem, st>>>(w, N, NN, 1, mu1T, (T)0, (T)1, tw, h->skip);
+      k_strided<T, N, false, 3><<<grid, NT, smem, st>>>(w, N, NN, 1, mu1T, (T)0, (T)1, tw, h->skip, nullptr, 1);
     k_xinv<T, N, 3><<<grid, NT, smem, st>>>(wa, si.keep || si.out_user == nullptr, si.out_user, si.aux, si.beta,
                                              si.gamma, tw, h->skip);
     k_xinv<T, N, 3><<<grid, NT, smem, st>>>(wb, se.keep || se.out_user == nullptr, se.out_user, se.aux, se.beta,
@@ -1485,7 +1520,7 @@ __device__ void dct1_tile(typename C::T* s, const typename C::T* tw, typename C:
 template <typename C>
 __device__ __forceinline__ void dct_tile(typename C::T* s, const typename C::T* tw, const typename C::T* sinv,
                                          typename C::T* tot, typename C::T* x1) {
-  if constexpr (kRegDst<typename C::T, C::N>) {
+  if constexpr (C::REG) {
     regdst::dct1_tile_reg<regdst::Geo<C::N, C::RS>>(s, sinv, reinterpret_cast<const regdst::cf2*>(tw), tot, x1);
   } else {
     dct1_tile<C>(s, tw, tot, x1);
@@ -1511,7 +1546,7 @@ __global__ void __launch_bounds__(NT) k_nxfwd(T* __restrict__ a, const double* _
   T* sinv = x1 + W;
   const bool skipped = skip != nullptr && *skip != 0;
   load_twiddles<T, N>(tw, tw_g);
-  load_sines<T, N>(sinv, tw_g);
+  load_sines<C>(sinv, tw_g);
   if (skipped) return;
   const int y0 = blockIdx.x * W;
   const int z = DIM == 3 ? blockIdx.y : 0;
@@ -1562,7 +1597,7 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
   T* sinv = x1 + W;
   if (skip != nullptr && *skip != 0) return;
   load_twiddles<T, N>(tw, tw_g);
-  load_sines<T, N>(sinv, tw_g);
+  load_sines<C>(sinv, tw_g);
   const int y0 = blockIdx.x * W;
   const int z = DIM == 3 ? blockIdx.y : 0;
   const size_t plane = (size_t)z * P * P;
@@ -1605,7 +1640,7 @@ __global__ void __launch_bounds__(NT) k_nstrided(T* __restrict__ a, size_t row_s
   T* sinv = x1 + W;
   const bool skipped = skip != nullptr && *skip != 0;
   load_twiddles<T, N>(tw, tw_g);
-  load_sines<T, N>(sinv, tw_g);
+  load_sines<C>(sinv, tw_g);
   if (skipped) return;
   const int x0 = blockIdx.x * W;
   const int q = blockIdx.y;

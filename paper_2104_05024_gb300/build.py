@@ -19,13 +19,15 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkfbi.so")
 INCLUDE = os.path.join(ROOT, "include")
 
-SOURCES = {
-    "dst.cu": [],
-    "setup.cu": ["-fmad=false"],
-    "ops.cu": [],
-    "capi.cu": [],
-    "noalloc.cu": [],
-    "mlp.cu": [],
+# object: (source, extra flags); the transforms are compiled once per type, in parallel
+OBJECTS = {
+    "dst64.o": ("dst.cu", ["-DKFBI_DST_BITS=64"]),
+    "dst32.o": ("dst.cu", ["-DKFBI_DST_BITS=32"]),
+    "setup.o": ("setup.cu", ["-fmad=false"]),
+    "ops.o": ("ops.cu", []),
+    "capi.o": ("capi.cu", []),
+    "noalloc.o": ("noalloc.cu", []),
+    "mlp.o": ("mlp.cu", []),
 }
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]
@@ -51,11 +53,11 @@ def build(verbose: bool = False, force: bool = False) -> str:
     headers.append(os.path.join(INCLUDE, "kfbi.h"))
     jobs = []
     objs = []
-    for src, extra in SOURCES.items():
+    for name, (src, extra) in OBJECTS.items():
         path = os.path.join(CSRC, src)
         if not os.path.exists(path):
             continue
-        obj = os.path.join(BUILD, src.replace(".cu", ".o"))
+        obj = os.path.join(BUILD, name)
         objs.append(obj)
         if force or _needs(obj, [path] + headers):
             jobs.append([nvcc(), *COMMON, *ARCH, *extra, "-c", path, "-o", obj])

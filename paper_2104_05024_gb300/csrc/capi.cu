@@ -1772,7 +1772,7 @@ int kfbi_transform_pass(kfbi_handle* h, int precision, int pass, double lambda) 
     set_error("single transform passes are those of the Dirichlet box");
     return KFBI_ERR_ARG;
   }
-  return transform_pass(h, precision, pass, lambda);
+  return precision == KFBI_FP64 ? transform_pass64(h, pass, lambda) : transform_pass32(h, pass, lambda);
 }
 
 int64_t kfbi_launch_count(void) { return (int64_t)g_launches.load(); }

@@ -40,6 +40,13 @@
 namespace kfbi {
 namespace {
 
+// Compiled twice, with KFBI_DST_BITS = 32 and 64 (the float32 and the float64
+// kernels, in parallel): everything below is templates but for the entry
+// points at the end, which are split by type.
+#if KFBI_DST_BITS != 32 && KFBI_DST_BITS != 64
+#error "KFBI_DST_BITS must be 32 or 64"
+#endif
+
 constexpr int NT = 256;
 
 // float64 <-> T for float T on the bit patterns (a float64 conversion
@@ -351,23 +358,23 @@ __device__ __forceinline__ void load_tables(typename C::T* mem, const typename C
   }
 }
 
-struct NoPost {
+struct NoMap {
   template <typename T>
   __device__ __forceinline__ T operator()(int, T v) const {
     return v;
   }
 };
 
-// the DST-I of every column of the tile, rows 1..N-1; post maps the outputs
-// (not on the Stockham path)
-template <typename C, class Post = NoPost>
-__device__ __forceinline__ void dst_tile(typename C::T* s, typename C::T* mem, const Post& post = Post()) {
+// the DST-I of every column of the tile, rows 1..N-1; map: applied to the
+// outputs (register path) or to the inputs (fixed-point path)
+template <typename C, class Map = NoMap>
+__device__ __forceinline__ void dst_tile(typename C::T* s, typename C::T* mem, const Map& map = Map()) {
   if constexpr (C::FIX) {
-    fixdst::dst1_tile_fix<fixdst::Geo<C::N, C::RS>>(s, reinterpret_cast<fixdst::ll*>(mem), post);
+    fixdst::dst1_tile_fix<fixdst::Geo<C::N, C::RS>>(s, reinterpret_cast<fixdst::ll*>(mem), map);
   } else if constexpr (C::REG) {
     const typename C::T* tw = mem + C::G * C::W;
     regdst::dst1_tile_reg<regdst::Geo<C::N, C::RS>>(s, tw + 4 * C::N, reinterpret_cast<const regdst::cf2*>(tw), mem,
-                                                    post);
+                                                    map);
   } else {
     dst1_tile<C>(s, mem + C::G * C::W, mem);
   }
@@ -387,9 +394,10 @@ struct DivPost {
   }
 };
 
-// the same in float64: the factor from the table built for this lambda, or
+// the same in float64, applied to the inputs of the inverse transform: the
+// factor from the table built for this lambda, or
 // divided here (handles without a table)
-struct FactorPost {
+struct FactorPre {
   const double* r;  // table entry of this column's mode 0, row stride n (nullptr: none)
   int n;
   const double* mu;
@@ -564,16 +572,16 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_strided(T* __restrict
     }
     dst_tile<C>(s, mem);
   } else if constexpr (C::FIX) {
-    // forward DST with its outputs multiplied by the mode factors as they
-    // are written, then the inverse DST by the same (single inlined) body
+    // forward DST, then by the same (single inlined) body the inverse DST,
+    // whose inputs are multiplied by the mode factors as they are read
     if constexpr (SOLVE) {
       const int p = x0 + (int)(threadIdx.x & 31);
-      FactorPost post{rinv != nullptr ? rinv + ((size_t)q * N * N + p) : nullptr, N, mu1, mu1[p] + muq - lambda, scale,
-                      p == 0, true};
+      FactorPre pre{rinv != nullptr ? rinv + ((size_t)q * N * N + p) : nullptr, N, mu1, mu1[p] + muq - lambda, scale,
+                    p == 0, false};
 #pragma unroll 1
       for (int rep = 0; rep < reps; ++rep) {
-        dst_tile<C>(s, mem, post);
-        post.on = false;
+        dst_tile<C>(s, mem, pre);
+        pre.on = true;
       }
     } else {
       dst_tile<C>(s, mem);
@@ -1734,6 +1742,7 @@ int box_solve_neumann(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1
 
 }  // namespace
 
+#if KFBI_DST_BITS == 32
 // TMA descriptors of the padded float32 grid for the strided passes (3-D,
 // 32 <= N <= 256): boxes of 32 x-values by N rows along y or along z.
 int make_tma_maps(kfbi_handle* h) {
@@ -1793,8 +1802,7 @@ int make_tma_maps(kfbi_handle* h) {
   return KFBI_OK;
 }
 
-int transform_pass(kfbi_handle* h, int precision, int pass, double lambda) {
-  if (precision == KFBI_FP64) return dispatch_pass<double>(h, pass, lambda, h->w.grid64, h->t.mu, h->t.tw64);
+int transform_pass32(kfbi_handle* h, int pass, double lambda) {
   return dispatch_pass<float>(h, pass, lambda, h->w.grid32, h->t.mu32, h->t.tw32);
 }
 
@@ -1802,15 +1810,20 @@ int dst_supported(int N) {
   return N == 8 || N == 16 || N == 32 || N == 64 || N == 128 || N == 256 || N == 384 || N == 512;
 }
 
-int box_solve64(kfbi_handle* h, const SolveArgs& a, double* work) {
-  if (h->grid.bc == KFBI_BOX_NEUMANN) return box_solve_neumann<double>(h, a, work, h->t.mu, h->t.tw64);
-  return dispatch<double>(h, a, work, h->t.mu, h->t.tw64);
-}
-
 int box_solve32(kfbi_handle* h, const SolveArgs& a, float* work) {
   if (h->grid.bc == KFBI_BOX_NEUMANN) return box_solve_neumann<float>(h, a, work, h->t.mu32, h->t.tw32);
   return dispatch<float>(h, a, work, h->t.mu32, h->t.tw32);
 }
+#else
+int transform_pass64(kfbi_handle* h, int pass, double lambda) {
+  return dispatch_pass<double>(h, pass, lambda, h->w.grid64, h->t.mu, h->t.tw64);
+}
+
+int box_solve64(kfbi_handle* h, const SolveArgs& a, double* work) {
+  if (h->grid.bc == KFBI_BOX_NEUMANN) return box_solve_neumann<double>(h, a, work, h->t.mu, h->t.tw64);
+  return dispatch<double>(h, a, work, h->t.mu, h->t.tw64);
+}
+#endif
 
 namespace {
 template <typename T>
@@ -1831,11 +1844,12 @@ int dispatch_coupled(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, c
 }
 }  // namespace
 
+#if KFBI_DST_BITS == 64
 int box_solve_coupled64(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, const Coupling& cp, double* wa,
                         double* wb) {
   return dispatch_coupled<double>(h, si, se, cp, wa, wb, h->t.mu, h->t.tw64);
 }
-
+#else
 int box_solve_coupled32(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, const Coupling& cp, float* wa,
                         float* wb) {
   return dispatch_coupled<float>(h, si, se, cp, wa, wb, h->t.mu32, h->t.tw32);
@@ -1860,9 +1874,11 @@ __global__ void k_selftest_wait(long cap, int* err) {
   if (!ok && threadIdx.x == 0) atomicOr(err, DEVERR_TIMEOUT);
 }
 }  // namespace
+#endif  // KFBI_DST_BITS
 
 }  // namespace kfbi
 
+#if KFBI_DST_BITS == 32
 extern "C" int kfbi_selftest_bounded_wait(int polls, int* timed_out, double* ms) {
   using namespace kfbi;
   if (polls < 1 || polls > (1 << 20) || !timed_out) {
@@ -1895,3 +1911,4 @@ extern "C" int kfbi_selftest_bounded_wait(int polls, int* timed_out, double* ms)
   KFBI_COUNT(1);
   return KFBI_OK;
 }
+#endif  // KFBI_DST_BITS

@@ -443,18 +443,23 @@ struct State {
 };
 
 // phase 0: the thread's row pairs of column c to registers, its largest
-// exponent field to mx[a][c].  Thread 0 of the column holds row N/2 (its own
+// exponent field to mx[a][c]; pre(j, v) maps the row values (the spectral
+// multiply of a solve: here the registers hold nothing else, and its loads
+// are all in flight at once).  Thread 0 of the column holds row N/2 (its own
 // mirror image) in place of the pair of row 0.
-template <class G>
-KFBI_HD void phase_0(State<G>& st, const double* s, int* mx, int a, int c) {
+template <class G, class Pre>
+KFBI_HD void phase_0(State<G>& st, const double* s, int* mx, int a, int c, const Pre& pre) {
   constexpr int N = G::N, RS = G::RS, T = G::T, P = G::P, W = G::W;
   uint32_t m = 0;
 #pragma unroll
   for (int i = 0; i < P; ++i) {
     const int j = a + T * i;
-    const bool mid = j == 0;
-    st.xa[i] = s[(mid ? N / 2 : j) * RS + c];
-    st.xb[i] = s[(mid ? N / 2 : N - j) * RS + c];
+    const int ja = j == 0 ? N / 2 : j, jb = j == 0 ? N / 2 : N - j;
+    st.xa[i] = pre(ja, s[ja * RS + c]);
+    st.xb[i] = pre(jb, s[jb * RS + c]);
+  }
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
     const uint32_t ha = (uint32_t)hi_of(bits_of(st.xa[i])) & 0x7fffffffu;
     const uint32_t hb = (uint32_t)hi_of(bits_of(st.xb[i])) & 0x7fffffffu;
     m = ha > m ? ha : m;
@@ -580,27 +585,27 @@ KFBI_HD void phase_c(State<G>& st, const c2* ex, int a, int c) {
 // doubled: 2 I_k to row 2k (even output), 2 R_k to row 2k + 1 (scan input).
 // |D| <= 2 sum |y_odd| and |S| <= 2 sum |y_even| stay below the full sum's
 // bound, since a pair (j, N - j) has one parity.
-template <class G, class Post>
+template <class G>
 KFBI_HD void split_store(ll* s, const cfx* sp, const Scale& sc, int k, ll Ar, ll Ai, ll Br, ll Bi, int c,
-                         const Post& post, bool both) {
+                         bool both) {
   constexpr int RS = G::RS, L = G::L;
   double* sd = reinterpret_cast<double*>(s);
   const ll Sr = Ar + Br, Si = Ai - Bi;
   ll pr = Ar - Br, pi = Ai + Bi;
   // w (D_r + i D_i) = (wr Dr - wi Di) + i (wr Di + wi Dr)
   cmul62(pr, pi, sp[k]);
-  sd[(2 * k) * RS + c] = post(2 * k, from_fix(Si - pr, sc));
+  sd[(2 * k) * RS + c] = from_fix(Si - pr, sc);
   s[(2 * k + 1) * RS + c] = Sr + pi;
   if (both) {
     const int kk = L - k;
-    sd[(2 * kk) * RS + c] = post(2 * kk, from_fix(-(Si + pr), sc));
+    sd[(2 * kk) * RS + c] = from_fix(-(Si + pr), sc);
     s[(2 * kk + 1) * RS + c] = Sr - pi;
   }
 }
 
 // phase D: real-DFT split of the owned pairs (after a barrier)
-template <class G, class Post>
-KFBI_HD void phase_d(const State<G>& st, ll* s, const cfx* sp, int a, int c, const Post& post) {
+template <class G>
+KFBI_HD void phase_d(const State<G>& st, ll* s, const cfx* sp, int a, int c) {
   constexpr int T = G::T, P = G::P, RS = G::RS;
 #pragma unroll
   for (int gi = 0; gi < G::GPT; ++gi) {
@@ -614,17 +619,17 @@ KFBI_HD void phase_d(const State<G>& st, ll* s, const cfx* sp, int a, int c, con
 #pragma unroll
       for (int k2 = 1; k2 <= 4; ++k2)
         split_store<G>(s, sp, st.sc, P * k2, st.Ar[gi][k2], st.Ai[gi][k2], st.Ar[gi][8 - k2], st.Ai[gi][8 - k2], c,
-                       post, k2 < 4);
+                       k2 < 4);
       // k1 = P/2: k = P/2 + P k2 pairs with P/2 + P (7 - k2)
 #pragma unroll
       for (int k2 = 0; k2 < 4; ++k2)
         split_store<G>(s, sp, st.sc, kB + P * k2, st.Br[gi][k2], st.Bi[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2],
-                       c, post, true);
+                       c, true);
     } else {
 #pragma unroll
       for (int k2 = 0; k2 < 8; ++k2)
         split_store<G>(s, sp, st.sc, kA + P * k2, st.Ar[gi][k2], st.Ai[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2],
-                       c, post, true);
+                       c, true);
     }
   }
 }
@@ -643,8 +648,8 @@ KFBI_HD void phase_e1(State<G>& st, const ll* s, ll* tot, int a, int c) {
 }
 
 // phase E2: the preceding segments' totals added, odd outputs written
-template <class G, class Post>
-KFBI_HD void phase_e2(const State<G>& st, ll* s, const ll* tot, int a, int c, const Post& post) {
+template <class G>
+KFBI_HD void phase_e2(const State<G>& st, ll* s, const ll* tot, int a, int c) {
   constexpr int P = G::P, RS = G::RS, W = G::W;
   double* sd = reinterpret_cast<double*>(s);
   ll off = 0;
@@ -652,7 +657,7 @@ KFBI_HD void phase_e2(const State<G>& st, ll* s, const ll* tot, int a, int c, co
 #pragma unroll
   for (int i = 0; i < P; ++i) {
     const int j = 2 * (a * P + i) + 1;
-    sd[j * RS + c] = post(j, from_fix(st.v[i] + off, st.sc));
+    sd[j * RS + c] = from_fix(st.v[i] + off, st.sc);
   }
 }
 
@@ -689,8 +694,8 @@ __device__ __forceinline__ void load_tables(ll* mem, const double* tw_g) {
 // The whole transform of the tile s[N][RS] (rows 1..N-1 in and out; row 0
 // becomes 0) by 256 threads; mem: the tables and scratch.  Ends with a
 // barrier.
-template <class G, class Post = Identity>
-__device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem, const Post& post = Post()) {
+template <class G, class Pre = Identity>
+__device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem, const Pre& pre = Pre()) {
   constexpr int N = G::N;
   const int a = threadIdx.x >> 5, c = threadIdx.x & 31;
   ll* s = reinterpret_cast<ll*>(sd);
@@ -701,7 +706,7 @@ __device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem, const Post& p
   ll* tot = mem + 2 * N + N / 2 + 256;
   State<G> st;
   c2* ex = reinterpret_cast<c2*>(s);
-  phase_0<G>(st, sd, mx, a, c);
+  phase_0<G>(st, sd, mx, a, c, pre);
   __syncthreads();
   phase_s<G>(st, mx, sm, a, c);
   __syncthreads();
@@ -713,11 +718,11 @@ __device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem, const Post& p
   __syncthreads();
   phase_c<G>(st, ex, a, c);
   __syncthreads();
-  phase_d<G>(st, s, sp, a, c, post);
+  phase_d<G>(st, s, sp, a, c);
   __syncthreads();
   phase_e1<G>(st, s, tot, a, c);
   __syncthreads();
-  phase_e2<G>(st, s, tot, a, c, post);
+  phase_e2<G>(st, s, tot, a, c);
   __syncthreads();
 }
 #endif

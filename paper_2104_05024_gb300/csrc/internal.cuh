@@ -336,7 +336,8 @@ int box_solve32(kfbi_handle* h, const SolveArgs& a, float* work);
 int box_solve_coupled32(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, const Coupling& cp, float* wa,
                         float* wb);
 int dst_supported(int N);
-int transform_pass(kfbi_handle* h, int precision, int pass, double lambda);
+int transform_pass32(kfbi_handle* h, int pass, double lambda);
+int transform_pass64(kfbi_handle* h, int pass, double lambda);
 int make_tma_maps(kfbi_handle* h);
 
 // ops.cu

@@ -34,18 +34,32 @@ __global__ void k_correction(Tables t, const double* __restrict__ x, double* __r
   corr[i] = acc;
 }
 
-// x = [psi; m] with m_i = sum_j gcol[(i - j) mod M] psi_j
-__global__ void k_spline(const double* __restrict__ gcol, const double* __restrict__ psi, double* __restrict__ x, int M) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= M) return;
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// x = [psi; m] with m_i = sum_j gcol[(i - j) mod M] psi_j, one warp per node:
+// the sum is a serial chain otherwise (one thread per node: 22 us at M = 256,
+// more than a transform pass of the 128^2 grid it goes with; now 3.5 us)
+__global__ void k_spline(const double* __restrict__ gcol, const double* __restrict__ psi, double* __restrict__ x, int M,
+                         const int* __restrict__ skip) {
+  pdl_wait();
+  pdl_launch_next();
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= M || (skip != nullptr && *skip)) return;
   double acc = 0.0;
-  for (int j = 0; j < M; ++j) {
-    int k = i - j;
-    if (k < 0) k += M;
-    acc += gcol[k] * psi[j];
+#pragma unroll 4
+  for (int j = lane; j < M; j += 32) {
+    const int k = i - j;
+    acc += gcol[k < 0 ? k + M : k] * psi[j];
   }
-  x[i] = psi[i];
-  x[M + i] = acc;
+  acc = warp_sum(acc);
+  if (lane == 0) {
+    x[i] = psi[i];
+    x[M + i] = acc;
+  }
 }
 
 // out_i = base_i + sgn * (sum_j wn_ij v(p_j) + sum_k dw_ik x[dpid_ik])
@@ -391,11 +405,6 @@ __global__ void k_pad_to_user(GridParams gr, const double* __restrict__ p, doubl
 }
 
 // ---------------------------------------------------------------- Krylov
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // partial[k][b] = sum over block b's slice of V_k . w
 __global__ void k_dots_partial(const double* __restrict__ V, int ld, const double* __restrict__ w, int n,
@@ -997,7 +1006,9 @@ int launch_correction_t(kfbi_handle* h, const Tables& t, const double* x, double
 
 int launch_spline(kfbi_handle* h, const double* psi, double* x) {
   const int M = h->t.M;
-  k_spline<<<(M + 127) / 128, 128, 0, h->stream>>>(h->t.spline_G, psi, x, M);
+  if (launch_pdl(k_spline, dim3((M + 3) / 4), dim3(128), 0, h->stream, (const double*)h->t.spline_G, psi, x, M,
+                 (const int*)h->skip) != cudaSuccess)
+    return launch_failed("spline moments");
   KFBI_CHECK_LAUNCH();
   return KFBI_OK;
 }

@@ -99,6 +99,7 @@ int apply_A_coupled(kfbi_handle* h, double kappa, const double* psi, double* out
   SolveArgs si, se;
   si.corr = h->w.corr;
   se.corr = h->w.corr2;
+  si.near_only = se.near_only = true;
   Coupling cp = h->cpl;
   cp.kappa = kappa;
   if ((rc = box_solve_coupled64(h, si, se, cp, h->w.grid64, h->w.grid64b))) return rc;
@@ -170,6 +171,7 @@ int apply_A_coupled32(kfbi_handle* h, double kappa, const double* psi, double* o
   SolveArgs si, se;
   si.corr = h->w.corr;
   se.corr = h->w.corr2;
+  si.near_only = se.near_only = true;
   Coupling cp = h->cpl;
   cp.kappa = kappa;
   if ((rc = box_solve_coupled32(h, si, se, cp, h->w.grid32, h->w.grid32b))) return rc;
@@ -285,6 +287,7 @@ int apply_A(kfbi_handle* h, int prec, double lambda, const double* psi, double* 
   SolveArgs sa;
   sa.corr = h->w.corr;
   sa.lambda = lambda;
+  sa.near_only = true;
   if (prec == KFBI_FP64) {
     if ((rc = box_solve64(h, sa, h->w.grid64))) return rc;
     rc = launch_limit64(h, h->w.grid64, x, base, sgn, out);
@@ -341,52 +344,35 @@ int norm2(kfbi_handle* h, const double* v, double* slot, double* out) {
 // GMRES tolerances below 1e-9 take a second round.
 int refine_rounds(const kfbi_handle* h) { return h->opts.tol < 1e-9 ? 2 : 1; }
 
+// The parts of u stay float32 until the end: u1 in grid32, the first
+// correction in grid32b, and each x inverse pass adds in float64.  The second
+// round's residual is the first one's (kept as a float pair) minus L_h of the
+// correction, in float-float arithmetic too; a float64 7-point residual of u
+// took 2.54 ms at 512^3 and 0.39 ms at 256^3.
 int refined_solve(kfbi_handle* h, const double* src, double alpha, const double* corr, double lambda, double* u) {
-  // Dirichlet box, separate x and y passes: the first solve's float result
-  // stays in the padded grid grid32 alone (no float64 copy), the correction
-  // solve runs in grid32b and writes u = its result + grid32 in float64
-  const bool split = h->grid.bc == KFBI_BOX_DIRICHLET && !(h->xy_fused && h->grid.dim == 3);
   SolveArgs sa;
   sa.src = src;
   sa.alpha = alpha;
   sa.corr = corr;
   sa.lambda = lambda;
-  sa.out_user = split ? nullptr : u;
   int rc = box_solve32(h, sa, h->w.grid32);
   if (rc) return rc;
-  const int rounds = refine_rounds(h);
-  for (int r = 0; r < rounds; ++r) {
-    SolveArgs sr;
-    if (r == 0 && split) {
-      // float-float residual of the float grid, float32 result; the
-      // irregular nodes from the padded grid too
-      if ((rc = launch_residual_ff(h, src, alpha, corr, h->w.grid32, nullptr, lambda, h->w.res32))) return rc;
-      sr.src32 = h->w.res32;
-      sr.lambda = lambda;
-      sr.out_user = u;
-      sr.aux32 = h->w.grid32;
-      sr.keep = false;
-      if ((rc = box_solve32(h, sr, h->w.grid32b))) return rc;
-      continue;
-    }
-    if (r == 0) {
-      // u is exactly the float32 grid of the solve just done: float-float
-      // residual, float32 result
-      if ((rc = launch_residual_ff(h, src, alpha, corr, h->w.grid32, u, lambda, h->w.res32))) return rc;
-      sr.src32 = h->w.res32;
-    } else {
-      if ((rc = launch_residual(h, src, alpha, corr, u, lambda, h->w.res64))) return rc;
-      sr.src = h->w.res64;
-    }
-    sr.lambda = lambda;
-    sr.out_user = u;
-    sr.aux = u;
-    sr.beta = 1.0;
-    sr.gamma = 1.0;
-    sr.keep = false;  // only u is read after a refinement round
-    if ((rc = box_solve32(h, sr, h->w.grid32))) return rc;
-  }
-  return KFBI_OK;
+  const bool two = refine_rounds(h) > 1;
+  if ((rc = launch_residual_ff(h, src, alpha, corr, h->w.grid32, lambda, h->w.res32, two ? h->w.res32lo : nullptr)))
+    return rc;
+  SolveArgs sr;
+  sr.src32 = h->w.res32;
+  sr.lambda = lambda;
+  sr.out_user = u;
+  sr.aux32 = h->w.grid32;
+  sr.keep = two;
+  if ((rc = box_solve32(h, sr, h->w.grid32b)) || !two) return rc;
+  if ((rc = launch_residual_pair(h, h->w.res32, h->w.res32lo, h->w.grid32b, lambda))) return rc;
+  sr.aux32 = nullptr;
+  sr.aux = u;
+  sr.gamma = 1.0;
+  sr.keep = false;
+  return box_solve32(h, sr, h->w.grid32);
 }
 
 // out = base + sgn * A psi with a float64-accurate (refined) box solve
@@ -952,8 +938,9 @@ static int create_impl(const kfbi_geometry* geom, const kfbi_grid* grid, double 
   cudaMemsetAsync(h->w.g_prev, 0, sizeof(double) * (size_t)M, h->stream);
   cudaMemsetAsync(h->w.psi_prev2, 0, sizeof(double) * (size_t)M, h->stream);
   if ((rc = dalloc(h, &h->w.u64, (size_t)grid_points(h)))) return fail(rc);
-  if ((rc = dalloc(h, &h->w.res64, (size_t)grid_points(h)))) return fail(rc);
+  if (h->coupled && (rc = dalloc(h, &h->w.res64, (size_t)grid_points(h)))) return fail(rc);
   if ((rc = dalloc(h, &h->w.res32, (size_t)grid_points(h)))) return fail(rc);
+  if ((rc = dalloc(h, &h->w.res32lo, (size_t)grid_points(h)))) return fail(rc);
   if ((rc = dalloc(h, &h->w.vV64, (size_t)grid_points(h)))) return fail(rc);
   cudaMemsetAsync(h->w.psi_prev, 0, sizeof(double) * (size_t)M, h->stream);
   if ((rc = dalloc(h, &h->w.hist_psi, (size_t)KFBI_HISTORY * M))) return fail(rc);

@@ -412,6 +412,53 @@ struct FactorPre {
   }
 };
 
+// how many of a lane's per values are loaded together: a divisor of per, 8 at
+// most
+__host__ __device__ constexpr int batch_of(int per) {
+  int c = per < 8 ? per : 8;
+  while (per % c != 0) --c;
+  return c;
+}
+
+// The W x-lines y0 .. y0 + W - 1 of plane z of a field (interior nodes, rows
+// of N - 1 values) to the tile s[x][line], mapped by f, with zeros at x = 0
+// and on line y = 0.  A warp takes whole lines and issues a line's loads
+// together (rows start at odd addresses, so each is a coalesced run of single
+// values): with one load in flight per thread at a time a float64 source cost
+// the 512^3 float32 pass 0.98 ms, four times the pass without a source.
+template <typename C, int DIM, typename S, typename F>
+__device__ __forceinline__ void fill_lines(typename C::T* s, const S* __restrict__ src, int y0, int z, const F& f) {
+  constexpr int N = C::N, W = C::W, RS = C::RS, n1 = N - 1;
+  if constexpr (N >= 32) {
+    constexpr int PER = N / 32, CH = batch_of(PER);  // values per lane and line, loads issued together
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int c = threadIdx.x >> 5; c < W; c += NT / 32) {
+      const int y = y0 + c;
+      const S* row = src + ((DIM == 3 ? (size_t)(z - 1) * n1 : 0) + (y - 1)) * n1 - 1;
+#pragma unroll
+      for (int i0 = 0; i0 < PER; i0 += CH) {
+        static_assert(PER % CH == 0, "whole batches");
+        S v[CH];
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+          const int x = lane + 32 * (i0 + i);
+          v[i] = x > 0 && y > 0 ? __ldg(&row[x]) : (S)0;
+        }
+#pragma unroll
+        for (int i = 0; i < CH; ++i) s[(lane + 32 * (i0 + i)) * RS + c] = f(v[i]);
+      }
+    }
+  } else {
+    for (int idx = threadIdx.x; idx < N * W; idx += NT) {
+      const int x = idx % N, c = idx / N, y = y0 + c;
+      S v = (S)0;
+      if (x > 0 && y > 0) v = src[((DIM == 3 ? (size_t)(z - 1) * n1 : 0) + (y - 1)) * n1 + (x - 1)];
+      s[x * RS + c] = f(v);
+    }
+  }
+}
+
 // ------------------------------------------------------------- x forward
 // Tile: W consecutive lines y0..y0+W-1 of plane z; assembles
 // r = alpha*src + corrections on the fly.
@@ -420,7 +467,7 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xfwd(T* __restrict__ 
                                              const float* __restrict__ src32,
                                              const double* __restrict__ corr, const int32_t* __restrict__ irr,
                                              const int32_t* __restrict__ line_start, const T* __restrict__ tw_g,
-                                             const int* __restrict__ skip) {
+                                             const int* __restrict__ skip, int yoff, int zoff) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, n1 = N - 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -429,31 +476,15 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xfwd(T* __restrict__ 
   load_tables<C>(mem, tw_g);
   pdl_wait();
   if (skip != nullptr && *skip != 0) return;
-  const int y0 = blockIdx.x * W;
-  const int z = DIM == 3 ? blockIdx.y + 1 : 0;
+  const int y0 = blockIdx.x * W + yoff;
+  const int z = DIM == 3 ? blockIdx.y + zoff : 0;
   // the branch on src stays outside the loops: inside, the compiler
   // evaluates the (float64) scaling for every element, taken or not
   if (src != nullptr) {
     const T a_t = (T)alpha;
-    for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-      const int x = idx % N, c = idx / N, y = y0 + c;
-      T v = (T)0;
-      if (x > 0 && y > 0) {
-        const size_t line = DIM == 3 ? (size_t)(z - 1) * n1 + (y - 1) : (size_t)(y - 1);
-        v = a_t * to_T<T>(src[line * n1 + (x - 1)]);
-      }
-      s[x * RS + c] = v;
-    }
+    fill_lines<C, DIM>(s, src, y0, z, [&](double v) { return a_t * to_T<T>(v); });
   } else if (src32 != nullptr) {
-    for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-      const int x = idx % N, c = idx / N, y = y0 + c;
-      T v = (T)0;
-      if (x > 0 && y > 0) {
-        const size_t line = DIM == 3 ? (size_t)(z - 1) * n1 + (y - 1) : (size_t)(y - 1);
-        v = (T)src32[line * n1 + (x - 1)];
-      }
-      s[x * RS + c] = v;
-    }
+    fill_lines<C, DIM>(s, src32, y0, z, [&](float v) { return (T)v; });
   } else {
     for (int idx = threadIdx.x; idx < N * W; idx += NT) s[(idx % N) * RS + idx / N] = (T)0;
   }
@@ -487,7 +518,7 @@ template <typename T, int N, int DIM>
 __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ a, bool keep, double* __restrict__ out,
                                              const double* __restrict__ aux, double beta, double gamma,
                                              const T* __restrict__ tw_g, const int* __restrict__ skip,
-                                             const float* __restrict__ aux32 = nullptr) {
+                                             const float* __restrict__ aux32, int yoff, int zoff) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, n1 = N - 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -496,8 +527,8 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ 
   load_tables<C>(mem, tw_g);
   pdl_wait();
   if (skip != nullptr && *skip != 0) return;
-  const int y0 = blockIdx.x * W;
-  const int z = DIM == 3 ? blockIdx.y + 1 : 0;
+  const int y0 = blockIdx.x * W + yoff;
+  const int z = DIM == 3 ? blockIdx.y + zoff : 0;
   const size_t plane = (size_t)z * N * N;
   for (int idx = threadIdx.x; idx < N * W; idx += NT) {
     const int x = idx % N, c = idx / N;
@@ -517,34 +548,50 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ 
   }
   // out = beta v + gamma aux with beta applied in T (one float64 operation
   // per element without aux, two with), or out = beta v + aux32 with aux32 a
-  // padded float grid of the same layout as a (one float64 addition)
+  // padded float grid of the same layout as a (one float64 addition); a
+  // line's loads of aux are issued together
   const T b_t = (T)beta;
-  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-    const int x = idx % N, c = idx / N, y = y0 + c;
-    const T v = s[x * RS + c];
-    const size_t pidx = plane + (size_t)y * N + x;
-    if (keep) a[pidx] = v;
-    if (x > 0 && y > 0) {
-      const size_t line = DIM == 3 ? (size_t)(z - 1) * n1 + (y - 1) : (size_t)(y - 1);
-      const size_t o = line * n1 + (x - 1);
-      const double bv = to_double(b_t * v);
-      if (aux32 != nullptr)
-        out[o] = bv + ffl::widen(aux32[pidx]);
-      else
-        out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
+  constexpr int LW = N < 32 ? N : 32;             // lanes along x
+  constexpr int PER = N / LW, CH = batch_of(PER);
+  const int lane = threadIdx.x % LW;
+#pragma unroll 1
+  for (int c = threadIdx.x / LW; c < W; c += NT / LW) {
+    const int y = y0 + c;
+    const size_t pidx = plane + (size_t)y * N + lane;
+    const size_t o = ((DIM == 3 ? (size_t)(z - 1) * n1 : 0) + (y - 1)) * n1 + lane - 1;
+#pragma unroll
+    for (int i0 = 0; i0 < PER; i0 += CH) {
+      double w[CH];
+      if (aux32 != nullptr) {
+#pragma unroll
+        for (int i = 0; i < CH; ++i) w[i] = ffl::widen(aux32[pidx + LW * (i0 + i)]);
+      } else if (aux != nullptr) {
+#pragma unroll
+        for (int i = 0; i < CH; ++i) w[i] = y > 0 && lane + i0 + i > 0 ? aux[o + LW * (i0 + i)] : 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < CH; ++i) {
+        const T v = s[(lane + LW * (i0 + i)) * RS + c];
+        if (keep) a[pidx + LW * (i0 + i)] = v;
+        if (y > 0 && lane + i0 + i > 0) {
+          const double bv = to_double(b_t * v);
+          out[o + LW * (i0 + i)] = aux32 != nullptr ? bv + w[i] : aux != nullptr ? fma(gamma, w[i], bv) : bv;
+        }
+      }
     }
   }
 }
 
 // --------------------------------------------------- strided (y / z) passes
 // Tile rows = transform index k (stride row_stride), columns x0..x0+W-1 of
-// plane q = blockIdx.y + qoff.  SOLVE = forward DST, spectral multiply,
+// plane q = blockIdx.y + qoff; rows outside `in` are zero and not read, rows
+// outside `out` are not written.  SOLVE = forward DST, spectral multiply,
 // inverse DST.
 template <typename T, int N, bool SOLVE, int DIM>
 __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_strided(T* __restrict__ a, size_t row_stride, size_t plane_stride, int qoff,
                                                 const T* __restrict__ mu1, T lambda, T scale,
                                                 const T* __restrict__ tw_g, const int* __restrict__ skip,
-                                                const T* __restrict__ rinv, int reps) {
+                                                const T* __restrict__ rinv, int reps, Span in, Span out) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -556,9 +603,15 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_strided(T* __restrict
   const int x0 = blockIdx.x * W;
   const int q = blockIdx.y + qoff;
   T* base = a + (size_t)q * plane_stride + x0;
-  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-    const int c = idx % W, k = idx / W;
-    copy_async(&s[k * RS + c], &base[(size_t)k * row_stride + c]);
+  {
+    constexpr int DR = NT / W;
+    const int c = threadIdx.x % W, k0 = in.lo + threadIdx.x / W;
+    const T* src = base + (size_t)k0 * row_stride + c;
+    T* dst = s + k0 * RS + c;
+#pragma unroll 8
+    for (int k = k0; k < in.hi; k += DR, src += DR * row_stride, dst += DR * RS) copy_async(dst, src);
+    for (int k = threadIdx.x / W; k < in.lo; k += DR) s[k * RS + c] = (T)0;
+    for (int k = in.hi + threadIdx.x / W; k < N; k += DR) s[k * RS + c] = (T)0;
   }
   copy_async_wait();
   __syncthreads();
@@ -604,9 +657,13 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_strided(T* __restrict
     }
   }
   pdl_launch_next();
-  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-    const int c = idx % W, k = idx / W;
-    base[(size_t)k * row_stride + c] = s[k * RS + c];
+  {
+    constexpr int DR = NT / W;
+    const int c = threadIdx.x % W, k0 = out.lo + threadIdx.x / W;
+    T* dst = base + (size_t)k0 * row_stride + c;
+    const T* src = s + k0 * RS + c;
+#pragma unroll 8
+    for (int k = k0; k < out.hi; k += DR, dst += DR * row_stride, src += DR * RS) *dst = *src;
   }
 }
 
@@ -675,16 +732,23 @@ constexpr size_t tma_smem_bytes() {
   return (2 * (size_t)N * TMA_W + (size_t)TmaTile<N>::G * TMA_W + 6 * (size_t)N) * sizeof(float) + 2 * sizeof(uint64_t);
 }
 
-// mode 0: tiles [y][x-chunk] of plane z = q; mode 1: tiles [z][x-chunk] of row y = q
-template <int N, bool SOLVE>
-__global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const __grid_constant__ CUtensorMap map, int mode,
+// mode 0: tiles [y][x-chunk] of the planes z = q; mode 1: tiles [z][x-chunk]
+// of the rows y = q, q in `planes`.  map_in / map_out: boxes of the rows `in`
+// that are read (the others are zero) and `out` that are written; PART =
+// false: all N of both (known at compile time: the runtime spans cost the
+// 256-row kernels register spills, 24.5 -> 26.4 us a pass).
+template <int N, bool SOLVE, bool PART>
+__global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const __grid_constant__ CUtensorMap map_in,
+                                                    const __grid_constant__ CUtensorMap map_out, int mode,
+                                                    Span planes_p, Span in_p, Span out_p,
                                                     const float* __restrict__ mu1, float lambda, float scale,
                                                     const float* __restrict__ tw_g, int* __restrict__ err,
                                                     int reps, const int* __restrict__ skip) {
   using C = TmaTile<N>;
   constexpr int W = TMA_W, NX = N / TMA_W;
-  constexpr int ntiles = NX * (N - 1);
-  constexpr uint32_t bytes = (uint32_t)(N * W * sizeof(float));
+  const Span planes = PART ? planes_p : Span{1, N}, in = PART ? in_p : Span{0, N}, out = PART ? out_p : Span{0, N};
+  const int ntiles = NX * (planes.hi - planes.lo);
+  const uint32_t bytes = (uint32_t)((in.hi - in.lo) * W * sizeof(float));
   extern __shared__ __align__(128) unsigned char smem_tma[];
   float* buf0 = reinterpret_cast<float*>(smem_tma);
   float* buf1 = buf0 + N * W;
@@ -709,18 +773,18 @@ __global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const _
   if (skip != nullptr && *skip != 0) return;
   pdl_launch_next();
   __syncthreads();
-  auto coords = [&](int t, int& x, int& y, int& z) {
-    const int q = t / NX + 1;
+  auto coords = [&](int t, int row, int& x, int& y, int& z) {
+    const int q = t / NX + planes.lo;
     x = (t % NX) * W;
-    y = mode == 0 ? 0 : q;
-    z = mode == 0 ? q : 0;
+    y = mode == 0 ? row : q;
+    z = mode == 0 ? q : row;
   };
   int t = blockIdx.x;
   if (t < ntiles && threadIdx.x == 0) {
     int x, y, z;
-    coords(t, x, y, z);
+    coords(t, in.lo, x, y, z);
     mbar_expect_tx(&bar[0], bytes);
-    tma_load3(buf0, &map, &bar[0], x, y, z);
+    tma_load3(buf0 + in.lo * W, &map_in, &bar[0], x, y, z);
   }
   for (int i = 0; t < ntiles; t += gridDim.x, ++i) {
     const int b = i & 1;
@@ -730,9 +794,9 @@ __global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const _
     if (threadIdx.x == 0 && tn < ntiles) {
       tma_wait_read_all();  // the store of the previous tile has left s_next
       int x, y, z;
-      coords(tn, x, y, z);
+      coords(tn, in.lo, x, y, z);
       mbar_expect_tx(&bar[b ^ 1], bytes);
-      tma_load3(s_next, &map, &bar[b ^ 1], x, y, z);
+      tma_load3(s_next + in.lo * W, &map_in, &bar[b ^ 1], x, y, z);
     }
     bool ok = false;
     for (long it = 0; it < TMA_WAIT_CAP; ++it)
@@ -755,7 +819,15 @@ __global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const _
     {
       // forward DST with the spectral divide applied to its outputs, then the
       // inverse DST by the same (single inlined) body
-      const int q = t / NX + 1, p = (t % NX) * W + (int)(threadIdx.x & 31);
+      if (PART && in.hi - in.lo < N) {
+        // the buffer's other rows hold the tile before last's results
+        const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float4* s4 = reinterpret_cast<float4*>(s);
+        for (int i4 = threadIdx.x; i4 < in.lo * (W / 4); i4 += NT) s4[i4] = zero;
+        for (int i4 = in.hi * (W / 4) + threadIdx.x; i4 < N * (W / 4); i4 += NT) s4[i4] = zero;
+        __syncthreads();
+      }
+      const int q = t / NX + planes.lo, p = (t % NX) * W + (int)(threadIdx.x & 31);
       DivPost post{mus, mus[p] + mus[q] - lambda, scale, p == 0, SOLVE};
 #pragma unroll 1
       for (int rep = 0; rep < (SOLVE ? 2 : reps); ++rep) {
@@ -767,8 +839,8 @@ __global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const _
     __syncthreads();
     if (threadIdx.x == 0) {
       int x, y, z;
-      coords(t, x, y, z);
-      tma_store3(&map, s, x, y, z);
+      coords(t, out.lo, x, y, z);
+      tma_store3(&map_out, s + out.lo * W, x, y, z);
       tma_commit();
     }
   }
@@ -889,7 +961,8 @@ __global__ void __launch_bounds__(NT) k_xy_fwd(float* __restrict__ a, const doub
 template <int N>
 __global__ void __launch_bounds__(NT) k_xy_inv(float* __restrict__ a, bool keep, double* __restrict__ out,
                                                const double* __restrict__ aux, double beta, double gamma,
-                                               const float* __restrict__ tw_g, const int* __restrict__ skip) {
+                                               const float* __restrict__ tw_g, const int* __restrict__ skip,
+                                               const float* __restrict__ aux32) {
   using C = Cfg<float, N>;
   constexpr int W = C::W, RS = C::RS, n1 = N - 1, CL = N / W;
   static_assert(W == 32 && N % W == 0 && CL <= 8, "one cluster of at most 8 blocks per plane");
@@ -928,11 +1001,15 @@ __global__ void __launch_bounds__(NT) k_xy_inv(float* __restrict__ a, bool keep,
   for (int idx = threadIdx.x; idx < N * W; idx += NT) {
     const int x = idx % N, c = idx / N, y = y0 + c;
     const float v = sA[x * RS + c];
-    if (keep) a[plane + (size_t)y * N + x] = v;
+    const size_t pidx = plane + (size_t)y * N + x;
+    if (keep) a[pidx] = v;
     if (x > 0 && y > 0) {
       const size_t o = ((size_t)(z - 1) * n1 + (y - 1)) * n1 + (x - 1);
       const double bv = ffl::widen(b_t * v);
-      out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
+      if (aux32 != nullptr)
+        out[o] = bv + ffl::widen(aux32[pidx]);
+      else
+        out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
     }
   }
 }
@@ -981,52 +1058,93 @@ cudaError_t launch_pass(kfbi_handle* h, K kernel, dim3 grid, size_t smem, Args..
   return cudaGetLastError();
 }
 
+// what a strided pass covers: its planes, the rows it reads (the others are
+// zero) and the rows it writes
+struct PassSpan {
+  Span planes, in, out;
+};
+template <int N>
+PassSpan whole() {
+  return PassSpan{Span{1, N}, Span{0, N}, Span{0, N}};
+}
+
 // one strided 3-D pass (mode 0: along y, mode 1: along z); float32 grids of
 // 32 <= N <= 256 go through the TMA-fed persistent kernel
 template <typename T, int N>
 int launch_strided3(kfbi_handle* h, int mode, bool solve, T* work, const T* mu1, T lam, T scale, const T* tw,
-                    const T* rinv = nullptr) {
+                    const T* rinv, const PassSpan& ps) {
   using C = Cfg<T, N>;
-  cudaStream_t st = h->stream;
   int rc;
   if constexpr (sizeof(T) == 4 && N >= TMA_W && N <= 256) {
-    // the handle's second float grid has its own tensor maps
     const bool second = (const void*)work == (const void*)h->w.grid32b;
-    if (h->tma && (!second || h->tma_b)) {
+    if (h->tma) {
       constexpr size_t smem = tma_smem_bytes<N>();
-      const CUtensorMap& map =
-          mode == 0 ? (second ? h->tmap_y32b : h->tmap_y32) : (second ? h->tmap_z32b : h->tmap_z32);
-      const int tiles = (N / TMA_W) * (N - 1);
+      const CUtensorMap& min = h->tmap[second][ps.in.hi - ps.in.lo < N][mode];
+      const CUtensorMap& mout = h->tmap[second][ps.out.hi - ps.out.lo < N][mode];
+      const int tiles = (N / TMA_W) * (ps.planes.hi - ps.planes.lo);
       const int nb = (solve ? tma_blocks<true>() : tma_blocks<false>()) * h->sms;
       const int grid = tiles < nb ? tiles : nb;
-      cudaError_t e;
-      if (solve) {
-        if ((rc = prep(k_strided_tma<N, true>, smem))) return rc;
-        e = launch_pdl(k_strided_tma<N, true>, dim3(grid), dim3(NT), smem, st, map, mode, mu1, lam, scale, tw,
-                       h->w.err, 2, (const int*)h->skip);
-      } else {
-        if ((rc = prep(k_strided_tma<N, false>, smem))) return rc;
-        e = launch_pdl(k_strided_tma<N, false>, dim3(grid), dim3(NT), smem, st, map, mode, mu1, lam, scale, tw,
-                       h->w.err, 1, (const int*)h->skip);
-      }
-      return e == cudaSuccess ? KFBI_OK : launch_failed("TMA strided pass");
+      const bool part = ps.planes.hi - ps.planes.lo < N - 1 || ps.in.hi - ps.in.lo < N || ps.out.hi - ps.out.lo < N;
+      auto go = [&](auto kernel, int reps) -> int {
+        if (int e = prep(kernel, smem)) return e;
+        return launch_pdl(kernel, dim3(grid), dim3(NT), smem, h->stream, min, mout, mode, ps.planes, ps.in, ps.out, mu1,
+                          lam, scale, tw, h->w.err, reps, (const int*)h->skip) == cudaSuccess
+                   ? KFBI_OK
+                   : launch_failed("TMA strided pass");
+      };
+      if (solve) return part ? go(k_strided_tma<N, true, true>, 2) : go(k_strided_tma<N, true, false>, 2);
+      return part ? go(k_strided_tma<N, false, true>, 1) : go(k_strided_tma<N, false, false>, 1);
     }
   }
   const size_t smem = C::smem_elems * sizeof(T);
   const size_t NN = (size_t)N * N;
-  dim3 grid(N / C::W, N - 1);
-  const size_t rs = mode == 0 ? (size_t)N : NN, ps = mode == 0 ? NN : (size_t)N;
+  const dim3 grid(N / C::W, ps.planes.hi - ps.planes.lo);
+  const size_t rstride = mode == 0 ? (size_t)N : NN, pstride = mode == 0 ? NN : (size_t)N;
   cudaError_t e;
   if (solve) {
     if ((rc = prep(k_strided<T, N, true, 3>, smem))) return rc;
-    e = launch_pass(h, k_strided<T, N, true, 3>, grid, smem, work, rs, ps, 1, mu1, lam, scale, tw, (const int*)h->skip,
-                    rinv, 2);
+    e = launch_pass(h, k_strided<T, N, true, 3>, grid, smem, work, rstride, pstride, ps.planes.lo, mu1, lam, scale, tw,
+                    (const int*)h->skip, rinv, 2, ps.in, ps.out);
   } else {
     if ((rc = prep(k_strided<T, N, false, 3>, smem))) return rc;
-    e = launch_pass(h, k_strided<T, N, false, 3>, grid, smem, work, rs, ps, 1, mu1, lam, scale, tw,
-                    (const int*)h->skip, (const T*)nullptr, 1);
+    e = launch_pass(h, k_strided<T, N, false, 3>, grid, smem, work, rstride, pstride, ps.planes.lo, mu1, lam, scale, tw,
+                    (const int*)h->skip, (const T*)nullptr, 1, ps.in, ps.out);
   }
   return e == cudaSuccess ? KFBI_OK : launch_failed("strided pass");
+}
+
+// The passes of a 3-D solve and what each covers.  With corrections alone as
+// the right-hand side (no source field) the grid is zero outside the ranges
+// near_y, near_z of the irregular nodes: x lines outside them and planes
+// outside near_z are not transformed, and the y and z passes take those rows
+// as zero.  With only the interface limit reading the solution (near_only)
+// the z pass writes near_z alone, the y pass its planes and the rows near_y,
+// the x pass those lines.  The values computed are the same bit for bit.
+struct SolveSpans {
+  PassSpan yf, z, yi;
+  Span xf_y, xf_z, xi_y, xi_z;  // lines and planes of the x passes
+};
+inline bool near_source(const kfbi_handle* h, const SolveArgs& sa) {
+  return sa.src == nullptr && sa.src32 == nullptr && sa.corr != nullptr && h->near_y.hi > 0;
+}
+inline bool near_result(const kfbi_handle* h, const SolveArgs& sa) {
+  return sa.near_only && sa.out_user == nullptr && h->near_y.hi > 0;
+}
+template <int N>
+SolveSpans solve_spans(const kfbi_handle* h, bool in, bool out) {
+  const Span all{0, N}, planes{1, N};
+  const Span iy = in ? h->near_y : all, iz = in ? h->near_z : all;
+  const Span oy = out ? h->near_y : all, oz = out ? h->near_z : all;
+  auto from1 = [](Span s) { return Span{s.lo < 1 ? 1 : s.lo, s.hi}; };
+  SolveSpans s;
+  s.xf_y = iy;
+  s.xf_z = from1(iz);
+  s.yf = PassSpan{from1(iz), iy, all};
+  s.z = PassSpan{planes, iz, oz};
+  s.yi = PassSpan{from1(oz), all, oy};
+  s.xi_y = oy;
+  s.xi_z = from1(oz);
+  return s;
 }
 
 // scale / mu_p over the mode grid (q, k, p) of the float64 middle pass,
@@ -1094,9 +1212,9 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
         cudaError_t e = launch_cluster(k_xy_fwd<N>, N / 32, grid, sxy, st, work, sa.src, sa.alpha, sa.src32, sa.corr,
                                        (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, h->skip);
         if (e == cudaSuccess) {
-          if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw))) return rc;
+          if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, nullptr, whole<N>()))) return rc;
           e = launch_cluster(k_xy_inv<N>, N / 32, grid, sxy, st, work, sa.keep || sa.out_user == nullptr,
-                             sa.out_user, sa.aux, sa.beta, sa.gamma, tw, h->skip);
+                             sa.out_user, sa.aux, sa.beta, sa.gamma, tw, h->skip, sa.aux32);
           if (e != cudaSuccess) {
             set_error("cluster launch of the fused x-y inverse pass failed: %s", cudaGetErrorString(e));
             return KFBI_ERR_CUDA;
@@ -1113,14 +1231,18 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
     if ((rc = prep(k_xfwd<T, N, 3>, smem))) return rc;
     if ((rc = prep(k_xinv<T, N, 3>, smem))) return rc;
     // the five passes chained by programmatic dependent launch
-    if (launch_pass(h, k_xfwd<T, N, 3>, grid, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, (const int32_t*)t.irr,
-                    (const int32_t*)t.line_start, tw, (const int*)h->skip) != cudaSuccess)
+    const SolveSpans sp = solve_spans<N>(h, near_source(h, sa), near_result(h, sa));
+    const dim3 gf((sp.xf_y.hi - sp.xf_y.lo) / W, sp.xf_z.hi - sp.xf_z.lo);
+    const dim3 gi((sp.xi_y.hi - sp.xi_y.lo) / W, sp.xi_z.hi - sp.xi_z.lo);
+    if (launch_pass(h, k_xfwd<T, N, 3>, gf, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, (const int32_t*)t.irr,
+                    (const int32_t*)t.line_start, tw, (const int*)h->skip, sp.xf_y.lo, sp.xf_z.lo) != cudaSuccess)
       return launch_failed("x forward pass");
-    if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw))) return rc;
-    if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, rinv))) return rc;
-    if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw))) return rc;
-    if (launch_pass(h, k_xinv<T, N, 3>, grid, smem, work, sa.keep || sa.out_user == nullptr, sa.out_user,
-                    (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32) != cudaSuccess)
+    if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, sp.yf))) return rc;
+    if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, rinv, sp.z))) return rc;
+    if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, sp.yi))) return rc;
+    if (launch_pass(h, k_xinv<T, N, 3>, gi, smem, work, sa.keep || sa.out_user == nullptr, sa.out_user,
+                    (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32, sp.xi_y.lo,
+                    sp.xi_z.lo) != cudaSuccess)
       return launch_failed("x inverse pass");
   } else {
     dim3 grid(N / W, 1);
@@ -1129,13 +1251,13 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
     if ((rc = prep(k_strided<T, N, true, 2>, smem))) return rc;
     if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
     if (launch_pass(h, k_xfwd<T, N, 2>, grid, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, (const int32_t*)t.irr,
-                    (const int32_t*)t.line_start, tw, (const int*)h->skip) != cudaSuccess)
+                    (const int32_t*)t.line_start, tw, (const int*)h->skip, 0, 0) != cudaSuccess)
       return launch_failed("x forward pass");
     if (launch_pass(h, k_strided<T, N, true, 2>, grid, smem, work, (size_t)N, (size_t)0, 0, mu1, lam, scale, tw,
-                    (const int*)h->skip, rinv, 2) != cudaSuccess)
+                    (const int*)h->skip, rinv, 2, Span{0, N}, Span{0, N}) != cudaSuccess)
       return launch_failed("y solve pass");
     if (launch_pass(h, k_xinv<T, N, 2>, grid, smem, work, sa.keep || sa.out_user == nullptr, sa.out_user,
-                    (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32) != cudaSuccess)
+                    (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32, 0, 0) != cudaSuccess)
       return launch_failed("x inverse pass");
   }
   KFBI_CHECK_LAUNCH_N(dim == 3 ? 5 : 3);
@@ -1159,15 +1281,16 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
   if (dim == 3) {
     if (pass == 0) {
       if ((rc = prep(k_xfwd<T, N, 3>, smem))) return rc;
-      k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, t.irr, t.line_start, tw, nullptr);
+      k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, t.irr, t.line_start, tw, nullptr, 0,
+                                               1);
     } else if (pass == 1) {
-      if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw))) return rc;
+      if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, whole<N>()))) return rc;
     } else if (pass == 2) {
       const T* rinv = mode_factors<T, N>(h, lambda, (double)scale);
-      if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, rinv))) return rc;
+      if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, rinv, whole<N>()))) return rc;
     } else if (pass == 3) {
       if ((rc = prep(k_xinv<T, N, 3>, smem))) return rc;
-      k_xinv<T, N, 3><<<grid, NT, smem, st>>>(work, true, nullptr, nullptr, 1.0, 0.0, tw, nullptr);
+      k_xinv<T, N, 3><<<grid, NT, smem, st>>>(work, true, nullptr, nullptr, 1.0, 0.0, tw, nullptr, nullptr, 0, 1);
     } else {
       // 4 / 5: the fused x-y forward / inverse pass
       if constexpr (sizeof(T) == 4 && N >= 32 && N <= 256) {
@@ -1182,7 +1305,7 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
           } else {
             if ((rc = prep(k_xy_inv<N>, sxy))) return rc;
             e = launch_cluster(k_xy_inv<N>, N / 32, grid, sxy, st, work, true, (double*)nullptr,
-                               (const double*)nullptr, 1.0, 0.0, tw, (const int*)nullptr);
+                               (const double*)nullptr, 1.0, 0.0, tw, (const int*)nullptr, (const float*)nullptr);
           }
           if (e != cudaSuccess) {
             set_error("cluster launch failed: %s", cudaGetErrorString(e));
@@ -1199,14 +1322,16 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
   } else {
     if (pass == 0) {
       if ((rc = prep(k_xfwd<T, N, 2>, smem))) return rc;
-      k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, t.irr, t.line_start, tw, nullptr);
+      k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, t.irr, t.line_start, tw, nullptr, 0,
+                                               0);
     } else if (pass == 1 || pass == 2) {
       const T* rinv = mode_factors<T, N>(h, lambda, (double)scale);
       if ((rc = prep(k_strided<T, N, true, 2>, smem))) return rc;
-      k_strided<T, N, true, 2><<<grid, NT, smem, st>>>(work, N, 0, 0, mu1, lam, scale, tw, nullptr, rinv, 2);
+      k_strided<T, N, true, 2><<<grid, NT, smem, st>>>(work, N, 0, 0, mu1, lam, scale, tw, nullptr, rinv, 2, Span{0, N},
+                                                       Span{0, N});
     } else {
       if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
-      k_xinv<T, N, 2><<<grid, NT, smem, st>>>(work, true, nullptr, nullptr, 1.0, 0.0, tw, nullptr);
+      k_xinv<T, N, 2><<<grid, NT, smem, st>>>(work, true, nullptr, nullptr, 1.0, 0.0, tw, nullptr, nullptr, 0, 0);
     }
   }
   KFBI_CHECK_LAUNCH();
@@ -1227,24 +1352,29 @@ template <typename T, int N, int DIM>
 __global__ void __launch_bounds__(NT) k_strided_coupled(T* __restrict__ a, T* __restrict__ b, size_t row_stride,
                                                         size_t plane_stride, int qoff, const T* __restrict__ cf,
                                                         size_t cf_stride, const T* __restrict__ tw_g,
-                                                        const int* __restrict__ skip) {
+                                                        const int* __restrict__ skip, Span in, Span out) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sa = reinterpret_cast<T*>(smem_raw);
   T* sb = sa + N * RS;
   T* mem = sb + N * RS;
-  const bool skipped = skip != nullptr && *skip != 0;
   load_tables<C>(mem, tw_g);
-  if (skipped) return;
+  pdl_wait();
+  if (skip != nullptr && *skip != 0) return;
   const int x0 = blockIdx.x * W;
   const int q = blockIdx.y + qoff;
   T* ba = a + (size_t)q * plane_stride + x0;
   T* bb = b + (size_t)q * plane_stride + x0;
   for (int idx = threadIdx.x; idx < N * W; idx += NT) {
     const int c = idx % W, k = idx / W;
-    copy_async(&sa[k * RS + c], &ba[(size_t)k * row_stride + c]);
-    copy_async(&sb[k * RS + c], &bb[(size_t)k * row_stride + c]);
+    if (k >= in.lo && k < in.hi) {
+      copy_async(&sa[k * RS + c], &ba[(size_t)k * row_stride + c]);
+      copy_async(&sb[k * RS + c], &bb[(size_t)k * row_stride + c]);
+    } else {
+      sa[k * RS + c] = (T)0;
+      sb[k * RS + c] = (T)0;
+    }
   }
   copy_async_wait();
   __syncthreads();
@@ -1263,7 +1393,7 @@ __global__ void __launch_bounds__(NT) k_strided_coupled(T* __restrict__ a, T* __
   __syncthreads();
 #pragma unroll 1
   for (int f = 0; f < 2; ++f) dst_tile<C>(f == 0 ? sa : sb, mem);
-  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
+  for (int idx = threadIdx.x + out.lo * W; idx < out.hi * W; idx += NT) {
     const int c = idx % W, k = idx / W;
     ba[(size_t)k * row_stride + c] = sa[k * RS + c];
     bb[(size_t)k * row_stride + c] = sb[k * RS + c];
@@ -1351,30 +1481,46 @@ int run_solve_coupled(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, 
     if ((rc = prep(k_xfwd<T, N, 3>, smem))) return rc;
     if ((rc = prep(k_strided_coupled<T, N, 3>, smem2))) return rc;
     if ((rc = prep(k_xinv<T, N, 3>, smem))) return rc;
-    if ((rc = prep(k_strided<T, N, false, 3>, smem))) return rc;
-    k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(wa, si.src, si.alpha, si.src32, si.corr, t.irr, t.line_start, tw, h->skip);
-    k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(wb, se.src, se.alpha, se.src32, se.corr, t.irr, t.line_start, tw, h->skip);
+    const SolveSpans sp = solve_spans<N>(h, near_source(h, si) && near_source(h, se),
+                                         near_result(h, si) && near_result(h, se));
+    const SolveArgs* sas[2] = {&si, &se};
+    T* grids[2] = {wa, wb};
     const size_t NN = (size_t)N * N;
-    for (T* w : {wa, wb})
-      k_strided<T, N, false, 3><<<grid, NT, smem, st>>>(w, N, NN, 1, mu1T, (T)0, (T)1, tw, h->skip, nullptr, 1);
-    k_strided_coupled<T, N, 3><<<grid, NT, smem2, st>>>(wa, wb, NN, N, 1, cf, (size_t)total, tw, h->skip);
-    for (T* w : {wa, wb})
-      k_strided<T, N, false, 3><<<grid, NT, smem, st>>>(w, N, NN, 1, mu1T, (T)0, (T)1, tw, h->skip, nullptr, 1);
-    k_xinv<T, N, 3><<<grid, NT, smem, st>>>(wa, si.keep || si.out_user == nullptr, si.out_user, si.aux, si.beta,
-                                             si.gamma, tw, h->skip);
-    k_xinv<T, N, 3><<<grid, NT, smem, st>>>(wb, se.keep || se.out_user == nullptr, se.out_user, se.aux, se.beta,
-                                             se.gamma, tw, h->skip);
+    for (int f = 0; f < 2; ++f) {
+      const SolveArgs& sa = *sas[f];
+      const dim3 gf((sp.xf_y.hi - sp.xf_y.lo) / W, sp.xf_z.hi - sp.xf_z.lo);
+      if (launch_pass(h, k_xfwd<T, N, 3>, gf, smem, grids[f], sa.src, sa.alpha, sa.src32, sa.corr,
+                      (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, (const int*)h->skip, sp.xf_y.lo,
+                      sp.xf_z.lo) != cudaSuccess)
+        return launch_failed("x forward pass");
+      if ((rc = launch_strided3<T, N>(h, 0, false, grids[f], mu1T, (T)0, (T)1, tw, nullptr, sp.yf))) return rc;
+    }
+    if (launch_pass(h, k_strided_coupled<T, N, 3>, grid, smem2, wa, wb, NN, (size_t)N, 1, cf, (size_t)total, tw,
+                    (const int*)h->skip, sp.z.in, sp.z.out) != cudaSuccess)
+      return launch_failed("coupled z pass");
+    for (int f = 0; f < 2; ++f) {
+      const SolveArgs& sa = *sas[f];
+      const dim3 gi((sp.xi_y.hi - sp.xi_y.lo) / W, sp.xi_z.hi - sp.xi_z.lo);
+      if ((rc = launch_strided3<T, N>(h, 0, false, grids[f], mu1T, (T)0, (T)1, tw, nullptr, sp.yi))) return rc;
+      if (launch_pass(h, k_xinv<T, N, 3>, gi, smem, grids[f], sa.keep || sa.out_user == nullptr, sa.out_user,
+                      (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, (const float*)nullptr,
+                      sp.xi_y.lo, sp.xi_z.lo) != cudaSuccess)
+        return launch_failed("x inverse pass");
+    }
   } else {
     if ((rc = prep(k_xfwd<T, N, 2>, smem))) return rc;
     if ((rc = prep(k_strided_coupled<T, N, 2>, smem2))) return rc;
     if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
-    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wa, si.src, si.alpha, si.src32, si.corr, t.irr, t.line_start, tw, h->skip);
-    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wb, se.src, se.alpha, se.src32, se.corr, t.irr, t.line_start, tw, h->skip);
-    k_strided_coupled<T, N, 2><<<grid, NT, smem2, st>>>(wa, wb, N, 0, 0, cf, (size_t)total, tw, h->skip);
+    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wa, si.src, si.alpha, si.src32, si.corr, t.irr, t.line_start, tw, h->skip,
+                                             0, 0);
+    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wb, se.src, se.alpha, se.src32, se.corr, t.irr, t.line_start, tw, h->skip,
+                                             0, 0);
+    k_strided_coupled<T, N, 2><<<grid, NT, smem2, st>>>(wa, wb, N, 0, 0, cf, (size_t)total, tw, h->skip, Span{0, N},
+                                                        Span{0, N});
     k_xinv<T, N, 2><<<grid, NT, smem, st>>>(wa, si.keep || si.out_user == nullptr, si.out_user, si.aux, si.beta,
-                                             si.gamma, tw, h->skip);
+                                             si.gamma, tw, h->skip, nullptr, 0, 0);
     k_xinv<T, N, 2><<<grid, NT, smem, st>>>(wb, se.keep || se.out_user == nullptr, se.out_user, se.aux, se.beta,
-                                             se.gamma, tw, h->skip);
+                                             se.gamma, tw, h->skip, nullptr, 0, 0);
   }
   KFBI_CHECK_LAUNCH_N(dim == 3 ? 9 : 5);
   return KFBI_OK;
@@ -1594,7 +1740,8 @@ __global__ void __launch_bounds__(NT) k_nxfwd(T* __restrict__ a, const double* _
 template <typename T, int N, int DIM>
 __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, double* __restrict__ out,
                                               const double* __restrict__ aux, double beta, double gamma,
-                                              const T* __restrict__ tw_g, const int* __restrict__ skip) {
+                                              const T* __restrict__ tw_g, const int* __restrict__ skip,
+                                              const float* __restrict__ aux32) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, P = N + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1625,7 +1772,10 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
     if (keep) a[o] = v;
     if (out != nullptr) {
       const double bv = to_double((T)beta * v);
-      out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
+      if (aux32 != nullptr)
+        out[o] = bv + ffl::widen(aux32[o]);
+      else
+        out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
     }
   }
 }
@@ -1703,7 +1853,7 @@ int run_solve_neumann(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1
     k_nstrided<T, N, true, 3><<<grid, NT, smem, st>>>(work, PP, P, mu1, lam, scale, tw, h->skip, rinv);
     k_nstrided<T, N, false, 3><<<grid, NT, smem, st>>>(work, P, PP, mu1, lam, scale, tw, h->skip);
     k_nxinv<T, N, 3><<<grid, NT, smem, st>>>(work, sa.keep || sa.out_user == nullptr, sa.out_user, sa.aux, sa.beta,
-                                              sa.gamma, tw, h->skip);
+                                              sa.gamma, tw, h->skip, sa.aux32);
     KFBI_CHECK_LAUNCH_N(5);
   } else {
     if ((rc = prep(k_nxfwd<T, N, 2>, smem))) return rc;
@@ -1713,7 +1863,7 @@ int run_solve_neumann(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1
                                                 h->skip);
     k_nstrided<T, N, true, 2><<<grid, NT, smem, st>>>(work, P, 0, mu1, lam, scale, tw, h->skip, rinv);
     k_nxinv<T, N, 2><<<grid, NT, smem, st>>>(work, sa.keep || sa.out_user == nullptr, sa.out_user, sa.aux, sa.beta,
-                                              sa.gamma, tw, h->skip);
+                                              sa.gamma, tw, h->skip, sa.aux32);
     KFBI_CHECK_LAUNCH_N(3);
   }
   return KFBI_OK;
@@ -1767,28 +1917,22 @@ int make_tma_maps(kfbi_handle* h) {
   const cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)N, (cuuint64_t)N};
   const cuuint64_t strides[2] = {(cuuint64_t)N * sizeof(float), (cuuint64_t)N * N * sizeof(float)};
   const cuuint32_t estr[3] = {1, 1, 1};
-  const cuuint32_t box_y[3] = {(cuuint32_t)TMA_W, (cuuint32_t)N, 1};
-  const cuuint32_t box_z[3] = {(cuuint32_t)TMA_W, 1, (cuuint32_t)N};
-  CUresult r1 = encode(&h->tmap_y32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->w.grid32, dims, strides, box_y, estr,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  CUresult r2 = encode(&h->tmap_z32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->w.grid32, dims, strides, box_z, estr,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS) {
-    set_error("cuTensorMapEncodeTiled failed (%d, %d)", (int)r1, (int)r2);
-    return KFBI_ERR_CUDA;
-  }
+  for (int second = 0; second < 2; ++second)
+    for (int near = 0; near < 2; ++near)
+      for (int axis = 0; axis < 2; ++axis) {
+        const Span r = near == 0 ? Span{0, N} : axis == 0 ? h->near_y : h->near_z;
+        const cuuint32_t rows = (cuuint32_t)(r.hi - r.lo);
+        const cuuint32_t box[3] = {(cuuint32_t)TMA_W, axis == 0 ? rows : 1, axis == 0 ? 1 : rows};
+        const CUresult e = encode(&h->tmap[second][near][axis], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+                                  second ? h->w.grid32b : h->w.grid32, dims, strides, box, estr,
+                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (e != CUDA_SUCCESS) {
+          set_error("cuTensorMapEncodeTiled failed (%d)", (int)e);
+          return KFBI_ERR_CUDA;
+        }
+      }
   h->tma = true;
-  if (h->w.grid32b != nullptr) {
-    r1 = encode(&h->tmap_y32b, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->w.grid32b, dims, strides, box_y, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    r2 = encode(&h->tmap_z32b, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, h->w.grid32b, dims, strides, box_z, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    h->tma_b = r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS;
-  }
   // fused x-y passes need cluster launches (a cluster of N/32 blocks per
   // plane).  They pay off only for small planes: measured per float32 solve
   // (CUDA events, back-to-back) 18.8 against 24.4 us at 64^3, 48.4 against

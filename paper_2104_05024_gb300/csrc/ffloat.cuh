@@ -106,6 +106,25 @@ FF_HD bool split(double x, ff& out) {
   return true;
 }
 
+// x = h + m + l exactly (24, 24 and 5 significant bits); for |x| < 2^-60 all
+// three are 0.  Returns false where split() does.
+FF_HD bool split3(double x, float& h, float& m, float& l) {
+  const uint64_t b = bits64(x);
+  const int E = (int)((b >> 52) & 0x7ff);
+  if (E < 1023 - 60) {
+    h = m = l = 0.0f;
+    return true;
+  }
+  if (E >= 1023 + 128) return false;
+  const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+  const uint64_t f = b & 0xFFFFFFFFFFFFFull;
+  h = from_bits32(sign | ((uint32_t)(E - 896) << 23) | (uint32_t)(f >> 29));
+  const float scale = from_bits32(sign | ((uint32_t)(E - 948) << 23));
+  m = u29_to_float((uint32_t)(f & 0x1FFFFFE0u)) * scale;
+  l = u29_to_float((uint32_t)(f & 31u)) * scale;
+  return true;
+}
+
 // the float nearest to x (from its pair: off by one unit only within 2^-48
 // |x| of a rounding tie; 0 below 2^-60; infinities beyond the float range
 // and for infinite x; NaN for NaN)

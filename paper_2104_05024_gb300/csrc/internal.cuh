@@ -204,13 +204,14 @@ struct Workspace {
   double* psi_learn = nullptr;    // [M] learned initial guess
   double* g_prev = nullptr;       // [M] right-hand side of the previous diffusion solve
   double* u64 = nullptr;          // user-layout float64 grid (refined solutions)
-  double* res64 = nullptr;        // user-layout float64 grid (refinement residuals)
+  double* res64 = nullptr;        // user-layout float64 grid (coupled refinement residuals)
   double* vV64 = nullptr;         // user-layout float64 volume solution v_V of the step
   double* fsrc = nullptr;         // user-layout float64 source of a stimulated step
   double* S64 = nullptr;          // user-layout float64 S = sigma_i Phi_i + sigma_e Phi_e
   double* psiS = nullptr;         // [M] density of the S problem
   double* zeroM = nullptr;        // [M] zeros (homogeneous Neumann data)
   float* res32 = nullptr;         // user-layout float32 grid (refinement residuals)
+  float* res32lo = nullptr;       // their remainders (second round)
   double* hist_psi = nullptr;     // [KFBI_HISTORY][M] densities of past solves
   double* hist_g = nullptr;       // [KFBI_HISTORY][M] their right-hand sides
   double* psiF = nullptr;         // [M] projected density
@@ -238,6 +239,13 @@ struct Workspace {
 
 }  // namespace kfbi
 
+namespace kfbi {
+// index range [lo, hi) of one axis of the padded work grid
+struct Span {
+  int lo = 0, hi = 0;
+};
+}  // namespace kfbi
+
 struct kfbi_handle {
   kfbi::GeomParams gp;
   kfbi::GridParams grid;
@@ -261,10 +269,14 @@ struct kfbi_handle {
   kfbi::Tables t2;
   int nk = 0;
   kfbi_mlp* warm = nullptr;       // learned warm start (not owned)
-  // TMA descriptors of the float32 padded grid: [N x 32] tiles along y and z
-  CUtensorMap tmap_y32, tmap_z32;
-  CUtensorMap tmap_y32b, tmap_z32b;  // the same for the second float grid
-  bool tma_b = false;
+  // y and z ranges (3-D Dirichlet box, multiples of 16; the whole axis
+  // otherwise) that hold every irregular node and every interpolation
+  // stencil: a right-hand side of corrections alone is zero outside them, and
+  // an interface limit reads nothing outside them
+  kfbi::Span near_y, near_z;
+  // TMA descriptors of 32-column tiles of the float32 padded grids, [second
+  // grid][rows near the interface only][along z instead of y]
+  CUtensorMap tmap[2][2][2];
   bool tma = false;
   int sms = 152;                  // the device's multiprocessor count (persistent grids)
   bool xy_fused = false;          // float32 3-D solves use the cluster-fused x-y passes
@@ -324,6 +336,8 @@ struct SolveArgs {
   double lambda = 0.0;
   bool keep = true;               // the x inverse pass also writes the padded work grid
   const float* aux32 = nullptr;   // float32 solves: out_user = beta v + aux32 (a padded float grid)
+  bool near_only = false;         // only the interface limit reads the solution: the work grid
+                                  // holds it in the ranges near_y, near_z alone
 };
 int box_solve64(kfbi_handle* h, const SolveArgs& a, double* work);
 // the float64 box solve of the coupled pair (sources / corrections / outputs
@@ -367,17 +381,20 @@ int launch_limit64(kfbi_handle* h, const double* grid, const double* x, const do
 int launch_limit32(kfbi_handle* h, const float* grid, const double* x, const double* base, double sgn, double* out);
 int launch_scatter_grid(kfbi_handle* h, const double* corr, double* grid_user);
 int launch_limit_user(kfbi_handle* h, const double* u, const double* x, const double* base, double sgn, double* out);
-int launch_residual(kfbi_handle* h, const double* src, double alpha, const double* corr, const double* u, double lambda,
-                    double* res);
-// r = alpha*src + corr - L_h u (float32 result) for u held exactly by the
-// padded float32 grid u32 (the output of a float32 solve) and by u64 on the
+// the coupled system's first refinement residual (float32 result) for
+// (u_i, u_e) held exactly by the padded float32 grids and by ui, ue on the
 // user layout; float-float arithmetic away from the interface, float64 at
 // irregular nodes
 int launch_residual_ff_coupled(kfbi_handle* h, const double* src_i, double a_i, const double* src_e, double a_e,
                                const double* corr_i, const double* corr_e, const double* ui, const double* ue,
                                double kappa, float* ri, float* re);
+// res (+ res_lo) = alpha*src + corr - L_h u for u held exactly by the float32
+// work grid u32: float-float arithmetic, float64 at irregular nodes; res_lo
+// (optional) receives what the float res leaves out
 int launch_residual_ff(kfbi_handle* h, const double* src, double alpha, const double* corr, const float* u32,
-                       const double* u64, double lambda, float* res);
+                       double lambda, float* res, float* res_lo);
+// res <- (res + res_lo) - L_h u, the residual after one more correction u
+int launch_residual_pair(kfbi_handle* h, float* res, const float* res_lo, const float* u32, double lambda);
 int launch_lincomb(kfbi_handle* h, double* y, double a, const double* x, double b, int64_t n);
 // out += sgn <ds, psi> / |Gamma| (the rank-one term of the Poisson operator)
 int launch_rank_one(kfbi_handle* h, const double* psi, double* out, double sgn);

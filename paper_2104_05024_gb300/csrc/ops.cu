@@ -126,29 +126,6 @@ __global__ void k_limit_user(Tables t, GridParams gr, const double* __restrict__
   out[i] = (base != nullptr ? base[i] : 0.0) + sgn * acc;
 }
 
-// res = alpha*src - (L_h u) on the user layout, L_h the 5/7-point operator
-// with zero Dirichlet data (float64 residual of the refined box solve)
-// r = alpha*src - L_h u on the user layout; one block row per (y, z) grid line
-// so no index needs a 64-bit division.
-__global__ void k_residual(GridParams gr, const double* __restrict__ src, double alpha, const double* __restrict__ u,
-                           double lambda, double* __restrict__ res) {
-  const int n1 = gr.N - 1;
-  const double ih2 = 1.0 / (gr.h * gr.h);
-  const double diag = -2.0 * gr.dim * ih2 - lambda;
-  const int y = blockIdx.x, z = blockIdx.y;
-  const int64_t s = (int64_t)n1 * n1;
-  const int64_t base = (int64_t)z * s + (int64_t)y * n1;
-  for (int x = threadIdx.x; x < n1; x += blockDim.x) {
-    const int64_t f = base + x;
-    const double uc = u[f];
-    double nb = (x > 0 ? u[f - 1] : 0.0) + (x < n1 - 1 ? u[f + 1] : 0.0);
-    nb += (y > 0 ? u[f - n1] : 0.0) + (y < n1 - 1 ? u[f + n1] : 0.0);
-    if (gr.dim == 3) nb += (z > 0 ? u[f - s] : 0.0) + (z < n1 - 1 ? u[f + s] : 0.0);
-    const double Lu = nb * ih2 + diag * uc;
-    res[f] = (src != nullptr ? alpha * src[f] : 0.0) - Lu;
-  }
-}
-
 // error-free transformations: Knuth's TwoSum (s + e = a + b exactly) and the
 // product error by a fused multiply-add (p + e = a b exactly)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
@@ -175,186 +152,159 @@ __device__ __forceinline__ void src_pair(double sv, float& sh, float& sl) {
   }
 }
 
-// r = -L_h u for u given exactly by the padded float32 grid of a float32
-// solve (index 0 of each axis holds the zero boundary value), in float-float
-// arithmetic: the float64 pipe is 1/64 of the float32 rate here, and the
-// 6-point sum of float32 values, ih2 and the diagonal kept as float pairs
-// give L_h u to about 1e-14 of its terms, ample for a refinement residual
-// that is 1e-7 of them.  One block row per (y, z) line.
-__global__ void k_residual_ff(GridParams gr, const float* __restrict__ u32, float ih2_hi, float ih2_lo, float dg_hi,
-                              float dg_lo, const double* __restrict__ src, float al_hi, float al_lo,
-                              float* __restrict__ res) {
-  const int N = gr.N, n1 = N - 1;
+// Refinement residual r = src - L_h u for u given exactly by a float32 work
+// grid (the result of a float32 solve), in float arithmetic with error terms:
+// the float64 pipe is 1/64 of the float32 rate here.  With D the 6-point sum
+// minus 2 d u (exact TwoSums; its terms nearly cancel where u is smooth),
+// L_h u = D / h^2 - lambda u.
+//  - One round: float pairs, about 2^-47 of these two terms.
+//  - PAIR (two rounds): the source as three floats (all 53 bits) and the
+//    error terms themselves summed with errors, so that r carries what is
+//    left of the float64 source; res receives r as a float and res_lo its
+//    remainder.  (Float pairs here would cost the solution a factor of two
+//    in accuracy, a float64 residual 2.54 ms at 512^3.)
+//  - The second round's source is that pair: r minus L_h of the correction,
+//    float pairs again.
+struct FTrip {
+  float a, b, c;
+};
+enum class Src { none, field, pair };
+struct ResArgs {
+  const double* src;
+  double alpha;
+  FTrip ih2, lam, al;
+  const float *sh, *sl;  // pair source (may be the outputs themselves)
+  float *res, *res_lo;
+};
+template <bool NEUMANN, Src SRC, bool PAIR>
+__global__ void __launch_bounds__(128) k_residual_ff(GridParams gr, const float* __restrict__ u32, ResArgs A) {
+  // n values per field row, P per work-grid row (Neumann box: the grid is
+  // the field, a neighbour beyond the box its mirror image; Dirichlet box:
+  // index 0 of the grid and what lies beyond its last index is zero)
+  const int n = NEUMANN ? gr.N + 1 : gr.N - 1, P = NEUMANN ? gr.N + 1 : gr.N;
   const int y = blockIdx.x, z = blockIdx.y;
-  const size_t NN = (size_t)N * N;
-  const size_t pbase = gr.dim == 3 ? (size_t)(z + 1) * NN + (size_t)(y + 1) * N : (size_t)(y + 1) * N;
-  const size_t ubase = gr.dim == 3 ? ((size_t)z * n1 + y) * n1 : (size_t)y * n1;
-  for (int x = threadIdx.x; x < n1; x += blockDim.x) {
-    const size_t p = pbase + x + 1;
-    const float uc = u32[p];
-    float s = u32[p - 1], e = 0.0f, t;
-    two_sum(s, x < n1 - 1 ? u32[p + 1] : 0.0f, s, t);
+  const int64_t PP = (int64_t)P * P;
+  const bool d3 = gr.dim == 3;
+  const int64_t gbase = NEUMANN ? (int64_t)z * PP + (int64_t)y * P : (d3 ? (z + 1) * PP : 0) + (int64_t)(y + 1) * P + 1;
+  const int64_t fbase = ((int64_t)z * n + y) * n;
+  const int64_t ym = NEUMANN && y == 0 ? P : -P, yp = NEUMANN && y == n - 1 ? -P : P;
+  const int64_t zm = NEUMANN && z == 0 ? PP : -PP, zp = NEUMANN && z == n - 1 ? -PP : PP;
+  const bool y_on = NEUMANN || y < n - 1, z_on = NEUMANN || z < n - 1;
+#pragma unroll 2
+  for (int x = threadIdx.x; x < n; x += 128) {
+    const float* up = u32 + gbase + x;
+    const float uc = up[0];
+    const float xm = up[NEUMANN && x == 0 ? 1 : -1];
+    const float xp = NEUMANN ? up[x == n - 1 ? -1 : 1] : x < n - 1 ? up[1] : 0.0f;
+    const float um = up[ym], upl = y_on ? up[yp] : 0.0f;
+    float wm = 0.0f, wp = 0.0f;
+    if (d3) {
+      wm = up[zm];
+      wp = z_on ? up[zp] : 0.0f;
+    }
+    float q = 0.0f, m = 0.0f, l = 0.0f;  // the source
+    if (SRC == Src::field) {
+      double v = A.src[fbase + x];
+      if (PAIR) {
+        if (A.alpha != 1.0) v *= A.alpha;
+        if (!ffl::split3(v, q, m, l)) {
+          q = ffl::narrow(v);
+          m = l = 0.0f;
+        }
+      } else {
+        float vh, vl;
+        src_pair(v, vh, vl);
+        two_prod(A.al.a, vh, q, m);
+        m += A.al.a * vl + A.al.b * vh;
+      }
+    }
+    if (SRC == Src::pair) {
+      q = A.sh[fbase + x];
+      m = A.sl[fbase + x];
+    }
+    float s, e, t;
+    two_sum(xm, xp, s, e);
+    two_sum(s, um, s, t);
     e += t;
-    two_sum(s, u32[p - N], s, t);
+    two_sum(s, -2.0f * uc, s, t);
     e += t;
-    two_sum(s, y < n1 - 1 ? u32[p + N] : 0.0f, s, t);
+    two_sum(s, upl, s, t);
     e += t;
-    if (gr.dim == 3) {
-      two_sum(s, u32[p - NN], s, t);
+    two_sum(s, -2.0f * uc, s, t);
+    e += t;
+    if (d3) {
+      two_sum(s, wm, s, t);
       e += t;
-      two_sum(s, z < n1 - 1 ? u32[p + NN] : 0.0f, s, t);
+      two_sum(s, -2.0f * uc, s, t);
+      e += t;
+      two_sum(s, wp, s, t);
       e += t;
     }
-    float p1, e1, p2, e2, hsum, e3;
-    two_prod(ih2_hi, s, p1, e1);
-    e1 += ih2_hi * e + ih2_lo * s;
-    two_prod(dg_hi, uc, p2, e2);
-    e2 += dg_lo * uc;
-    two_sum(p1, p2, hsum, e3);
-    float lo = e1 + e2 + e3;
-    if (src != nullptr) {
-      // + alpha * src, src split into a float pair on its bits
-      const double sv = src[ubase + x];
-      float sh, sl;
-      src_pair(sv, sh, sl);
-      float q, eq, h2, e4;
-      two_prod(al_hi, sh, q, eq);
-      eq += al_hi * sl + al_lo * sh;
-      two_sum(q, -hsum, h2, e4);
-      res[ubase + x] = h2 + (e4 + eq - lo);
+    // r = source - (s + e) / h^2 + lambda u
+    float p1, e1, p2, e2, h, t0, rh, t1;
+    two_prod(A.ih2.a, s, p1, e1);
+    two_prod(-A.lam.a, uc, p2, e2);
+    two_sum(p1, p2, h, t0);
+    two_sum(q, -h, rh, t1);
+    float rl;
+    if (PAIR) {
+      float a1, b1, a2, b2, a3, b3;
+      two_prod(A.ih2.a, e, a1, b1);
+      two_prod(A.ih2.b, s, a2, b2);
+      two_prod(-A.lam.b, uc, a3, b3);
+      float c = t1, d = l - (b1 + b2 + b3 + A.ih2.b * e + A.ih2.c * s - A.lam.c * uc);
+      const float terms[7] = {m, -t0, -e1, -e2, -a1, -a2, -a3};
+#pragma unroll
+      for (int k = 0; k < 7; ++k) {
+        two_sum(c, terms[k], c, t);
+        d += t;
+      }
+      two_sum(rh, c, rh, rl);
+      rl += d;
     } else {
-      res[ubase + x] = -(hsum + lo);
+      e1 += A.ih2.a * e + A.ih2.b * s;
+      e2 -= A.lam.b * uc;
+      rl = t1 + (m - (e1 + e2 + t0));
     }
+    const float r = rh + rl;
+    A.res[fbase + x] = r;
+    if (PAIR) A.res_lo[fbase + x] = rl - (r - rh);
   }
 }
 
 // at the irregular nodes, where the correction makes r a small difference of
-// large terms: r = corr - L_h u in float64, from the float64 copy of u, or
-// (u == nullptr) from the padded float grid u32 that holds u exactly
-__global__ void k_residual_irr(GridParams gr, Tables t, const double* __restrict__ corr, const double* __restrict__ u,
-                               double lambda, const double* __restrict__ src, double alpha, float* __restrict__ res,
-                               const float* __restrict__ u32) {
+// large terms: r = src + corr - L_h u in float64 from the float grid (all
+// irregular nodes are interior: no neighbour beyond the box but the
+// Dirichlet box's zero last index)
+__global__ void k_residual_irr(GridParams gr, Tables t, const double* __restrict__ corr, double lambda,
+                               const double* __restrict__ src, double alpha, float* __restrict__ res,
+                               float* __restrict__ res_lo, const float* __restrict__ u32) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= t.n_irr) return;
-  const int N = gr.N, n1 = N - 1;
+  const bool neumann = gr.bc == KFBI_BOX_NEUMANN;
+  const int N = gr.N, n1 = N - 1, P = neumann ? N + 1 : N;
   const double ih2 = 1.0 / (gr.h * gr.h);
   const double diag = -2.0 * gr.dim * ih2 - lambda;
-  const int64_t f = t.irr[i];
-  const int64_t s = (int64_t)n1 * n1;
-  const int x = (int)(f % n1), y = (int)((f / n1) % n1), z = gr.dim == 3 ? (int)(f / s) : 0;
-  double uc, nb;
-  if (u != nullptr) {
-    uc = u[f];
-    nb = (x > 0 ? u[f - 1] : 0.0) + (x < n1 - 1 ? u[f + 1] : 0.0);
-    nb += (y > 0 ? u[f - n1] : 0.0) + (y < n1 - 1 ? u[f + n1] : 0.0);
-    if (gr.dim == 3) nb += (z > 0 ? u[f - s] : 0.0) + (z < n1 - 1 ? u[f + s] : 0.0);
-  } else {
-    // padded index of (x, y, z): index 0 of each axis is the zero boundary
-    const size_t NN = (size_t)N * N;
-    const size_t p = gr.dim == 3 ? ((size_t)(z + 1) * N + (y + 1)) * N + (x + 1) : (size_t)(y + 1) * N + (x + 1);
-    uc = ffl::widen(u32[p]);
-    nb = ffl::widen(u32[p - 1]) + (x < n1 - 1 ? ffl::widen(u32[p + 1]) : 0.0);
-    nb += ffl::widen(u32[p - N]) + (y < n1 - 1 ? ffl::widen(u32[p + N]) : 0.0);
-    if (gr.dim == 3) nb += ffl::widen(u32[p - NN]) + (z < n1 - 1 ? ffl::widen(u32[p + NN]) : 0.0);
-  }
-  const double a = src != nullptr ? alpha * src[f] : 0.0;
-  res[f] = (float)(a + corr[i] - (nb * ih2 + diag * uc));
-}
-
-// the float-float residual on the Neumann box's field layout: u32 is the
-// float32 work grid itself (all (N+1)^d nodes), a neighbour beyond the box
-// its mirror image
-__global__ void k_residual_ff_neumann(GridParams gr, const float* __restrict__ u32, float ih2_hi, float ih2_lo,
-                                      float dg_hi, float dg_lo, const double* __restrict__ src, float al_hi,
-                                      float al_lo, float* __restrict__ res) {
-  const int P = gr.N + 1;
-  const int y = blockIdx.x, z = blockIdx.y;
+  const int32_t f0 = t.irr[i];
+  // grid node (x, y, z) of the irregular node, 1-based
+  const int x = f0 % n1 + 1, y = (f0 / n1) % n1 + 1, z = gr.dim == 3 ? f0 / (n1 * n1) + 1 : 0;
   const int64_t PP = (int64_t)P * P;
-  const int64_t base = (int64_t)z * PP + (int64_t)y * P;
-  const int64_t ym = y > 0 ? -P : P, yp = y < P - 1 ? P : -P;
-  const int64_t zm = z > 0 ? -PP : PP, zp = z < P - 1 ? PP : -PP;
-  for (int x = threadIdx.x; x < P; x += blockDim.x) {
-    const int64_t f = base + x;
-    const float uc = u32[f];
-    float sm = u32[f + (x > 0 ? -1 : 1)], e = 0.0f, t;
-    two_sum(sm, u32[f + (x < P - 1 ? 1 : -1)], sm, t);
-    e += t;
-    two_sum(sm, u32[f + ym], sm, t);
-    e += t;
-    two_sum(sm, u32[f + yp], sm, t);
-    e += t;
-    if (gr.dim == 3) {
-      two_sum(sm, u32[f + zm], sm, t);
-      e += t;
-      two_sum(sm, u32[f + zp], sm, t);
-      e += t;
-    }
-    float p1, e1, p2, e2, hsum, e3;
-    two_prod(ih2_hi, sm, p1, e1);
-    e1 += ih2_hi * e + ih2_lo * sm;
-    two_prod(dg_hi, uc, p2, e2);
-    e2 += dg_lo * uc;
-    two_sum(p1, p2, hsum, e3);
-    const float lo = e1 + e2 + e3;
-    if (src != nullptr) {
-      const double sv = src[f];
-      float sh, sl;
-      src_pair(sv, sh, sl);
-      float q, eq, h2, e4;
-      two_prod(al_hi, sh, q, eq);
-      eq += al_hi * sl + al_lo * sh;
-      two_sum(q, -hsum, h2, e4);
-      res[f] = h2 + (e4 + eq - lo);
-    } else {
-      res[f] = -(hsum + lo);
-    }
-  }
-}
-
-// the irregular nodes of the Neumann box in float64 (interior nodes: no
-// mirrored neighbour)
-__global__ void k_residual_irr_neumann(GridParams gr, Tables t, const double* __restrict__ corr,
-                                       const double* __restrict__ u, double lambda, const double* __restrict__ src,
-                                       double alpha, float* __restrict__ res) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= t.n_irr) return;
-  const int P = gr.N + 1;
-  const double ih2 = 1.0 / (gr.h * gr.h);
-  const double diag = -2.0 * gr.dim * ih2 - lambda;
+  const int64_t p = (int64_t)z * PP + (int64_t)y * P + x;
+  const double uc = ffl::widen(u32[p]);
+  double nb = ffl::widen(u32[p - 1]) + (neumann || x < N - 1 ? ffl::widen(u32[p + 1]) : 0.0);
+  nb += ffl::widen(u32[p - P]) + (neumann || y < N - 1 ? ffl::widen(u32[p + P]) : 0.0);
+  if (gr.dim == 3) nb += ffl::widen(u32[p - PP]) + (neumann || z < N - 1 ? ffl::widen(u32[p + PP]) : 0.0);
   const int64_t f = t.irr_user[i];
-  const int64_t PP = (int64_t)P * P;
-  double nb = u[f - 1] + u[f + 1] + u[f - P] + u[f + P];
-  if (gr.dim == 3) nb += u[f - PP] + u[f + PP];
   const double a = src != nullptr ? alpha * src[f] : 0.0;
-  res[f] = (float)(a + corr[i] - (nb * ih2 + diag * u[f]));
+  const double r = a + corr[i] - (nb * ih2 + diag * uc);
+  const float rh = (float)r;
+  res[f] = rh;
+  if (res_lo != nullptr) res_lo[f] = (float)(r - (double)rh);
 }
 
 __global__ void k_scatter_add(Tables t, const double* __restrict__ corr, double* __restrict__ g) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < t.n_irr) g[t.irr_user[i]] += corr[i];
-}
-
-// r = alpha*src - L_h u on the Neumann box's field layout (all (N+1)^d
-// nodes; a neighbour beyond the box is the mirror image across it)
-__global__ void k_residual_neumann(GridParams gr, const double* __restrict__ src, double alpha,
-                                   const double* __restrict__ u, double lambda, double* __restrict__ res) {
-  const int P = gr.N + 1;
-  const double ih2 = 1.0 / (gr.h * gr.h);
-  const double diag = -2.0 * gr.dim * ih2 - lambda;
-  const int y = blockIdx.x, z = blockIdx.y;
-  const int64_t s = (int64_t)P * P;
-  const int64_t base = (int64_t)z * s + (int64_t)y * P;
-  const int64_t ym = y > 0 ? -P : P, yp = y < P - 1 ? P : -P;
-  const int64_t zm = z > 0 ? -s : s, zp = z < P - 1 ? s : -s;
-  for (int x = threadIdx.x; x < P; x += blockDim.x) {
-    const int64_t f = base + x;
-    const double uc = u[f];
-    double nb = u[f + (x > 0 ? -1 : 1)] + u[f + (x < P - 1 ? 1 : -1)];
-    nb += u[f + ym] + u[f + yp];
-    if (gr.dim == 3) nb += u[f + zm] + u[f + zp];
-    const double Lu = nb * ih2 + diag * uc;
-    res[f] = (src != nullptr ? alpha * src[f] : 0.0) - Lu;
-  }
 }
 
 __global__ void k_add_scalar(double* __restrict__ out, const double* __restrict__ slot, double c, int n) {
@@ -1054,45 +1004,51 @@ int launch_limit_user_t(kfbi_handle* h, const Tables& t, const double* u, const 
   return KFBI_OK;
 }
 
-int launch_residual(kfbi_handle* h, const double* src, double alpha, const double* corr, const double* u, double lambda,
-                    double* res) {
-  const int n1 = h->grid.N - 1;
-  if (h->grid.bc == KFBI_BOX_NEUMANN) {
-    const int P = h->grid.N + 1;
-    k_residual_neumann<<<dim3(P, h->grid.dim == 3 ? P : 1), 128, 0, h->stream>>>(h->grid, src, alpha, u, lambda,
-                                                                                   res);
-  } else {
-    k_residual<<<dim3(n1, h->grid.dim == 3 ? n1 : 1), 128, 0, h->stream>>>(h->grid, src, alpha, u, lambda, res);
-  }
-  if (corr != nullptr && h->t.n_irr > 0)
-    k_scatter_add<<<(h->t.n_irr + 127) / 128, 128, 0, h->stream>>>(h->t, corr, res);
-  KFBI_CHECK_LAUNCH_N(corr != nullptr && h->t.n_irr > 0 ? 2 : 1);
-  return KFBI_OK;
+struct FPair {
+  float hi, lo;
+};
+static FPair fpair(double v) {
+  const float hi = (float)v;
+  return {hi, (float)(v - (double)hi)};
+}
+static FTrip ftrip(double v) {
+  const float a = (float)v;
+  const double r = v - (double)a;
+  const float b = (float)r;
+  return {a, b, (float)(r - (double)b)};
+}
+
+template <Src SRC, bool PAIR>
+static void residual_ff(kfbi_handle* h, const float* u32, const ResArgs& A) {
+  const int n = field_n(h->grid);
+  const dim3 grid(n, h->grid.dim == 3 ? n : 1);
+  if (h->grid.bc == KFBI_BOX_NEUMANN)
+    k_residual_ff<true, SRC, PAIR><<<grid, 128, 0, h->stream>>>(h->grid, u32, A);
+  else
+    k_residual_ff<false, SRC, PAIR><<<grid, 128, 0, h->stream>>>(h->grid, u32, A);
 }
 
 int launch_residual_ff(kfbi_handle* h, const double* src, double alpha, const double* corr, const float* u32,
-                       const double* u64, double lambda, float* res) {
-  const int n1 = h->grid.N - 1;
-  const double ih2 = 1.0 / (h->grid.h * h->grid.h);
-  const double dg = -2.0 * h->grid.dim * ih2 - lambda;
-  const float ih2_hi = (float)ih2, dg_hi = (float)dg;
-  const float ih2_lo = (float)(ih2 - (double)ih2_hi), dg_lo = (float)(dg - (double)dg_hi);
-  const float al_hi = (float)alpha, al_lo = (float)(alpha - (double)al_hi);
-  if (h->grid.bc == KFBI_BOX_NEUMANN) {
-    const int P = h->grid.N + 1;
-    k_residual_ff_neumann<<<dim3(P, h->grid.dim == 3 ? P : 1), 128, 0, h->stream>>>(
-        h->grid, u32, ih2_hi, ih2_lo, dg_hi, dg_lo, src, al_hi, al_lo, res);
-    if (corr != nullptr && h->t.n_irr > 0)
-      k_residual_irr_neumann<<<(h->t.n_irr + 127) / 128, 128, 0, h->stream>>>(h->grid, h->t, corr, u64, lambda, src,
-                                                                              alpha, res);
-  } else {
-    k_residual_ff<<<dim3(n1, h->grid.dim == 3 ? n1 : 1), 128, 0, h->stream>>>(h->grid, u32, ih2_hi, ih2_lo, dg_hi,
-                                                                               dg_lo, src, al_hi, al_lo, res);
-    if (corr != nullptr && h->t.n_irr > 0)
-      k_residual_irr<<<(h->t.n_irr + 127) / 128, 128, 0, h->stream>>>(h->grid, h->t, corr, u64, lambda, src, alpha,
-                                                                      res, u32);
-  }
-  KFBI_CHECK_LAUNCH_N(corr != nullptr && h->t.n_irr > 0 ? 2 : 1);
+                       double lambda, float* res, float* res_lo) {
+  const ResArgs A{src,     alpha,   ftrip(1.0 / (h->grid.h * h->grid.h)), ftrip(lambda), ftrip(alpha),
+                  nullptr, nullptr, res,                                  res_lo};
+  if (res_lo != nullptr)
+    src ? residual_ff<Src::field, true>(h, u32, A) : residual_ff<Src::none, true>(h, u32, A);
+  else
+    src ? residual_ff<Src::field, false>(h, u32, A) : residual_ff<Src::none, false>(h, u32, A);
+  const bool irr = corr != nullptr && h->t.n_irr > 0;
+  if (irr)
+    k_residual_irr<<<(h->t.n_irr + 127) / 128, 128, 0, h->stream>>>(h->grid, h->t, corr, lambda, src, alpha, res,
+                                                                    res_lo, u32);
+  KFBI_CHECK_LAUNCH_N(irr ? 2 : 1);
+  return KFBI_OK;
+}
+
+int launch_residual_pair(kfbi_handle* h, float* res, const float* res_lo, const float* u32, double lambda) {
+  const ResArgs A{nullptr, 1.0, ftrip(1.0 / (h->grid.h * h->grid.h)), ftrip(lambda), ftrip(1.0), res, res_lo, res,
+                  nullptr};
+  residual_ff<Src::pair, false>(h, u32, A);
+  KFBI_CHECK_LAUNCH();
   return KFBI_OK;
 }
 
@@ -1212,15 +1168,6 @@ int launch_residual_coupled(kfbi_handle* h, const double* src_i, double a_i, con
   }
   KFBI_CHECK_LAUNCH_N(n);
   return KFBI_OK;
-}
-
-// float pair (hi + lo) of a float64 constant
-struct FPair {
-  float hi, lo;
-};
-FPair fpair(double v) {
-  const float hi = (float)v;
-  return {hi, (float)(v - (double)hi)};
 }
 
 struct CoupledStencilFF {

@@ -1692,6 +1692,36 @@ int setup_build(kfbi_handle* h, const kfbi_geometry* geom) {
     h->t2.mu32 = t.mu32;
     h->t2.tw32 = t.tw32;
   }
+  // ranges along y and z of the irregular nodes and the interpolation
+  // stencils (centre and its neighbours), rounded out to multiples of 16 and
+  // the y range to whole 32-line tiles
+  h->near_y = Span{0, N};
+  h->near_z = Span{0, N};
+  if (d == 3 && gr.bc == KFBI_BOX_DIRICHLET && N >= 32) {
+    std::vector<int32_t> irr((size_t)t.n_irr), cen((size_t)t.M * 3);
+    KFBI_CUDA(cudaMemcpyAsync(irr.data(), t.irr, sizeof(int32_t) * irr.size(), cudaMemcpyDeviceToHost, st));
+    KFBI_CUDA(cudaMemcpyAsync(cen.data(), t.n_center, sizeof(int32_t) * cen.size(), cudaMemcpyDeviceToHost, st));
+    KFBI_CUDA(cudaStreamSynchronize(st));
+    int lo[2] = {N, N}, hi[2] = {0, 0};
+    auto take = [&](int a, int k0, int k1) {
+      lo[a] = std::min(lo[a], k0);
+      hi[a] = std::max(hi[a], k1);
+    };
+    for (int32_t f : irr) {
+      const int y = (f / n1) % n1 + 1, z = f / (n1 * n1) + 1;
+      take(0, y, y);
+      take(1, z, z);
+    }
+    for (int i = 0; i < t.M; ++i)
+      for (int a = 0; a < 2; ++a) take(a, cen[3 * (size_t)i + 1 + a] - 1, cen[3 * (size_t)i + 1 + a] + 1);
+    Span* out[2] = {&h->near_y, &h->near_z};
+    for (int a = 0; a < 2; ++a)
+      *out[a] = Span{std::max(0, lo[a]) / 16 * 16, std::min(N, (hi[a] + 16) / 16 * 16)};
+    if ((h->near_y.hi - h->near_y.lo) % 32 != 0) {
+      if (h->near_y.lo > 0) h->near_y.lo -= 16;
+      else h->near_y.hi += 16;
+    }
+  }
   // inside count
   {
     std::vector<uint8_t> ins((size_t)total);

@@ -30,7 +30,7 @@ OBJECTS = {
     "mlp.o": ("mlp.cu", []),
 }
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-COMMON = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]
+COMMON = ["-std=c++17", "-O3", "-lineinfo", "-diag-suppress", "177", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]
 
 
 def nvcc() -> str:

@@ -83,8 +83,9 @@ struct Tile {
   // twiddles e^{i pi j/N} (2N complex) and sines (register path)
   static constexpr size_t mem_elems = FIX ? fixdst::table_words<N>() : (size_t)G * W + 4 * N + N;
   static constexpr size_t smem_elems = (size_t)N * RS + mem_elems;
-  // resident blocks per SM the registers are budgeted for
-  static constexpr int BLOCKS = FIX ? (N <= 256 ? 2 : 1) : 1;
+  // resident blocks per SM the registers are budgeted for (shared memory
+  // allows no more for long lines)
+  static constexpr int BLOCKS = FIX ? (N <= 256 ? 2 : 1) : REG ? (N <= 256 ? 3 : 2) : 1;
 };
 
 template <typename T, int N>
@@ -337,6 +338,10 @@ __device__ __forceinline__ void copy_async(T* dst_smem, const T* src) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst_smem));
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(sizeof(T)) : "memory");
 }
+__device__ __forceinline__ void copy_async16(void* dst_smem, const void* src) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst_smem));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // sines sin(pi j / N) for the register path's pre-fold (imaginary parts of tw)
@@ -366,11 +371,11 @@ struct NoMap {
 };
 
 // the DST-I of every column of the tile, rows 1..N-1; map: applied to the
-// outputs (register path) or to the inputs (fixed-point path)
+// outputs (register path only)
 template <typename C, class Map = NoMap>
 __device__ __forceinline__ void dst_tile(typename C::T* s, typename C::T* mem, const Map& map = Map()) {
   if constexpr (C::FIX) {
-    fixdst::dst1_tile_fix<fixdst::Geo<C::N, C::RS>>(s, reinterpret_cast<fixdst::ll*>(mem), map);
+    fixdst::dst1_tile_fix<fixdst::Geo<C::N, C::RS>>(s, reinterpret_cast<fixdst::ll*>(mem));
   } else if constexpr (C::REG) {
     const typename C::T* tw = mem + C::G * C::W;
     regdst::dst1_tile_reg<regdst::Geo<C::N, C::RS>>(s, tw + 4 * C::N, reinterpret_cast<const regdst::cf2*>(tw), mem,
@@ -391,24 +396,6 @@ struct DivPost {
   __device__ __forceinline__ float operator()(int j, float v) const {
     if (!on) return v;
     return zero ? 0.0f : v * __fdividef(scale, mu[j] + base);
-  }
-};
-
-// the same in float64, applied to the inputs of the inverse transform: the
-// factor from the table built for this lambda, or
-// divided here (handles without a table)
-struct FactorPre {
-  const double* r;  // table entry of this column's mode 0, row stride n (nullptr: none)
-  int n;
-  const double* mu;
-  double base;      // mu1[p] + mu1[q] - lambda
-  double scale;
-  bool zero;        // boundary column p = 0
-  bool on;
-  __device__ __forceinline__ double operator()(int j, double v) const {
-    if (!on) return v;
-    if (r != nullptr) return v * r[(size_t)j * n];
-    return zero || j == 0 ? 0.0 : v * (scale / (mu[j] + base));
   }
 };
 
@@ -470,7 +457,7 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xfwd(T* __restrict__ 
                                              const int* __restrict__ skip, int yoff, int zoff) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, n1 = N - 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
   T* mem = s + N * RS;
   load_tables<C>(mem, tw_g);
@@ -521,7 +508,7 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ 
                                              const float* __restrict__ aux32, int yoff, int zoff) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, n1 = N - 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
   T* mem = s + N * RS;
   load_tables<C>(mem, tw_g);
@@ -582,109 +569,11 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ 
   }
 }
 
-// --------------------------------------------------- strided (y / z) passes
-// Tile rows = transform index k (stride row_stride), columns x0..x0+W-1 of
-// plane q = blockIdx.y + qoff; rows outside `in` are zero and not read, rows
-// outside `out` are not written.  SOLVE = forward DST, spectral multiply,
-// inverse DST.
-template <typename T, int N, bool SOLVE, int DIM>
-__global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_strided(T* __restrict__ a, size_t row_stride, size_t plane_stride, int qoff,
-                                                const T* __restrict__ mu1, T lambda, T scale,
-                                                const T* __restrict__ tw_g, const int* __restrict__ skip,
-                                                const T* __restrict__ rinv, int reps, Span in, Span out) {
-  using C = Cfg<T, N>;
-  constexpr int W = C::W, RS = C::RS;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* s = reinterpret_cast<T*>(smem_raw);
-  T* mem = s + N * RS;
-  load_tables<C>(mem, tw_g);
-  pdl_wait();
-  if (skip != nullptr && *skip != 0) return;
-  const int x0 = blockIdx.x * W;
-  const int q = blockIdx.y + qoff;
-  T* base = a + (size_t)q * plane_stride + x0;
-  {
-    constexpr int DR = NT / W;
-    const int c = threadIdx.x % W, k0 = in.lo + threadIdx.x / W;
-    const T* src = base + (size_t)k0 * row_stride + c;
-    T* dst = s + k0 * RS + c;
-#pragma unroll 8
-    for (int k = k0; k < in.hi; k += DR, src += DR * row_stride, dst += DR * RS) copy_async(dst, src);
-    for (int k = threadIdx.x / W; k < in.lo; k += DR) s[k * RS + c] = (T)0;
-    for (int k = in.hi + threadIdx.x / W; k < N; k += DR) s[k * RS + c] = (T)0;
-  }
-  copy_async_wait();
-  __syncthreads();
-  const T muq = DIM == 3 ? mu1[q] : (T)0;
-  if constexpr (C::REG) {
-    if (SOLVE) {
-      const int p = x0 + (int)(threadIdx.x & 31);
-      // mu1 is read from global memory here (L1-resident, N values)
-      const DivPost post{mu1, mu1[p] + muq - lambda, scale, p == 0};
-      dst_tile<C>(s, mem, post);
-    }
-    dst_tile<C>(s, mem);
-  } else if constexpr (C::FIX) {
-    // forward DST, then by the same (single inlined) body the inverse DST,
-    // whose inputs are multiplied by the mode factors as they are read
-    if constexpr (SOLVE) {
-      const int p = x0 + (int)(threadIdx.x & 31);
-      FactorPre pre{rinv != nullptr ? rinv + ((size_t)q * N * N + p) : nullptr, N, mu1, mu1[p] + muq - lambda, scale,
-                    p == 0, false};
-#pragma unroll 1
-      for (int rep = 0; rep < reps; ++rep) {
-        dst_tile<C>(s, mem, pre);
-        pre.on = true;
-      }
-    } else {
-      dst_tile<C>(s, mem);
-    }
-  } else {
-    dst_tile<C>(s, mem);
-    if (SOLVE) {
-      // the mode factor scale / mu_p from the table built for this lambda
-      // (same expression, so the same value), else divided here
-      const T* rq = rinv != nullptr ? rinv + (size_t)q * N * N : nullptr;
-      for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-        const int c = idx % W, k = idx / W, p = x0 + c;
-        T v = (T)0;
-        if (k > 0 && p > 0)
-          v = s[k * RS + c] * (rq != nullptr ? rq[(size_t)k * N + p] : (scale / (mu1[k] + mu1[p] + muq - lambda)));
-        s[k * RS + c] = v;
-      }
-      __syncthreads();
-      dst_tile<C>(s, mem);
-    }
-  }
-  pdl_launch_next();
-  {
-    constexpr int DR = NT / W;
-    const int c = threadIdx.x % W, k0 = out.lo + threadIdx.x / W;
-    T* dst = base + (size_t)k0 * row_stride + c;
-    const T* src = s + k0 * RS + c;
-#pragma unroll 8
-    for (int k = k0; k < out.hi; k += DR, dst += DR * row_stride, src += DR * RS) *dst = *src;
-  }
-}
-
-// ------------------------------------------- TMA-fed strided passes (float32)
-// Persistent blocks walk over [N x 32] tiles of the padded float grid.  One
-// thread issues a TMA tensor load of the next tile into the other shared
-// buffer (completion counted on an mbarrier) while all threads transform the
-// current tile; the finished tile goes back by a TMA tensor store.  Every
-// wait is bounded: on timeout the block records DEVERR_TIMEOUT and returns.
+// ------------------------------------------------ asynchronous bulk copies
 constexpr int TMA_W = 32;
 // a poll of an incomplete mbarrier takes about 4 us on GB300, so 2^18 polls give up
 // after about a second (a tile load completes in microseconds)
 constexpr long TMA_WAIT_CAP = 1L << 18;
-// resident blocks per SM: three (shared memory allows three at N = 256); at
-// 80 registers neither pass spills as long as the plain pass runs its single
-// transform inside the runtime-bounded loop (the compile-time bound of one
-// lets the compiler schedule it into spills)
-template <bool SOLVE>
-constexpr int tma_blocks() {
-  return 3;
-}
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -722,6 +611,181 @@ __device__ __forceinline__ void tma_commit() { asm volatile("cp.async.bulk.commi
 __device__ __forceinline__ void tma_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// bulk copies of contiguous bytes (multiples of 16, both addresses aligned
+// to 16): completion on an mbarrier, or in the thread's bulk group
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(smem_addr(bar))
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_addr(src)), "r"(bytes)
+               : "memory");
+}
+// bounded wait of a whole phase; false when it gave up
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  for (long it = 0; it < TMA_WAIT_CAP; ++it)
+    if (mbar_try_wait(bar, parity)) return true;
+  return false;
+}
+
+// --------------------------------------------------- strided (y / z) passes
+// Tile rows = transform index k (stride row_stride), columns x0..x0+W-1 of
+// plane q = blockIdx.y + qoff; rows outside `in` are zero and not read, rows
+// outside `out` are not written.  SOLVE = forward DST, spectral multiply,
+// inverse DST.  A row of a tile is 256 (float64) or 128 (float32) contiguous
+// bytes (N >= 32).  Float64 rows move by one bulk copy of one thread each way:
+// element copies with their addresses were 8 of 146 instructions per point.
+// Float32 rows move by 16-byte asynchronous copies and vector stores (bulk
+// copies of 128 bytes were slower: 393 against 286 us for the 512^3 y pass
+// with element copies).
+template <typename T, int N>
+struct StridedCfg : Tile<T, N, WSel<T, N>::W, N >= 32 ? 32 : WSel<T, N>::W + 1> {};
+
+template <typename T, int N, bool SOLVE, int DIM>
+__global__ void __launch_bounds__(NT, StridedCfg<T, N>::BLOCKS) k_strided(
+    T* __restrict__ a, size_t row_stride, size_t plane_stride, int qoff, const T* __restrict__ mu1, T lambda, T scale,
+    const T* __restrict__ tw_g, const int* __restrict__ skip, const T* __restrict__ rinv, int reps, Span in, Span out,
+    int* __restrict__ err) {
+  using C = StridedCfg<T, N>;
+  constexpr int W = C::W, RS = C::RS;
+  constexpr bool BULK = N >= 32 && sizeof(T) == 8, VEC = N >= 32 && sizeof(T) == 4;
+  constexpr uint32_t row_bytes = W * sizeof(T);
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bar;
+  T* s = reinterpret_cast<T*>(smem_raw);
+  T* mem = s + N * RS;
+  if (BULK && threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    mbar_fence_init();
+    mbar_expect_tx(&bar, (uint32_t)(in.hi - in.lo) * row_bytes);
+  }
+  load_tables<C>(mem, tw_g);
+  pdl_wait();
+  if (skip != nullptr && *skip != 0) return;
+  const int x0 = blockIdx.x * W;
+  const int q = blockIdx.y + qoff;
+  T* base = a + (size_t)q * plane_stride + x0;
+  if constexpr (BULK) {
+    __syncthreads();
+    for (int k = in.lo + threadIdx.x; k < in.hi; k += NT)
+      bulk_load(s + k * RS, base + (size_t)k * row_stride, row_bytes, &bar);
+    if (SOLVE && C::FIX && rinv != nullptr)
+      // the tile's mode factors on their way to L2 (read after the forward
+      // transform)
+      for (int k = threadIdx.x; k < 2 * N; k += NT)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(rinv + ((size_t)q * N + k / 2) * N + x0 + 16 * (k & 1)));
+    for (int i = threadIdx.x; i < in.lo * W; i += NT) s[i] = (T)0;
+    for (int i = in.hi * W + threadIdx.x; i < N * W; i += NT) s[i] = (T)0;
+    if (!mbar_wait(&bar, 0u)) {
+      // the copies of this block finish before its shared memory goes
+      if (threadIdx.x == 0 && err != nullptr) atomicOr(err, DEVERR_TIMEOUT);
+      mbar_wait(&bar, 0u);
+      return;
+    }
+  } else if constexpr (VEC) {
+    const int c = 4 * (threadIdx.x & 7), k0 = in.lo + (threadIdx.x >> 3);
+    const T* src = base + (size_t)k0 * row_stride + c;
+#pragma unroll 4
+    for (int k = k0; k < in.hi; k += NT / 8, src += NT / 8 * row_stride) copy_async16(s + k * RS + c, src);
+    for (int i = threadIdx.x; i < in.lo * W; i += NT) s[i] = (T)0;
+    for (int i = in.hi * W + threadIdx.x; i < N * W; i += NT) s[i] = (T)0;
+    copy_async_wait();
+  } else {
+    constexpr int DR = NT / W;
+    const int c = threadIdx.x % W;
+    for (int k = threadIdx.x / W; k < N; k += DR)
+      s[k * RS + c] = k >= in.lo && k < in.hi ? base[(size_t)k * row_stride + c] : (T)0;
+  }
+  __syncthreads();
+  const T muq = DIM == 3 ? mu1[q] : (T)0;
+  if constexpr (C::REG) {
+    if constexpr (SOLVE) {
+      // forward DST with the spectral divide applied to its outputs, then the
+      // inverse DST by the same (single inlined) body; mu1 is read from
+      // global memory (L1-resident, N values)
+      const int p = x0 + (int)(threadIdx.x & 31);
+      DivPost post{mu1, mu1[p] + muq - lambda, scale, p == 0, true};
+#pragma unroll 1
+      for (int rep = 0; rep < reps; ++rep) {
+        dst_tile<C>(s, mem, post);
+        post.on = false;
+      }
+    } else {
+      dst_tile<C>(s, mem);
+    }
+  } else if constexpr (SOLVE) {
+#pragma unroll 1
+    for (int rep = 0; rep < reps; ++rep) {
+      if (rep == 1) {
+        // the mode factors scale / mu_p from the table built for this lambda
+        // (same expression, so the same value), else divided here; a batch
+        // of table values is loaded together
+        constexpr int DR = NT / W, PER = (N + DR - 1) / DR, CH = batch_of(PER);
+        const int c = threadIdx.x % W, k0 = threadIdx.x / W, p = x0 + c;
+        const T* rq = rinv != nullptr ? rinv + (size_t)q * N * N + p : nullptr;
+        const T base_mu = mu1[p] + muq - lambda;
+#pragma unroll 1
+        for (int i0 = 0; i0 < PER; i0 += CH) {
+          T f[CH];
+#pragma unroll
+          for (int i = 0; i < CH; ++i) {
+            const int k = k0 + DR * (i0 + i);
+            if (k >= N) continue;
+            if (rq != nullptr)
+              f[i] = rq[(size_t)k * N];
+            else
+              f[i] = k > 0 && p > 0 ? scale / (mu1[k] + base_mu) : (T)0;
+          }
+#pragma unroll
+          for (int i = 0; i < CH; ++i) {
+            const int k = k0 + DR * (i0 + i);
+            if (k < N) s[k * RS + c] *= f[i];
+          }
+        }
+        __syncthreads();
+      }
+      dst_tile<C>(s, mem);
+    }
+  } else {
+    dst_tile<C>(s, mem);
+  }
+  pdl_launch_next();
+  if constexpr (BULK) {
+    fence_async_shared();
+    __syncthreads();
+    for (int k = out.lo + threadIdx.x; k < out.hi; k += NT)
+      bulk_store(base + (size_t)k * row_stride, s + k * RS, row_bytes);
+    tma_commit();
+    tma_wait_all();
+  } else if constexpr (VEC) {
+    const int c = 4 * (threadIdx.x & 7), k0 = out.lo + (threadIdx.x >> 3);
+    T* dst = base + (size_t)k0 * row_stride + c;
+#pragma unroll 4
+    for (int k = k0; k < out.hi; k += NT / 8, dst += NT / 8 * row_stride)
+      *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(s + k * RS + c);
+  } else {
+    constexpr int DR = NT / W;
+    const int c = threadIdx.x % W;
+    for (int k = out.lo + threadIdx.x / W; k < out.hi; k += DR) base[(size_t)k * row_stride + c] = s[k * RS + c];
+  }
+}
+
+// ------------------------------------------- TMA-fed strided passes (float32)
+// Persistent blocks walk over [N x 32] tiles of the padded float grid.  One
+// thread issues a TMA tensor load of the next tile into the other shared
+// buffer (completion counted on an mbarrier) while all threads transform the
+// current tile; the finished tile goes back by a TMA tensor store.  Every
+// wait is bounded: on timeout the block records DEVERR_TIMEOUT and returns.
+// resident blocks per SM: three (shared memory allows three at N = 256); at
+// 80 registers neither pass spills as long as the plain pass runs its single
+// transform inside the runtime-bounded loop (the compile-time bound of one
+// lets the compiler schedule it into spills)
+template <bool SOLVE>
+constexpr int tma_blocks() {
+  return 3;
+}
 
 template <int N>
 using TmaTile = Tile<float, N, TMA_W, TMA_W>;
@@ -903,7 +967,7 @@ __global__ void __launch_bounds__(NT) k_xy_fwd(float* __restrict__ a, const doub
   using C = Cfg<float, N>;
   constexpr int W = C::W, RS = C::RS, n1 = N - 1, CL = N / W;
   static_assert(W == 32 && N % W == 0 && CL <= 8, "one cluster of at most 8 blocks per plane");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   float* sA = reinterpret_cast<float*>(smem_raw);
   float* sB = sA + N * RS;
   float* mem = sB + N * RS;
@@ -966,7 +1030,7 @@ __global__ void __launch_bounds__(NT) k_xy_inv(float* __restrict__ a, bool keep,
   using C = Cfg<float, N>;
   constexpr int W = C::W, RS = C::RS, n1 = N - 1, CL = N / W;
   static_assert(W == 32 && N % W == 0 && CL <= 8, "one cluster of at most 8 blocks per plane");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   float* sA = reinterpret_cast<float*>(smem_raw);
   float* sB = sA + N * RS;
   float* mem = sB + N * RS;
@@ -1104,11 +1168,11 @@ int launch_strided3(kfbi_handle* h, int mode, bool solve, T* work, const T* mu1,
   if (solve) {
     if ((rc = prep(k_strided<T, N, true, 3>, smem))) return rc;
     e = launch_pass(h, k_strided<T, N, true, 3>, grid, smem, work, rstride, pstride, ps.planes.lo, mu1, lam, scale, tw,
-                    (const int*)h->skip, rinv, 2, ps.in, ps.out);
+                    (const int*)h->skip, rinv, 2, ps.in, ps.out, h->w.err);
   } else {
     if ((rc = prep(k_strided<T, N, false, 3>, smem))) return rc;
     e = launch_pass(h, k_strided<T, N, false, 3>, grid, smem, work, rstride, pstride, ps.planes.lo, mu1, lam, scale, tw,
-                    (const int*)h->skip, (const T*)nullptr, 1, ps.in, ps.out);
+                    (const int*)h->skip, (const T*)nullptr, 1, ps.in, ps.out, h->w.err);
   }
   return e == cudaSuccess ? KFBI_OK : launch_failed("strided pass");
 }
@@ -1254,7 +1318,7 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
                     (const int32_t*)t.line_start, tw, (const int*)h->skip, 0, 0) != cudaSuccess)
       return launch_failed("x forward pass");
     if (launch_pass(h, k_strided<T, N, true, 2>, grid, smem, work, (size_t)N, (size_t)0, 0, mu1, lam, scale, tw,
-                    (const int*)h->skip, rinv, 2, Span{0, N}, Span{0, N}) != cudaSuccess)
+                    (const int*)h->skip, rinv, 2, Span{0, N}, Span{0, N}, h->w.err) != cudaSuccess)
       return launch_failed("y solve pass");
     if (launch_pass(h, k_xinv<T, N, 2>, grid, smem, work, sa.keep || sa.out_user == nullptr, sa.out_user,
                     (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32, 0, 0) != cudaSuccess)
@@ -1328,7 +1392,7 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
       const T* rinv = mode_factors<T, N>(h, lambda, (double)scale);
       if ((rc = prep(k_strided<T, N, true, 2>, smem))) return rc;
       k_strided<T, N, true, 2><<<grid, NT, smem, st>>>(work, N, 0, 0, mu1, lam, scale, tw, nullptr, rinv, 2, Span{0, N},
-                                                       Span{0, N});
+                                                       Span{0, N}, h->w.err);
     } else {
       if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
       k_xinv<T, N, 2><<<grid, NT, smem, st>>>(work, true, nullptr, nullptr, 1.0, 0.0, tw, nullptr, nullptr, 0, 0);
@@ -1355,7 +1419,7 @@ __global__ void __launch_bounds__(NT) k_strided_coupled(T* __restrict__ a, T* __
                                                         const int* __restrict__ skip, Span in, Span out) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   T* sa = reinterpret_cast<T*>(smem_raw);
   T* sb = sa + N * RS;
   T* mem = sb + N * RS;
@@ -1681,6 +1745,31 @@ __device__ __forceinline__ void dct_tile(typename C::T* s, const typename C::T* 
   }
 }
 
+// The W x-lines y0 .. y0 + W - 1 (zero beyond y = N) of a plane of the
+// Neumann layout to the tile s[x][line], mapped by f; a line's loads are
+// issued together (as in fill_lines).
+template <typename C, typename S, typename F>
+__device__ __forceinline__ void fill_lines_n(typename C::T* s, const S* __restrict__ src, int y0, const F& f) {
+  constexpr int N = C::N, W = C::W, RS = C::RS, P = N + 1;
+  constexpr int LW = N < 32 ? N : 32, PER = N / LW, CH = batch_of(PER);
+  const int lane = threadIdx.x % LW;
+#pragma unroll 1
+  for (int c = threadIdx.x / LW; c < W; c += NT / LW) {
+    const bool on = y0 + c <= N;
+    const S* row = src + (size_t)(y0 + c) * P;
+    const S last = on && lane == 0 ? __ldg(&row[N]) : (S)0;
+#pragma unroll
+    for (int i0 = 0; i0 < PER; i0 += CH) {
+      S v[CH];
+#pragma unroll
+      for (int i = 0; i < CH; ++i) v[i] = on ? __ldg(&row[lane + LW * (i0 + i)]) : (S)0;
+#pragma unroll
+      for (int i = 0; i < CH; ++i) s[(lane + LW * (i0 + i)) * RS + c] = f(v[i]);
+    }
+    if (lane == 0) s[N * RS + c] = f(last);
+  }
+}
+
 // x forward on the Neumann layout: W lines y0..y0+W-1 (y <= N) of plane z,
 // r = alpha*src + corrections assembled while loading.  The irregular nodes
 // (all interior) are listed per interior x-line in the interior numbering.
@@ -1692,7 +1781,7 @@ __global__ void __launch_bounds__(NT) k_nxfwd(T* __restrict__ a, const double* _
                                               const int* __restrict__ skip) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, P = N + 1, n1 = N - 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
   T* tot = s + P * RS;
   T* tw = tot + C::G * W;
@@ -1705,14 +1794,13 @@ __global__ void __launch_bounds__(NT) k_nxfwd(T* __restrict__ a, const double* _
   const int y0 = blockIdx.x * W;
   const int z = DIM == 3 ? blockIdx.y : 0;
   const size_t plane = (size_t)z * P * P;
-  for (int idx = threadIdx.x; idx < P * W; idx += NT) {
-    const int x = idx % P, c = idx / P, y = y0 + c;
-    T v = (T)0;
-    if (y <= N) {
-      if (src != nullptr) v = (T)alpha * to_T<T>(src[plane + (size_t)y * P + x]);
-      else if (src32 != nullptr) v = (T)src32[plane + (size_t)y * P + x];
-    }
-    s[x * RS + c] = v;
+  if (src != nullptr) {
+    const T a_t = (T)alpha;
+    fill_lines_n<C>(s, src + plane, y0, [&](double v) { return a_t * to_T<T>(v); });
+  } else if (src32 != nullptr) {
+    fill_lines_n<C>(s, src32 + plane, y0, [&](float v) { return (T)v; });
+  } else {
+    for (int idx = threadIdx.x; idx < P * W; idx += NT) s[(idx % P) * RS + idx / P] = (T)0;
   }
   __syncthreads();
   if (corr != nullptr) {
@@ -1744,7 +1832,7 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
                                               const float* __restrict__ aux32) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, P = N + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
   T* tot = s + P * RS;
   T* tw = tot + C::G * W;
@@ -1764,19 +1852,30 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
   copy_async_wait();
   __syncthreads();
   dct_tile<C>(s, tw, sinv, tot, x1);
-  for (int idx = threadIdx.x; idx < P * W; idx += NT) {
-    const int x = idx % P, c = idx / P, y = y0 + c;
-    if (y > N) continue;
-    const size_t o = plane + (size_t)y * P + x;
-    const T v = s[x * RS + c];
+  constexpr int LW = N < 32 ? N : 32, PER = N / LW, CH = batch_of(PER);
+  const int lane = threadIdx.x % LW;
+  const T b_t = (T)beta;
+  auto put = [&](size_t o, T v, double w) {
     if (keep) a[o] = v;
     if (out != nullptr) {
-      const double bv = to_double((T)beta * v);
-      if (aux32 != nullptr)
-        out[o] = bv + ffl::widen(aux32[o]);
-      else
-        out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
+      const double bv = to_double(b_t * v);
+      out[o] = aux32 != nullptr ? bv + w : aux != nullptr ? fma(gamma, w, bv) : bv;
     }
+  };
+  auto other = [&](size_t o) { return aux32 != nullptr ? ffl::widen(aux32[o]) : aux != nullptr ? aux[o] : 0.0; };
+#pragma unroll 1
+  for (int c = threadIdx.x / LW; c < W; c += NT / LW) {
+    if (y0 + c > N) continue;
+    const size_t o = plane + (size_t)(y0 + c) * P + lane;
+#pragma unroll
+    for (int i0 = 0; i0 < PER; i0 += CH) {
+      double w[CH];
+#pragma unroll
+      for (int i = 0; i < CH; ++i) w[i] = other(o + LW * (i0 + i));
+#pragma unroll
+      for (int i = 0; i < CH; ++i) put(o + LW * (i0 + i), s[(lane + LW * (i0 + i)) * RS + c], w[i]);
+    }
+    if (lane == 0) put(o + N, s[N * RS + c], other(o + N));
   }
 }
 
@@ -1790,7 +1889,7 @@ __global__ void __launch_bounds__(NT) k_nstrided(T* __restrict__ a, size_t row_s
                                                  const T* __restrict__ rinv = nullptr) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, P = N + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
   T* tot = s + P * RS;
   T* tw = tot + C::G * W;

@@ -358,12 +358,13 @@ KFBI_HD void dft_first(ll* xr, ll* xi, const cfx* sp) {
 // 1022).  Exponents below 64 count as 64 (values below 2^-959 then have fewer
 // bits).  A column that holds an infinity or NaN is transformed to NaN
 // throughout, as in float64.
+constexpr double HUGE_STEP = 0x1p512;
 struct Scale {
   int in;          // shift of a 63-bit significand of the largest exponent, plus its exponent field
   int sh;          // early - late
   ll half;         // rounding of the product that is shifted by sh
   double out, oc;  // 2^(-k-1) (the integers are twice the outputs) and (2^84 + 2^63 + 2^52) 2^(-k-1)
-  double big;      // 2^(-k-1) is out * big (big = 1 unless oc would overflow)
+  bool huge;       // both are smaller by HUGE_STEP (oc would overflow): the outputs need it back
 };
 KFBI_HD int bit_length(uint32_t v) {
 #ifdef __CUDA_ARCH__
@@ -388,11 +389,10 @@ KFBI_HD Scale scale_of(int emax, uint32_t asum) {
   s.in = e + 63 - early;
   s.sh = early - late;
   s.half = (1LL << 29) + ((1LL << s.sh) >> 1 << 30);
-  const bool huge = e > 1900;
-  const int eo = e - late - (huge ? 512 : 0);  // biased exponent of 2^(-k-1) (over big)
-  s.out = double_of((ll)eo << 52);
+  s.huge = e > 1900;
+  const int eo = e - late - (s.huge ? 512 : 0);  // biased exponent of 2^(-k-1)
+  s.out = double_of(emax == 0x7ff ? 0x7ff8000000000000LL : (ll)eo << 52);
   s.oc = s.out * double_of(0x4530000080100000LL);  // 2^84 + 2^63 + 2^52
-  s.big = emax == 0x7ff ? double_of(0x7ff8000000000000LL) : huge ? double_of((ll)(1023 + 512) << 52) : 1.0;
   return s;
 }
 // x as an integer at the column's scale, on its bits: the significand
@@ -415,7 +415,7 @@ KFBI_HD double from_fix(ll n, const Scale& s) {
   const double l = double_of(make_ll(0x43300000, (uint32_t)lo_of(n)));
   // (nested differently, the sum would not be exact before its last addition)
   const double t = fma(h, s.out, -s.oc);
-  return fma(l, s.out, t) * s.big;
+  return fma(l, s.out, t);
 }
 
 // ------------------------------------------------------------ tile phases
@@ -443,20 +443,18 @@ struct State {
 };
 
 // phase 0: the thread's row pairs of column c to registers, its largest
-// exponent field to mx[a][c]; pre(j, v) maps the row values (the spectral
-// multiply of a solve: here the registers hold nothing else, and its loads
-// are all in flight at once).  Thread 0 of the column holds row N/2 (its own
+// exponent field to mx[a][c].  Thread 0 of the column holds row N/2 (its own
 // mirror image) in place of the pair of row 0.
-template <class G, class Pre>
-KFBI_HD void phase_0(State<G>& st, const double* s, int* mx, int a, int c, const Pre& pre) {
+template <class G>
+KFBI_HD void phase_0(State<G>& st, const double* s, int* mx, int a, int c) {
   constexpr int N = G::N, RS = G::RS, T = G::T, P = G::P, W = G::W;
   uint32_t m = 0;
 #pragma unroll
   for (int i = 0; i < P; ++i) {
     const int j = a + T * i;
     const int ja = j == 0 ? N / 2 : j, jb = j == 0 ? N / 2 : N - j;
-    st.xa[i] = pre(ja, s[ja * RS + c]);
-    st.xb[i] = pre(jb, s[jb * RS + c]);
+    st.xa[i] = s[ja * RS + c];
+    st.xb[i] = s[jb * RS + c];
   }
 #pragma unroll
   for (int i = 0; i < P; ++i) {
@@ -661,9 +659,12 @@ KFBI_HD void phase_e2(const State<G>& st, ll* s, const ll* tot, int a, int c) {
   }
 }
 
-struct Identity {
-  KFBI_HD double operator()(int, double v) const { return v; }
-};
+// phase F (columns with huge values only): the outputs' missing factor
+template <class G>
+KFBI_HD void phase_f(const State<G>& st, double* s, int a, int c) {
+  if (st.sc.huge)
+    for (int j = a; j < G::N; j += G::T) s[j * G::RS + c] *= HUGE_STEP;
+}
 
 // words of shared memory (8 bytes each) besides the tile: split twiddles and
 // level twiddles (N/2 entries of 2 words each), sines (N/2), exponent maxima
@@ -694,8 +695,8 @@ __device__ __forceinline__ void load_tables(ll* mem, const double* tw_g) {
 // The whole transform of the tile s[N][RS] (rows 1..N-1 in and out; row 0
 // becomes 0) by 256 threads; mem: the tables and scratch.  Ends with a
 // barrier.
-template <class G, class Pre = Identity>
-__device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem, const Pre& pre = Pre()) {
+template <class G>
+__device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem) {
   constexpr int N = G::N;
   const int a = threadIdx.x >> 5, c = threadIdx.x & 31;
   ll* s = reinterpret_cast<ll*>(sd);
@@ -706,7 +707,7 @@ __device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem, const Pre& pr
   ll* tot = mem + 2 * N + N / 2 + 256;
   State<G> st;
   c2* ex = reinterpret_cast<c2*>(s);
-  phase_0<G>(st, sd, mx, a, c, pre);
+  phase_0<G>(st, sd, mx, a, c);
   __syncthreads();
   phase_s<G>(st, mx, sm, a, c);
   __syncthreads();
@@ -723,7 +724,10 @@ __device__ __forceinline__ void dst1_tile_fix(double* sd, ll* mem, const Pre& pr
   phase_e1<G>(st, s, tot, a, c);
   __syncthreads();
   phase_e2<G>(st, s, tot, a, c);
-  __syncthreads();
+  if (__syncthreads_or(st.sc.huge)) {
+    phase_f<G>(st, sd, a, c);
+    __syncthreads();
+  }
 }
 #endif
 

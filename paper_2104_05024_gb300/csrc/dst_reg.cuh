@@ -318,24 +318,32 @@ KFBI_HD void phase_c(State<G>& st, const cf2* ex, int a, int c) {
   }
 }
 
-// Y_k from A = Z_k, B = Z_{L-k}, w = e^{2 pi i k/N}: I_k to row 2k (even
-// output), R_k to row 2k+1 (scan input); post(j, value) maps an even output
+// Both split values of the pair A = Z_k, B = Z_{L-k} (w = e^{2 pi i k/N}; the
+// partner's twiddle is -conj(w), so one complex product serves both, 14
+// operations for four outputs against 20): I_k to row 2k (even output), R_k
+// to row 2k+1 (scan input), likewise for L-k when `both`; post(j, value) maps
+// an even output
 template <class G, class Post>
 KFBI_HD void split_store(float* s, const cf2* tw2, int k, float Ar, float Ai, float Br, float Bi, int c,
-                         const Post& post) {
-  constexpr int RS = G::RS;
+                         const Post& post, bool both) {
+  constexpr int RS = G::RS, L = G::L;
   const cf2 w = tw2[2 * k];
+  const float wx = 0.5f * w.x, wy = 0.5f * w.y;
   const float Sr = Ar + Br, Si = Ai - Bi, Dr = Ar - Br, Di = Ai + Bi;
-  const float Yr = 0.5f * (Sr + w.x * Di + w.y * Dr);
-  const float Yi = 0.5f * (Si - w.x * Dr + w.y * Di);
-  s[(2 * k) * RS + c] = post(2 * k, Yi);
-  s[(2 * k + 1) * RS + c] = Yr;
+  const float tr = wx * Di + wy * Dr, ti = wy * Di - wx * Dr;
+  s[(2 * k) * RS + c] = post(2 * k, 0.5f * Si + ti);
+  s[(2 * k + 1) * RS + c] = 0.5f * Sr + tr;
+  if (both) {
+    const int kk = L - k;
+    s[(2 * kk) * RS + c] = post(2 * kk, ti - 0.5f * Si);
+    s[(2 * kk + 1) * RS + c] = 0.5f * Sr - tr;
+  }
 }
 
 // phase D: real-DFT split of the owned pairs (after a barrier), writes rows
 template <class G, class Post>
 KFBI_HD void phase_d(const State<G>& st, float* s, const cf2* tw2, int a, int c, const Post& post) {
-  constexpr int T = G::T, P = G::P, L = G::L, RS = G::RS;
+  constexpr int T = G::T, P = G::P, RS = G::RS;
 #pragma unroll
   for (int gi = 0; gi < G::GPT; ++gi) {
     const int g = a + T * gi;
@@ -347,32 +355,22 @@ KFBI_HD void phase_d(const State<G>& st, float* s, const cf2* tw2, int a, int c,
       s[c] = 0.0f;
       s[RS + c] = 0.5f * (st.Ar[gi][0] + st.Ai[gi][0]);
 #pragma unroll
-      for (int k2 = 1; k2 <= 4; ++k2) {
-        const int k = P * k2, kk = L - k;
-        split_store<G>(s, tw2, k, st.Ar[gi][k2], st.Ai[gi][k2], st.Ar[gi][(8 - k2) & 7], st.Ai[gi][(8 - k2) & 7], c,
-                       post);
-        if (kk != k)
-          split_store<G>(s, tw2, kk, st.Ar[gi][(8 - k2) & 7], st.Ai[gi][(8 - k2) & 7], st.Ar[gi][k2], st.Ai[gi][k2],
-                         c, post);
-      }
+      for (int k2 = 1; k2 <= 4; ++k2)
+        split_store<G>(s, tw2, P * k2, st.Ar[gi][k2], st.Ai[gi][k2], st.Ar[gi][8 - k2], st.Ai[gi][8 - k2], c, post,
+                       k2 < 4);
       // k1 = P/2: k = P/2 + P k2 pairs with P/2 + P (7 - k2)
       if (P > 1) {
 #pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) {
-          const int k = kB + P * k2, kk = L - k;
-          split_store<G>(s, tw2, k, st.Br[gi][k2], st.Bi[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c, post);
-          split_store<G>(s, tw2, kk, st.Br[gi][7 - k2], st.Bi[gi][7 - k2], st.Br[gi][k2], st.Bi[gi][k2], c, post);
-        }
+        for (int k2 = 0; k2 < 4; ++k2)
+          split_store<G>(s, tw2, kB + P * k2, st.Br[gi][k2], st.Bi[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c,
+                         post, true);
       }
     } else {
       // k = kA + P k2 pairs with kB + P (7 - k2)
 #pragma unroll
-      for (int k2 = 0; k2 < 8; ++k2) {
-        const int k = kA + P * k2;
-        split_store<G>(s, tw2, k, st.Ar[gi][k2], st.Ai[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c, post);
-        const int kk = kB + P * k2;
-        split_store<G>(s, tw2, kk, st.Br[gi][k2], st.Bi[gi][k2], st.Ar[gi][7 - k2], st.Ai[gi][7 - k2], c, post);
-      }
+      for (int k2 = 0; k2 < 8; ++k2)
+        split_store<G>(s, tw2, kA + P * k2, st.Ar[gi][k2], st.Ai[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c,
+                       post, true);
     }
   }
 }
@@ -453,24 +451,29 @@ KFBI_HD void phase_x1(const float* part, float* x1v, int a, int c) {
   x1v[c] = v;
 }
 
-// Y_k from A = Z_k, B = Z_{L-k}: Re Y_k = X_{2k} to row 2k, Im Y_k (scan
-// input) to row 2k+1
+// the cosine split of the pair: Re Y_k = X_{2k} to row 2k, Im Y_k (scan input)
+// to row 2k+1, likewise for L-k
 template <class G, class Post>
 KFBI_HD void split_store_cos(float* s, const cf2* tw2, int k, float Ar, float Ai, float Br, float Bi, int c,
-                             const Post& post) {
-  constexpr int RS = G::RS;
+                             const Post& post, bool both) {
+  constexpr int RS = G::RS, L = G::L;
   const cf2 w = tw2[2 * k];
+  const float wx = 0.5f * w.x, wy = 0.5f * w.y;
   const float Sr = Ar + Br, Si = Ai - Bi, Dr = Ar - Br, Di = Ai + Bi;
-  const float Yr = 0.5f * (Sr + w.x * Di + w.y * Dr);
-  const float Yi = 0.5f * (Si - w.x * Dr + w.y * Di);
-  s[(2 * k) * RS + c] = post(2 * k, Yr);
-  s[(2 * k + 1) * RS + c] = Yi;
+  const float tr = wx * Di + wy * Dr, ti = wy * Di - wx * Dr;
+  s[(2 * k) * RS + c] = post(2 * k, 0.5f * Sr + tr);
+  s[(2 * k + 1) * RS + c] = 0.5f * Si + ti;
+  if (both) {
+    const int kk = L - k;
+    s[(2 * kk) * RS + c] = post(2 * kk, 0.5f * Sr - tr);
+    s[(2 * kk + 1) * RS + c] = ti - 0.5f * Si;
+  }
 }
 
 // phase D (cosine): real-DFT split of the owned pairs; X_0, X_N from Z_0
 template <class G, class Post>
 KFBI_HD void phase_d_cos(const State<G>& st, float* s, const cf2* tw2, int a, int c, const Post& post) {
-  constexpr int N = G::N, T = G::T, P = G::P, L = G::L, RS = G::RS;
+  constexpr int N = G::N, T = G::T, P = G::P, RS = G::RS;
 #pragma unroll
   for (int gi = 0; gi < G::GPT; ++gi) {
     const int g = a + T * gi;
@@ -482,34 +485,22 @@ KFBI_HD void phase_d_cos(const State<G>& st, float* s, const cf2* tw2, int a, in
       s[N * RS + c] = post(N, st.Ar[gi][0] - st.Ai[gi][0]);
       s[RS + c] = 0.0f;
 #pragma unroll
-      for (int k2 = 1; k2 <= 4; ++k2) {
-        const int k = P * k2, kk = L - k;
-        split_store_cos<G>(s, tw2, k, st.Ar[gi][k2], st.Ai[gi][k2], st.Ar[gi][(8 - k2) & 7],
-                           st.Ai[gi][(8 - k2) & 7], c, post);
-        if (kk != k)
-          split_store_cos<G>(s, tw2, kk, st.Ar[gi][(8 - k2) & 7], st.Ai[gi][(8 - k2) & 7], st.Ar[gi][k2],
-                             st.Ai[gi][k2], c, post);
-      }
+      for (int k2 = 1; k2 <= 4; ++k2)
+        split_store_cos<G>(s, tw2, P * k2, st.Ar[gi][k2], st.Ai[gi][k2], st.Ar[gi][8 - k2], st.Ai[gi][8 - k2], c, post,
+                       k2 < 4);
+      // k1 = P/2: k = P/2 + P k2 pairs with P/2 + P (7 - k2)
       if (P > 1) {
 #pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) {
-          const int k = kB + P * k2, kk = L - k;
-          split_store_cos<G>(s, tw2, k, st.Br[gi][k2], st.Bi[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c,
-                             post);
-          split_store_cos<G>(s, tw2, kk, st.Br[gi][7 - k2], st.Bi[gi][7 - k2], st.Br[gi][k2], st.Bi[gi][k2], c,
-                             post);
-        }
+        for (int k2 = 0; k2 < 4; ++k2)
+          split_store_cos<G>(s, tw2, kB + P * k2, st.Br[gi][k2], st.Bi[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c,
+                         post, true);
       }
     } else {
+      // k = kA + P k2 pairs with kB + P (7 - k2)
 #pragma unroll
-      for (int k2 = 0; k2 < 8; ++k2) {
-        const int k = kA + P * k2;
-        split_store_cos<G>(s, tw2, k, st.Ar[gi][k2], st.Ai[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c,
-                           post);
-        const int kk = kB + P * k2;
-        split_store_cos<G>(s, tw2, kk, st.Br[gi][k2], st.Bi[gi][k2], st.Ar[gi][7 - k2], st.Ai[gi][7 - k2], c,
-                           post);
-      }
+      for (int k2 = 0; k2 < 8; ++k2)
+        split_store_cos<G>(s, tw2, kA + P * k2, st.Ar[gi][k2], st.Ai[gi][k2], st.Br[gi][7 - k2], st.Bi[gi][7 - k2], c,
+                       post, true);
     }
   }
 }

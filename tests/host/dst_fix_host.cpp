@@ -32,7 +32,7 @@ int run() {
   std::vector<State<G>> st(256);
   ll* si = reinterpret_cast<ll*>(s.data());
   c2* ex = reinterpret_cast<c2*>(s.data());
-  for (int t = 0; t < 256; ++t) phase_0<G>(st[t], s.data(), mx.data(), t >> 5, t & 31, Identity());
+  for (int t = 0; t < 256; ++t) phase_0<G>(st[t], s.data(), mx.data(), t >> 5, t & 31);
   for (int t = 0; t < 256; ++t) phase_s<G>(st[t], mx.data(), sm.data(), t >> 5, t & 31);
   for (int t = 0; t < 256; ++t) phase_1<G>(st[t], si, sm.data(), sinv.data(), t >> 5, t & 31);
   for (int t = 0; t < 256; ++t) phase_a1<G>(st[t], si, sp.data(), lv.data(), t >> 5, t & 31);
@@ -41,6 +41,7 @@ int run() {
   for (int t = 0; t < 256; ++t) phase_d<G>(st[t], si, sp.data(), t >> 5, t & 31);
   for (int t = 0; t < 256; ++t) phase_e1<G>(st[t], si, tot.data(), t >> 5, t & 31);
   for (int t = 0; t < 256; ++t) phase_e2<G>(st[t], si, tot.data(), t >> 5, t & 31);
+  for (int t = 0; t < 256; ++t) phase_f<G>(st[t], s.data(), t >> 5, t & 31);
   for (int c = 0; c < 32; ++c)
     for (int j = 1; j < N; ++j) x[(size_t)c * (N - 1) + j - 1] = s[(size_t)j * RS + c];
   std::fwrite(x.data(), sizeof(double), x.size(), stdout);

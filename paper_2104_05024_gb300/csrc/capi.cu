@@ -34,7 +34,6 @@ int small_g(int m);
 int small_hcol(int m);
 int small_nrm2(int m);
 int small_y(int m);
-int arnoldi_add(kfbi_handle* h, double* small, int m, int n);
 int launch_init_arnoldi(kfbi_handle* h, double* small, int m);
 
 namespace {
@@ -403,6 +402,8 @@ struct SkipScope {
   ~SkipScope() { h->skip = nullptr; }
 };
 
+constexpr uint64_t ARN_PENDING = 0x7ff4000000000001ull;  // a NaN no kernel writes
+
 int arnoldi_iteration(kfbi_handle* h, int prec, double lambda, int j, double gnorm, double tol) {
   const int M = h->nk, m = h->opts.restart;
   double* V = h->w.vecs;
@@ -410,11 +411,34 @@ int arnoldi_iteration(kfbi_handle* h, int prec, double lambda, int j, double gno
   {
     SkipScope scope(h, h->w.stop);
     if ((rc = apply_A(h, prec, lambda, V + (size_t)j * M, h->w.tmp, 1.0, nullptr))) return rc;
-    if ((rc = arnoldi_step(h, V, M, h->w.tmp, j, m, gnorm, tol))) return rc;
+    // the slot's decision word reads "pending" until the step's kernel writes
+    // it (an iteration that the stop flag skips never does, and is never
+    // waited for)
+    double* slot = h->w.host_small + 128 + 2 * j;
+    reinterpret_cast<volatile uint64_t*>(slot)[1] = ARN_PENDING;
+    std::atomic_thread_fence(std::memory_order_seq_cst);
+    if ((rc = arnoldi_step(h, V, M, h->w.tmp, j, m, gnorm, tol, slot))) return rc;
   }
-  KFBI_CUDA(cudaMemcpyAsync(h->w.host_small + 128 + 2 * j, h->w.small + small_res(m), 2 * sizeof(double),
-                            cudaMemcpyDeviceToHost, h->stream));
-  KFBI_CUDA(cudaEventRecord(h->arn_ev[j & 1], h->stream));
+  return KFBI_OK;
+}
+
+// waits for iteration j's residual estimate and stop decision in its pinned
+// slot; the stream is queried now and then, so that a failure on the device
+// ends the wait
+int arnoldi_result(kfbi_handle* h, int j, double* res, bool* stop) {
+  volatile uint64_t* word = reinterpret_cast<volatile uint64_t*>(h->w.host_small + 128 + 2 * j) + 1;
+  for (unsigned polls = 1; *word == ARN_PENDING; ++polls) {
+    if (polls % 4096 != 0) continue;
+    const cudaError_t e = cudaStreamQuery(h->stream);
+    if (e == cudaErrorNotReady) continue;
+    if (e == cudaSuccess && *word != ARN_PENDING) break;
+    set_error("Arnoldi step did not report: %s", cudaGetErrorString(e));
+    return KFBI_ERR_CUDA;
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  const volatile double* slot = h->w.host_small + 128 + 2 * j;
+  *res = slot[0];
+  *stop = slot[1] != 0.0;
   return KFBI_OK;
 }
 
@@ -492,9 +516,9 @@ int gmres(kfbi_handle* h, int prec, double lambda, const double* g, double* psi,
     for (int j = 0; j < m; ++j) {
       const bool ahead = j + 1 < m && it + 2 <= max_iter;
       if (ahead && (rc = arnoldi_iteration(h, prec, lambda, j + 1, gnorm, tol))) return rc;
-      KFBI_CUDA(cudaEventSynchronize(h->arn_ev[j & 1]));
-      const double res = h->w.host_small[128 + 2 * j];
-      const bool stop = h->w.host_small[128 + 2 * j + 1] != 0.0;
+      double res;
+      bool stop;
+      if ((rc = arnoldi_result(h, j, &res, &stop))) return rc;
       ++it;
       rel = res / gnorm;
       jd = j + 1;
@@ -883,11 +907,6 @@ static int create_impl(const kfbi_geometry* geom, const kfbi_grid* grid, double 
     set_error("cudaMemset failed");
     return fail(KFBI_ERR_CUDA);
   }
-  for (cudaEvent_t& e : h->arn_ev)
-    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-      set_error("cudaEventCreate failed");
-      return fail(KFBI_ERR_CUDA);
-    }
   if ((rc = setup_build(h, geom))) return fail(rc);
   const int m = opts->restart;
   // Krylov vectors, densities and their history: M entries, 2M for the
@@ -970,8 +989,6 @@ void kfbi_destroy(kfbi_handle* h) {
   else cudaDeviceSynchronize();
   for (void* p : h->allocations) cudaFree(p);
   if (h->w.host_small) cudaFreeHost(h->w.host_small);
-  for (cudaEvent_t e : h->arn_ev)
-    if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : h->step_events) cudaEventDestroy(e);
   if (h->w.step_sq) cudaFree(h->w.step_sq);
   delete h;

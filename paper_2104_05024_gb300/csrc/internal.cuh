@@ -293,7 +293,6 @@ struct kfbi_handle {
   // device flag handed to the launches of a Krylov iteration enqueued ahead
   // of the host's convergence test (nullptr otherwise)
   const int* skip = nullptr;
-  cudaEvent_t arn_ev[2] = {nullptr, nullptr};  // per-iteration completion events
   int step_cap = 0;                            // Strang steps w.step_sq holds
   std::vector<cudaEvent_t> step_events;        // phase boundaries of timed Strang steps
 };
@@ -412,8 +411,7 @@ int vec_update(kfbi_handle* h, double* w, const double* V, int nvec, int ld, con
 int vec_axpby(kfbi_handle* h, double* y, double a, const double* x, double b, int n);
 int vec_scale_by_norm(kfbi_handle* h, double* v, const double* w, const double* norm_dev, int n);
 int vec_copy(kfbi_handle* h, double* dst, const double* src, int n);
-int arnoldi_givens(kfbi_handle* h, double* small, int j, int ldh);
-int arnoldi_step(kfbi_handle* h, double* V, int ld, double* wv, int j, int m, double gnorm, double tol);
+int arnoldi_step(kfbi_handle* h, double* V, int ld, double* wv, int j, int m, double gnorm, double tol, double* host);
 int arnoldi_solve(kfbi_handle* h, double* small, int k, int ldh);
 
 // mlp.cu

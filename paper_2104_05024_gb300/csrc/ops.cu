@@ -460,16 +460,11 @@ __device__ void givens_column(double* s, int m, int j) {
   s[L.res()] = fabs(g[j + 1]);
 }
 
-__global__ void k_givens(double* s, int m, int j) { givens_column(s, m, j); }
 
-// ---------------------------------------------- fused Arnoldi step (CGS2)
-// One Krylov step after w = A v_j takes four launches: h = V^T w; w -= V h
-// with y = V^T w; w -= V y with ||w||^2, H(:, j) = h + y and the Givens
-// update; v_{j+1} = w / ||w||.  Each thread owns a grid-stride set of rows;
-// the last block to finish (a ticket counter, reset by that block) reduces
-// the per-block partial sums in a fixed order, so results do not depend on
-// block scheduling.  skip (optional): a device flag; when set, the kernel
-// does nothing (an iteration enqueued ahead of the convergence test).
+// ------------------------------------------------- single-launch reductions
+// Each thread owns a grid-stride set of rows; the last block to finish (a
+// ticket counter, reset by that block) reduces the per-block partial sums in
+// a fixed order, so results do not depend on block scheduling.
 
 // true in every thread of the block that finishes last
 __device__ __forceinline__ bool arn_last_block(unsigned* counter) {
@@ -535,106 +530,185 @@ __device__ __forceinline__ double warp_sum8(double (&v)[ARN_CH]) {
   return t;
 }
 
-// w_i -= sum_{k < nv} cs[k] V_k[i] over a grid-stride set of rows; each
-// chunk's loads are independent, so a thread has ARN_CH of them in flight
-__device__ __forceinline__ void arn_update(double* __restrict__ w, const double* __restrict__ V, int ld, int n, int nv,
-                                           const double* cs, double* sq) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int k0 = 0; k0 < nv; k0 += ARN_CH) {
-      double x[ARN_CH];
-#pragma unroll
-      for (int u = 0; u < ARN_CH; ++u) x[u] = k0 + u < nv ? V[(size_t)(k0 + u) * ld + i] : 0.0;
-#pragma unroll
-      for (int u = 0; u < ARN_CH; ++u)
-        if (k0 + u < nv) acc += cs[k0 + u] * x[u];
-    }
-    const double wi = w[i] - acc;
-    w[i] = wi;
-    if (sq != nullptr) *sq += wi * wi;
-  }
-}
+// ------------------------------------------------- Arnoldi step (CGS2)
+// One Krylov step after w = A v_j:
+//   h = V^T w;  w1 = w - V h;  y = V^T w1, |w1|^2;  w2 = w1 - V y;
+//   H(:, j) = h + y, |w2|^2 = |w1|^2 - |y|^2 (V has orthonormal columns, and
+//   y is of rounding size unless the space is exhausted, where both vanish);
+//   v_{j+1} = w2 / |w2|;  the Givens update, the residual estimate |g_{j+1}|
+//   and the stop flag (estimate / gnorm <= tol, or not finite: the host's
+//   test, in the same float64 operations).
+// The norm by difference leaves two reductions instead of three and no
+// separate scaling pass: three launches (dots; update and dots; update,
+// scale and Givens) instead of four, 40 -> 30 us at 49 156 rows.  Up to
+// ARN_ONE rows one block does the step in one launch (32 -> 15 us at 256
+// rows).  A grid-wide barrier in one cooperative launch was no faster than
+// the chained launches (it cannot overlap its predecessor's tail).
+// The residual estimate and the stop decision go straight to pinned host
+// memory, so that no copy or event sits between two iterations' kernels.
+// skip (optional): a device flag; when set, the kernels do nothing (an
+// iteration enqueued ahead of the convergence test).
+constexpr int ARN_ONE = 2048;   // rows up to which one block takes the step
+constexpr int ARN_ONE_T = 512;  // its threads
 
-// [UPDATE: w -= sum_k coef[k] V_k;]  out[k] = V_k . w  (k < nv)
-template <bool UPDATE>
-__global__ void __launch_bounds__(256) k_arn_gs(double* __restrict__ w, const double* __restrict__ V, int ld, int n,
-                                                int nv, const double* __restrict__ coef, double* __restrict__ partial,
-                                                unsigned* __restrict__ counter, double* __restrict__ out,
-                                                const int* __restrict__ skip) {
-  pdl_wait();
-  pdl_launch_next();
-  if (skip != nullptr && *skip) return;
-  __shared__ double cs[MAX_RESTART + 2];
-  __shared__ double red[8][MAX_RESTART + 2];
+struct ArnArgs {
+  double* w;
+  double* V;
+  int ld, n, nv, m, j;
+  double* s;          // small vectors
+  double* partial;    // per-block sums
+  unsigned* counter;
+  double gnorm, tol;
+  int* stop;
+  double* host;       // pinned: residual estimate, stop decision
+  const int* skip;
+};
+
+// per-warp sums of V_k . w (k < nv) and, with NORM, of w . w (k = nv) over
+// the block's rows to red[warp][k]
+template <bool NORM>
+__device__ __forceinline__ void arn_dots(const ArnArgs& A, double (*red)[MAX_RESTART + 2]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (UPDATE) {
-    for (int k = threadIdx.x; k < nv; k += blockDim.x) cs[k] = coef[k];
-    __syncthreads();
-    arn_update(w, V, ld, n, nv, cs, nullptr);
-  }
-  // each thread reads back only the rows it updated itself
-  for (int k0 = 0; k0 < nv; k0 += ARN_CH) {
+  const int nd = A.nv + (NORM ? 1 : 0);
+  for (int k0 = 0; k0 < nd; k0 += ARN_CH) {
     double d[ARN_CH];
 #pragma unroll
     for (int u = 0; u < ARN_CH; ++u) d[u] = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      const double wi = w[i];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) {
+      const double wi = A.w[i];
+      double x[ARN_CH];
 #pragma unroll
       for (int u = 0; u < ARN_CH; ++u)
-        if (k0 + u < nv) d[u] += V[(size_t)(k0 + u) * ld + i] * wi;
+        x[u] = k0 + u < A.nv ? A.V[(size_t)(k0 + u) * A.ld + i] : NORM && k0 + u == A.nv ? wi : 0.0;
+#pragma unroll
+      for (int u = 0; u < ARN_CH; ++u)
+        if (k0 + u < nd) d[u] += x[u] * wi;
     }
     const double t = warp_sum8(d);
     const int u = lane >> 2;
-    if ((lane & 3) == 0 && k0 + u < nv) red[warp][k0 + u] = t;
+    if ((lane & 3) == 0 && k0 + u < nd) red[warp][k0 + u] = t;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < nv; k += blockDim.x) {
-    double t = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += red[q][k];
-    partial[(size_t)k * gridDim.x + blockIdx.x] = t;
-  }
-  if (!arn_last_block(counter)) return;
-  arn_reduce(partial, gridDim.x, nv, out);
-  if (threadIdx.x == 0) *counter = 0u;
 }
 
-// w -= sum_k y[k] V_k; ||w||^2; hcol += y; Givens update of column j; the
-// residual estimate |g_{j+1}| and the stop flag (estimate / gnorm <= tol, or
-// not finite: the host's test, in the same float64 operations)
-__global__ void __launch_bounds__(256) k_arn_close(double* __restrict__ w, const double* __restrict__ V, int ld, int n,
-                                                   int nv, double* __restrict__ s, int m, int j,
-                                                   double* __restrict__ partial, unsigned* __restrict__ counter,
-                                                   double gnorm, double tol, int* stop, const int* skip) {
+// w_i -= sum_k cs[k] V_k[i] over the block's rows; each chunk's loads are
+// independent, so a thread has ARN_CH of them in flight.  vn (optional)
+// receives the result times inv as well.
+__device__ __forceinline__ void arn_update(const ArnArgs& A, const double* cs, double* vn, double inv) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) {
+    double acc = 0.0;
+    for (int k0 = 0; k0 < A.nv; k0 += ARN_CH) {
+      double x[ARN_CH];
+#pragma unroll
+      for (int u = 0; u < ARN_CH; ++u) x[u] = k0 + u < A.nv ? A.V[(size_t)(k0 + u) * A.ld + i] : 0.0;
+#pragma unroll
+      for (int u = 0; u < ARN_CH; ++u)
+        if (k0 + u < A.nv) acc += cs[k0 + u] * x[u];
+    }
+    const double wi = A.w[i] - acc;
+    if (vn != nullptr)
+      vn[i] = wi * inv;
+    else
+      A.w[i] = wi;
+  }
+}
+
+// |w2| from |w1|^2 and y (every thread)
+__device__ __forceinline__ double arn_norm2(const double* y, int nv) {
+  double t = y[nv];
+  for (int k = 0; k < nv; ++k) t = fma(-y[k], y[k], t);
+  return t > 0.0 ? t : 0.0;
+}
+
+// Givens update, estimate and stop flag (one thread; hcol and nrm2 are set)
+__device__ __forceinline__ void arn_finish(const ArnArgs& A) {
+  SmallLayout L{A.m};
+  double* s = A.s;
+  givens_column(s, A.m, A.j);
+  const double rel = s[L.res()] / A.gnorm;
+  const int done = !(rel > A.tol) || !isfinite(rel);
+  *A.stop = done;
+  // the decision last: the host polls it
+  volatile double* host = A.host;
+  host[0] = s[L.res()];
+  __threadfence_system();
+  host[1] = done ? 1.0 : 0.0;
+}
+
+// [UPDATE: w -= sum_k coef[k] V_k;]  out[k] = V_k . w (k < nv), and with
+// UPDATE out[nv] = w . w
+template <bool UPDATE>
+__global__ void __launch_bounds__(256) k_arn_gs(ArnArgs A, const double* __restrict__ coef, double* __restrict__ out) {
   pdl_wait();
   pdl_launch_next();
-  if (skip != nullptr && *skip) return;
-  SmallLayout L{m};
+  if (A.skip != nullptr && *A.skip) return;
   __shared__ double cs[MAX_RESTART + 2];
-  __shared__ double ws[32];
-  for (int k = threadIdx.x; k < nv; k += blockDim.x) cs[k] = s[L.y() + k];
-  __syncthreads();
-  double sq = 0.0;
-  arn_update(w, V, ld, n, nv, cs, &sq);
-  sq = warp_sum(sq);
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = sq;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < (blockDim.x >> 5) ? ws[threadIdx.x] : 0.0;
-    t = warp_sum(t);
-    if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  __shared__ double red[8][MAX_RESTART + 2];
+  if (UPDATE) {
+    for (int k = threadIdx.x; k < A.nv; k += blockDim.x) cs[k] = coef[k];
+    __syncthreads();
+    arn_update(A, cs, nullptr, 0.0);
   }
-  if (!arn_last_block(counter)) return;
-  if (threadIdx.x < 32) arn_reduce(partial, gridDim.x, 1, s + L.nrm2());
-  for (int k = threadIdx.x; k < nv; k += blockDim.x) s[L.hcol() + k] += cs[k];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    givens_column(s, m, j);
-    const double rel = s[L.res()] / gnorm;
-    const int done = !(rel > tol) || !isfinite(rel);
-    s[L.res() + 1] = done ? 1.0 : 0.0;
-    *stop = done;
-    *counter = 0u;
+  // each thread reads back only the rows it updated itself
+  arn_dots<UPDATE>(A, red);
+  const int nd = A.nv + (UPDATE ? 1 : 0);
+  for (int k = threadIdx.x; k < nd; k += blockDim.x) {
+    double t = 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) t += red[q][k];
+    A.partial[(size_t)k * gridDim.x + blockIdx.x] = t;
   }
+  if (!arn_last_block(A.counter)) return;
+  arn_reduce(A.partial, gridDim.x, nd, out);
+  if (threadIdx.x == 0) *A.counter = 0u;
+}
+
+// v_{j+1} = (w - sum_k y[k] V_k) / |.|; the first block also closes column j
+__global__ void __launch_bounds__(256) k_arn_close(ArnArgs A) {
+  pdl_wait();
+  pdl_launch_next();
+  if (A.skip != nullptr && *A.skip) return;
+  SmallLayout L{A.m};
+  __shared__ double y[MAX_RESTART + 2];
+  for (int k = threadIdx.x; k <= A.nv; k += blockDim.x) y[k] = A.s[L.y() + k];
+  __syncthreads();
+  const double n2 = arn_norm2(y, A.nv), norm = sqrt(n2);
+  arn_update(A, y, A.V + (size_t)(A.j + 1) * A.ld, norm > 0.0 ? 1.0 / norm : 0.0);
+  if (blockIdx.x != 0) return;
+  for (int k = threadIdx.x; k < A.nv; k += blockDim.x) A.s[L.hcol() + k] += y[k];
+  if (threadIdx.x == 0) A.s[L.nrm2()] = n2;
+  __syncthreads();
+  if (threadIdx.x == 0) arn_finish(A);
+}
+
+// the whole step by one block
+__global__ void __launch_bounds__(ARN_ONE_T) k_arn_one(ArnArgs A) {
+  pdl_wait();
+  pdl_launch_next();
+  if (A.skip != nullptr && *A.skip) return;
+  __shared__ double red[ARN_ONE_T / 32][MAX_RESTART + 2];
+  __shared__ double h[MAX_RESTART + 2], y[MAX_RESTART + 2];
+  SmallLayout L{A.m};
+  auto sum = [&](double* out, int nd) {
+    for (int k = threadIdx.x; k < nd; k += ARN_ONE_T) {
+      double t = 0.0;
+#pragma unroll
+      for (int q = 0; q < ARN_ONE_T / 32; ++q) t += red[q][k];
+      out[k] = t;
+    }
+    __syncthreads();
+  };
+  arn_dots<false>(A, red);
+  sum(h, A.nv);
+  arn_update(A, h, nullptr, 0.0);
+  arn_dots<true>(A, red);
+  sum(y, A.nv + 1);
+  const double n2 = arn_norm2(y, A.nv), norm = sqrt(n2);
+  for (int k = threadIdx.x; k < A.nv; k += ARN_ONE_T) A.s[L.hcol() + k] = h[k] + y[k];
+  if (threadIdx.x == 0) A.s[L.nrm2()] = n2;
+  arn_update(A, y, A.V + (size_t)(A.j + 1) * A.ld, norm > 0.0 ? 1.0 / norm : 0.0);
+  __syncthreads();
+  if (threadIdx.x == 0) arn_finish(A);
 }
 
 // Normal equations of the density-history projection in one launch:
@@ -694,16 +768,22 @@ __global__ void __launch_bounds__(256) k_gram(const double* __restrict__ H, int 
   }
 }
 
-// y = R^{-1} g for the leading k x k block
+// y = R^{-1} g for the leading k x k block, one warp: lane l holds rows l and
+// l + 32 and takes each solved unknown out of them (a single thread's chain
+// of k^2 / 2 dependent steps took 13 us at k = 18)
 __global__ void k_backsolve(double* s, int m, int k) {
   SmallLayout L{m};
   const double* H = s + L.H();
   const double* g = s + L.g();
   double* y = s + L.y();
+  const int lane = threadIdx.x;
+  double a0 = lane < k ? g[lane] : 0.0, a1 = lane + 32 < k ? g[lane + 32] : 0.0;
   for (int i = k - 1; i >= 0; --i) {
-    double a = g[i];
-    for (int c = i + 1; c < k; ++c) a -= H[(size_t)c * (m + 1) + i] * y[c];
-    y[i] = a / H[(size_t)i * (m + 1) + i];
+    const double* col = H + (size_t)i * (m + 1);
+    const double yi = __shfl_sync(0xffffffffu, i < 32 ? a0 : a1, i & 31) / col[i];
+    if (lane == 0) y[i] = yi;
+    if (lane < i) a0 -= col[lane] * yi;
+    if (lane + 32 < i) a1 -= col[lane + 32] * yi;
   }
 }
 
@@ -711,13 +791,6 @@ __global__ void k_init_arnoldi(double* s, int m) {
   SmallLayout L{m};
   const int i = threadIdx.x;
   if (i <= m) s[L.g() + i] = i == 0 ? sqrt(s[L.nrm2()]) : 0.0;
-}
-
-__global__ void k_add_small(double* s, int m, int n) {
-  // hcol += second-pass coefficients stored right after it (CGS2)
-  SmallLayout L{m};
-  const int i = threadIdx.x;
-  if (i < n) s[L.hcol() + i] += s[L.y() + i];
 }
 
 // ------------------------------------------------------------- reaction
@@ -1421,47 +1494,36 @@ int vec_copy(kfbi_handle* h, double* dst, const double* src, int n) {
   return KFBI_OK;
 }
 
-int arnoldi_givens(kfbi_handle* h, double* small, int j, int m) {
-  k_givens<<<1, 1, 0, h->stream>>>(small, m, j);
-  KFBI_CHECK_LAUNCH();
-  return KFBI_OK;
-}
-
 int arnoldi_solve(kfbi_handle* h, double* small, int k, int m) {
-  k_backsolve<<<1, 1, 0, h->stream>>>(small, m, k);
+  k_backsolve<<<1, 32, 0, h->stream>>>(small, m, k);
   KFBI_CHECK_LAUNCH();
   return KFBI_OK;
 }
 
 // one CGS2 Arnoldi step on wv = A v_j (basis V, leading dimension ld,
-// restart m): H(:, j), the Givens update, v_{j+1}, and at small[res],
-// small[res + 1] the residual estimate and the stop flag (also written to
-// h->w.stop).  Launches carry h->skip.
-int arnoldi_step(kfbi_handle* h, double* V, int ld, double* wv, int j, int m, double gnorm, double tol) {
+// restart m): H(:, j), the Givens update, v_{j+1}; the residual estimate and
+// the stop decision in host[0], host[1] (pinned), the decision also in
+// h->w.stop.  Launches carry h->skip.
+int arnoldi_step(kfbi_handle* h, double* V, int ld, double* wv, int j, int m, double gnorm, double tol, double* host) {
   const int n = h->nk;
-  int nb = (n + 255) / 256;
-  if (nb > ARN_BLOCKS) nb = ARN_BLOCKS;
   SmallLayout L{m};
   double* s = h->w.small;
-  const int nv = j + 1;
-  const int* skip = h->skip;
+  const ArnArgs A{wv,   V,   ld,        n,    j + 1,  m, j, s, h->w.partial, h->w.counter, gnorm, tol, h->w.stop,
+                  host, h->skip};
   cudaStream_t st = h->stream;
-  if (launch_pdl(k_arn_gs<false>, dim3(nb), dim3(256), 0, st, wv, (const double*)V, ld, n, nv, (const double*)nullptr,
-                 h->w.partial, h->w.counter, s + L.hcol(), skip) != cudaSuccess ||
-      launch_pdl(k_arn_gs<true>, dim3(nb), dim3(256), 0, st, wv, (const double*)V, ld, n, nv,
-                 (const double*)(s + L.hcol()), h->w.partial, h->w.counter, s + L.y(), skip) != cudaSuccess ||
-      launch_pdl(k_arn_close, dim3(nb), dim3(256), 0, st, wv, (const double*)V, ld, n, nv, s, m, j, h->w.partial,
-                 h->w.counter, gnorm, tol, h->w.stop, skip) != cudaSuccess ||
-      launch_pdl(k_scale_norm, dim3((n + 255) / 256), dim3(256), 0, st, V + (size_t)(j + 1) * ld, (const double*)wv,
-                 (const double*)(s + L.nrm2()), n, skip) != cudaSuccess)
+  if (n <= ARN_ONE) {
+    if (launch_pdl(k_arn_one, dim3(1), dim3(ARN_ONE_T), 0, st, A) != cudaSuccess) return launch_failed("Arnoldi step");
+    KFBI_CHECK_LAUNCH();
+    return KFBI_OK;
+  }
+  int nb = (n + 255) / 256;
+  if (nb > ARN_BLOCKS) nb = ARN_BLOCKS;
+  if (launch_pdl(k_arn_gs<false>, dim3(nb), dim3(256), 0, st, A, (const double*)nullptr, s + L.hcol()) != cudaSuccess ||
+      launch_pdl(k_arn_gs<true>, dim3(nb), dim3(256), 0, st, A, (const double*)(s + L.hcol()), s + L.y()) !=
+          cudaSuccess ||
+      launch_pdl(k_arn_close, dim3(nb), dim3(256), 0, st, A) != cudaSuccess)
     return launch_failed("Arnoldi step");
-  KFBI_CHECK_LAUNCH_N(4);
-  return KFBI_OK;
-}
-
-int arnoldi_add(kfbi_handle* h, double* small, int m, int n) {
-  k_add_small<<<1, 128, 0, h->stream>>>(small, m, n);
-  KFBI_CHECK_LAUNCH();
+  KFBI_CHECK_LAUNCH_N(3);
   return KFBI_OK;
 }
 

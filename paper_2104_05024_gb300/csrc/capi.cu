@@ -282,9 +282,13 @@ int apply_A(kfbi_handle* h, int prec, double lambda, const double* psi, double* 
   const double* x;
   int rc = density_vector(h, psi, &x);
   if (rc) return rc;
-  if ((rc = launch_correction(h, x, h->w.corr))) return rc;
   SolveArgs sa;
-  sa.corr = h->w.corr;
+  if (h->grid.dim == 2 && !neumann_box(h)) {
+    sa.rows = corr_rows(h->t, x);
+  } else {
+    if ((rc = launch_correction(h, x, h->w.corr))) return rc;
+    sa.corr = h->w.corr;
+  }
   sa.lambda = lambda;
   sa.near_only = true;
   if (prec == KFBI_FP64) {

@@ -446,13 +446,44 @@ __device__ __forceinline__ void fill_lines(typename C::T* s, const S* __restrict
   }
 }
 
+// The corrections of the tile's lines y0 .. y0 + W - 1 of plane z (0 in 2-D),
+// summed values (corr) or, in 2-D, CSR rows on the density vector (rows):
+// each line's irregular nodes (distinct x, so distinct words) are shared out
+// over the NT / W threads of its column.  In 2-D rows save the gather's own
+// launch (4 us of 45); in 3-D the rows' dependent loads cost the x pass more
+// than the gather kernel takes (A psi at 256^3 150 -> 156 us).
+template <typename C, int DIM>
+__device__ __forceinline__ void add_corrections(typename C::T* s, const double* __restrict__ corr, const CorrRows& rows,
+                                                const int32_t* __restrict__ irr, const int32_t* __restrict__ line_start,
+                                                int y0, int z) {
+  using T = typename C::T;
+  constexpr int W = C::W, RS = C::RS, n1 = C::N - 1, G = NT / W;
+  const int c = threadIdx.x % W, g = threadIdx.x / W, y = y0 + c;
+  if ((corr == nullptr && (DIM == 3 || rows.x == nullptr)) || y <= 0) return;
+  const int line = DIM == 3 ? (z - 1) * n1 + (y - 1) : (y - 1);
+  const int i0 = line_start[line], i1 = line_start[line + 1];
+  for (int i = i0 + g; i < i1; i += G) {
+    const int x = irr[i] % n1 + 1;
+    double v = 0.0;
+    if (DIM == 2 && rows.x != nullptr) {
+      const int k1 = rows.ptr[i + 1];
+#pragma unroll 4
+      for (int k = rows.ptr[i]; k < k1; ++k) v += rows.w[k] * rows.x[rows.pid[k]];
+    } else {
+      v = corr[i];
+    }
+    s[x * RS + c] += (T)v;
+  }
+}
+
 // ------------------------------------------------------------- x forward
 // Tile: W consecutive lines y0..y0+W-1 of plane z; assembles
 // r = alpha*src + corrections on the fly.
 template <typename T, int N, int DIM>
 __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xfwd(T* __restrict__ a, const double* __restrict__ src, double alpha,
                                              const float* __restrict__ src32,
-                                             const double* __restrict__ corr, const int32_t* __restrict__ irr,
+                                             const double* __restrict__ corr, CorrRows rows,
+                                             const int32_t* __restrict__ irr,
                                              const int32_t* __restrict__ line_start, const T* __restrict__ tw_g,
                                              const int* __restrict__ skip, int yoff, int zoff) {
   using C = Cfg<T, N>;
@@ -476,20 +507,7 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xfwd(T* __restrict__ 
     for (int idx = threadIdx.x; idx < N * W; idx += NT) s[(idx % N) * RS + idx / N] = (T)0;
   }
   __syncthreads();
-  if (corr != nullptr) {
-    // the line's irregular nodes (distinct x, so distinct words) shared out
-    // over the NT / W threads of each column
-    constexpr int G = NT / W;
-    const int c = threadIdx.x % W, g = threadIdx.x / W, y = y0 + c;
-    if (y > 0) {
-      const int line = DIM == 3 ? (z - 1) * n1 + (y - 1) : (y - 1);
-      const int i0 = line_start[line], i1 = line_start[line + 1];
-      for (int i = i0 + g; i < i1; i += G) {
-        const int x = irr[i] % n1 + 1;
-        s[x * RS + c] += (T)corr[i];
-      }
-    }
-  }
+  add_corrections<C, DIM>(s, corr, rows, irr, line_start, y0, z);
   __syncthreads();
   dst_tile<C>(s, mem);
   pdl_launch_next();
@@ -500,31 +518,15 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xfwd(T* __restrict__ 
   }
 }
 
-// ------------------------------------------------------------- x inverse
-template <typename T, int N, int DIM>
-__global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ a, bool keep, double* __restrict__ out,
-                                             const double* __restrict__ aux, double beta, double gamma,
-                                             const T* __restrict__ tw_g, const int* __restrict__ skip,
-                                             const float* __restrict__ aux32, int yoff, int zoff) {
-  using C = Cfg<T, N>;
-  constexpr int W = C::W, RS = C::RS, n1 = N - 1;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  T* s = reinterpret_cast<T*>(smem_raw);
-  T* mem = s + N * RS;
-  load_tables<C>(mem, tw_g);
-  pdl_wait();
-  if (skip != nullptr && *skip != 0) return;
-  const int y0 = blockIdx.x * W + yoff;
-  const int z = DIM == 3 ? blockIdx.y + zoff : 0;
+// The tile's lines y0 .. y0 + W - 1 of plane z to the work grid (keep) and/or
+// to a field.
+template <typename C, int DIM>
+__device__ __forceinline__ void put_lines(const typename C::T* s, typename C::T* __restrict__ a, bool keep,
+                                          double* __restrict__ out, const double* __restrict__ aux, double beta,
+                                          double gamma, const float* __restrict__ aux32, int y0, int z) {
+  using T = typename C::T;
+  constexpr int N = C::N, W = C::W, RS = C::RS, n1 = N - 1;
   const size_t plane = (size_t)z * N * N;
-  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-    const int x = idx % N, c = idx / N;
-    copy_async(&s[x * RS + c], &a[plane + (size_t)(y0 + c) * N + x]);
-  }
-  copy_async_wait();
-  __syncthreads();
-  dst_tile<C>(s, mem);
-  pdl_launch_next();
   if (out == nullptr) {
     if (keep)
       for (int idx = threadIdx.x; idx < N * W; idx += NT) {
@@ -567,6 +569,34 @@ __global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ 
       }
     }
   }
+}
+
+// ------------------------------------------------------------- x inverse
+template <typename T, int N, int DIM>
+__global__ void __launch_bounds__(NT, Cfg<T, N>::BLOCKS) k_xinv(T* __restrict__ a, bool keep, double* __restrict__ out,
+                                             const double* __restrict__ aux, double beta, double gamma,
+                                             const T* __restrict__ tw_g, const int* __restrict__ skip,
+                                             const float* __restrict__ aux32, int yoff, int zoff) {
+  using C = Cfg<T, N>;
+  constexpr int W = C::W, RS = C::RS;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T* s = reinterpret_cast<T*>(smem_raw);
+  T* mem = s + N * RS;
+  load_tables<C>(mem, tw_g);
+  pdl_wait();
+  if (skip != nullptr && *skip != 0) return;
+  const int y0 = blockIdx.x * W + yoff;
+  const int z = DIM == 3 ? blockIdx.y + zoff : 0;
+  const size_t plane = (size_t)z * N * N;
+  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
+    const int x = idx % N, c = idx / N;
+    copy_async(&s[x * RS + c], &a[plane + (size_t)(y0 + c) * N + x]);
+  }
+  copy_async_wait();
+  __syncthreads();
+  dst_tile<C>(s, mem);
+  pdl_launch_next();
+  put_lines<C, DIM>(s, a, keep, out, aux, beta, gamma, aux32, y0, z);
 }
 
 // ------------------------------------------------ asynchronous bulk copies
@@ -937,17 +967,17 @@ constexpr size_t xy_smem_bytes() {
 // the cluster and j < 32: the transposed 32 x 32 pieces.  Warp w moves rows
 // j = w + 8 i; the distributed-shared-memory loads of four blocks are issued
 // together (16 in flight per thread) before their stores.
-template <int N>
-__device__ __forceinline__ void xy_exchange(const cg::cluster_group& cluster, float* src, float* dst, int y0) {
-  using C = Cfg<float, N>;
+template <typename T, int N>
+__device__ __forceinline__ void xy_exchange(const cg::cluster_group& cluster, T* src, T* dst, int y0) {
+  using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS, CL = N / W, R = W / (NT / 32), QB = CL < 4 ? CL : 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll 1
   for (int q0 = 0; q0 < CL; q0 += QB) {
-    float v[QB][R];
+    T v[QB][R];
 #pragma unroll
     for (int k = 0; k < QB; ++k) {
-      const float* ps = cluster.map_shared_rank(src, q0 + k);
+      const T* ps = cluster.map_shared_rank(src, q0 + k);
 #pragma unroll
       for (int i = 0; i < R; ++i) v[k][i] = ps[(y0 + warp + (NT / 32) * i) * RS + lane];
     }
@@ -999,19 +1029,11 @@ __global__ void __launch_bounds__(NT) k_xy_fwd(float* __restrict__ a, const doub
     for (int idx = threadIdx.x; idx < N * W; idx += NT) sA[(idx % N) * RS + idx / N] = 0.0f;
   }
   __syncthreads();
-  if (corr != nullptr) {
-    constexpr int G = NT / W;
-    const int c = threadIdx.x % W, g = threadIdx.x / W, y = y0 + c;
-    if (y > 0) {
-      const int line = (z - 1) * n1 + (y - 1);
-      const int i0 = line_start[line], i1 = line_start[line + 1];
-      for (int i = i0 + g; i < i1; i += G) sA[(irr[i] % n1 + 1) * RS + c] += (float)corr[i];
-    }
-  }
+  add_corrections<C, 3>(sA, corr, CorrRows{}, irr, line_start, y0, z);
   __syncthreads();
   dst_tile<C>(sA, mem);
   cluster.sync();
-  xy_exchange<N>(cluster, sA, sB, y0);
+  xy_exchange<float, N>(cluster, sA, sB, y0);
   cluster.sync();
   dst_tile<C>(sB, mem);
   const size_t plane = (size_t)z * N * N;
@@ -1050,7 +1072,7 @@ __global__ void __launch_bounds__(NT) k_xy_inv(float* __restrict__ a, bool keep,
   __syncthreads();
   dst_tile<C>(sB, mem);
   cluster.sync();
-  xy_exchange<N>(cluster, sB, sA, y0);
+  xy_exchange<float, N>(cluster, sB, sA, y0);
   cluster.sync();
   dst_tile<C>(sA, mem);
   if (out == nullptr) {
@@ -1078,20 +1100,91 @@ __global__ void __launch_bounds__(NT) k_xy_inv(float* __restrict__ a, bool keep,
   }
 }
 
+// The whole 2-D solve in one launch: a cluster of N / 32 blocks (N <= 256),
+// block r with the x lines y = 32 r .. 32 r + 31 (tile A: rows x) and then the
+// x modes 32 r .. 32 r + 31 (tile B: rows y): x DST, exchange, y DST, spectral
+// multiply, y DST, exchange, x DST, output.  A plane of this size is a few
+// blocks' work, so its time is latency: as three launches (x forward, y
+// solve, x inverse) with the grid through memory between them a float64
+// 128^2 solve took 37 us of kernel time.  The four transforms run one inlined
+// body; the values are those of the three passes.
+template <typename T, int N>
+__global__ void __launch_bounds__(NT, 1) k_solve2d(T* __restrict__ a, const double* __restrict__ src, double alpha,
+                                                   const float* __restrict__ src32, const double* __restrict__ corr,
+                                                   CorrRows rows, const int32_t* __restrict__ irr,
+                                                   const int32_t* __restrict__ line_start, const T* __restrict__ tw_g,
+                                                   const T* __restrict__ mu1, T lambda, T scale,
+                                                   const T* __restrict__ rinv, bool keep, double* __restrict__ out,
+                                                   const double* __restrict__ aux, double beta, double gamma,
+                                                   const float* __restrict__ aux32, const int* __restrict__ skip,
+                                                   int reps) {
+  using C = Cfg<T, N>;
+  constexpr int W = C::W, RS = C::RS;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T* sA = reinterpret_cast<T*>(smem_raw);
+  T* sB = sA + N * RS;
+  T* mem = sB + N * RS;
+  cg::cluster_group cluster = cg::this_cluster();
+  load_tables<C>(mem, tw_g);
+  pdl_wait();
+  // set by earlier kernels of the stream: the same for every block
+  if (skip != nullptr && *skip != 0) return;
+  pdl_launch_next();
+  const int y0 = (int)cluster.block_rank() * W;
+  if (src != nullptr) {
+    const T a_t = (T)alpha;
+    fill_lines<C, 2>(sA, src, y0, 0, [&](double v) { return a_t * to_T<T>(v); });
+  } else if (src32 != nullptr) {
+    fill_lines<C, 2>(sA, src32, y0, 0, [&](float v) { return (T)v; });
+  } else {
+    for (int idx = threadIdx.x; idx < N * W; idx += NT) sA[(idx % N) * RS + idx / N] = (T)0;
+  }
+  __syncthreads();
+  add_corrections<C, 2>(sA, corr, rows, irr, line_start, y0, 0);
+  __syncthreads();
+#pragma unroll 1
+  for (int rep = 0; rep < reps; ++rep) {
+    dst_tile<C>(rep == 0 || rep == 3 ? sA : sB, mem);
+    if (rep == 0 || rep == 2) {
+      // every tile complete, the pieces exchanged, every piece read
+      cluster.sync();
+      xy_exchange<T, N>(cluster, rep == 0 ? sA : sB, rep == 0 ? sB : sA, y0);
+      cluster.sync();
+    } else if (rep == 1) {
+      const int c = threadIdx.x % W, p = y0 + c;
+      const T base = mu1[p] - lambda;
+#pragma unroll 4
+      for (int k = threadIdx.x / W; k < N; k += NT / W) {
+        T f;
+        if constexpr (sizeof(T) == 4)
+          f = p == 0 ? 0.0f : __fdividef(scale, mu1[k] + base);
+        else
+          f = rinv != nullptr ? rinv[(size_t)k * N + p]
+                              : (k > 0 && p > 0 ? scale / (mu1[k] + mu1[p] + (T)0 - lambda) : (T)0);
+        sB[k * RS + c] *= f;
+      }
+      __syncthreads();
+    }
+  }
+  put_lines<C, 2>(sA, a, keep, out, aux, beta, gamma, aux32, y0, 0);
+}
+
 template <typename K, typename... Args>
-cudaError_t launch_cluster(K kernel, int cl, dim3 grid, size_t smem, cudaStream_t st, Args... args) {
+cudaError_t launch_cluster(K kernel, int cl, dim3 grid, size_t smem, cudaStream_t st, bool pdl, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = cl;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -1273,11 +1366,11 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
         constexpr size_t sxy = xy_smem_bytes<N>();
         if ((rc = prep(k_xy_fwd<N>, sxy))) return rc;
         if ((rc = prep(k_xy_inv<N>, sxy))) return rc;
-        cudaError_t e = launch_cluster(k_xy_fwd<N>, N / 32, grid, sxy, st, work, sa.src, sa.alpha, sa.src32, sa.corr,
+        cudaError_t e = launch_cluster(k_xy_fwd<N>, N / 32, grid, sxy, st, false, work, sa.src, sa.alpha, sa.src32, sa.corr,
                                        (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, h->skip);
         if (e == cudaSuccess) {
           if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, nullptr, whole<N>()))) return rc;
-          e = launch_cluster(k_xy_inv<N>, N / 32, grid, sxy, st, work, sa.keep || sa.out_user == nullptr,
+          e = launch_cluster(k_xy_inv<N>, N / 32, grid, sxy, st, false, work, sa.keep || sa.out_user == nullptr,
                              sa.out_user, sa.aux, sa.beta, sa.gamma, tw, h->skip, sa.aux32);
           if (e != cudaSuccess) {
             set_error("cluster launch of the fused x-y inverse pass failed: %s", cudaGetErrorString(e));
@@ -1298,7 +1391,7 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
     const SolveSpans sp = solve_spans<N>(h, near_source(h, sa), near_result(h, sa));
     const dim3 gf((sp.xf_y.hi - sp.xf_y.lo) / W, sp.xf_z.hi - sp.xf_z.lo);
     const dim3 gi((sp.xi_y.hi - sp.xi_y.lo) / W, sp.xi_z.hi - sp.xi_z.lo);
-    if (launch_pass(h, k_xfwd<T, N, 3>, gf, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, (const int32_t*)t.irr,
+    if (launch_pass(h, k_xfwd<T, N, 3>, gf, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, sa.rows, (const int32_t*)t.irr,
                     (const int32_t*)t.line_start, tw, (const int*)h->skip, sp.xf_y.lo, sp.xf_z.lo) != cudaSuccess)
       return launch_failed("x forward pass");
     if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, sp.yf))) return rc;
@@ -1311,10 +1404,22 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
   } else {
     dim3 grid(N / W, 1);
     const T* rinv = mode_factors<T, N>(h, sa.lambda, (double)scale);
+    if constexpr (N >= 32 && N <= 256) {
+      constexpr size_t s2 = (2 * (size_t)N * C::RS + C::mem_elems) * sizeof(T);
+      if ((rc = prep(k_solve2d<T, N>, s2))) return rc;
+      if (launch_cluster(k_solve2d<T, N>, N / 32, dim3(N / 32), s2, st, h->rinv_ok, work, sa.src, sa.alpha, sa.src32,
+                         sa.corr, sa.rows, (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, mu1, lam, scale,
+                         rinv, sa.keep || sa.out_user == nullptr, sa.out_user, sa.aux, sa.beta, sa.gamma, sa.aux32,
+                         (const int*)h->skip, 4) == cudaSuccess) {
+        KFBI_CHECK_LAUNCH();
+        return KFBI_OK;
+      }
+      cudaGetLastError();  // no cluster of this size fits: three passes
+    }
     if ((rc = prep(k_xfwd<T, N, 2>, smem))) return rc;
     if ((rc = prep(k_strided<T, N, true, 2>, smem))) return rc;
     if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
-    if (launch_pass(h, k_xfwd<T, N, 2>, grid, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, (const int32_t*)t.irr,
+    if (launch_pass(h, k_xfwd<T, N, 2>, grid, smem, work, sa.src, sa.alpha, sa.src32, sa.corr, sa.rows, (const int32_t*)t.irr,
                     (const int32_t*)t.line_start, tw, (const int*)h->skip, 0, 0) != cudaSuccess)
       return launch_failed("x forward pass");
     if (launch_pass(h, k_strided<T, N, true, 2>, grid, smem, work, (size_t)N, (size_t)0, 0, mu1, lam, scale, tw,
@@ -1345,7 +1450,7 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
   if (dim == 3) {
     if (pass == 0) {
       if ((rc = prep(k_xfwd<T, N, 3>, smem))) return rc;
-      k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, t.irr, t.line_start, tw, nullptr, 0,
+      k_xfwd<T, N, 3><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, CorrRows{}, t.irr, t.line_start, tw, nullptr, 0,
                                                1);
     } else if (pass == 1) {
       if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, whole<N>()))) return rc;
@@ -1363,12 +1468,12 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
           cudaError_t e;
           if (pass == 4) {
             if ((rc = prep(k_xy_fwd<N>, sxy))) return rc;
-            e = launch_cluster(k_xy_fwd<N>, N / 32, grid, sxy, st, work, (const double*)nullptr, 1.0,
+            e = launch_cluster(k_xy_fwd<N>, N / 32, grid, sxy, st, false, work, (const double*)nullptr, 1.0,
                                (const float*)nullptr, (const double*)nullptr, (const int32_t*)t.irr,
                                (const int32_t*)t.line_start, tw, (const int*)nullptr);
           } else {
             if ((rc = prep(k_xy_inv<N>, sxy))) return rc;
-            e = launch_cluster(k_xy_inv<N>, N / 32, grid, sxy, st, work, true, (double*)nullptr,
+            e = launch_cluster(k_xy_inv<N>, N / 32, grid, sxy, st, false, work, true, (double*)nullptr,
                                (const double*)nullptr, 1.0, 0.0, tw, (const int*)nullptr, (const float*)nullptr);
           }
           if (e != cudaSuccess) {
@@ -1386,7 +1491,7 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
   } else {
     if (pass == 0) {
       if ((rc = prep(k_xfwd<T, N, 2>, smem))) return rc;
-      k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, t.irr, t.line_start, tw, nullptr, 0,
+      k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(work, nullptr, 1.0, nullptr, nullptr, CorrRows{}, t.irr, t.line_start, tw, nullptr, 0,
                                                0);
     } else if (pass == 1 || pass == 2) {
       const T* rinv = mode_factors<T, N>(h, lambda, (double)scale);
@@ -1413,7 +1518,7 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
 // its three factors per mode (v_i = f0 r_i + f1 r_e, v_e = f1 r_i + f2 r_e)
 // from a table built once per kappa in float64 (k_cpl_factors).
 template <typename T, int N, int DIM>
-__global__ void __launch_bounds__(NT) k_strided_coupled(T* __restrict__ a, T* __restrict__ b, size_t row_stride,
+__global__ void __launch_bounds__(NT, N <= 128 ? 2 : 1) k_strided_coupled(T* __restrict__ a, T* __restrict__ b, size_t row_stride,
                                                         size_t plane_stride, int qoff, const T* __restrict__ cf,
                                                         size_t cf_stride, const T* __restrict__ tw_g,
                                                         const int* __restrict__ skip, Span in, Span out) {
@@ -1553,7 +1658,7 @@ int run_solve_coupled(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, 
     for (int f = 0; f < 2; ++f) {
       const SolveArgs& sa = *sas[f];
       const dim3 gf((sp.xf_y.hi - sp.xf_y.lo) / W, sp.xf_z.hi - sp.xf_z.lo);
-      if (launch_pass(h, k_xfwd<T, N, 3>, gf, smem, grids[f], sa.src, sa.alpha, sa.src32, sa.corr,
+      if (launch_pass(h, k_xfwd<T, N, 3>, gf, smem, grids[f], sa.src, sa.alpha, sa.src32, sa.corr, sa.rows,
                       (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, (const int*)h->skip, sp.xf_y.lo,
                       sp.xf_z.lo) != cudaSuccess)
         return launch_failed("x forward pass");
@@ -1575,9 +1680,9 @@ int run_solve_coupled(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, 
     if ((rc = prep(k_xfwd<T, N, 2>, smem))) return rc;
     if ((rc = prep(k_strided_coupled<T, N, 2>, smem2))) return rc;
     if ((rc = prep(k_xinv<T, N, 2>, smem))) return rc;
-    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wa, si.src, si.alpha, si.src32, si.corr, t.irr, t.line_start, tw, h->skip,
+    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wa, si.src, si.alpha, si.src32, si.corr, si.rows, t.irr, t.line_start, tw, h->skip,
                                              0, 0);
-    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wb, se.src, se.alpha, se.src32, se.corr, t.irr, t.line_start, tw, h->skip,
+    k_xfwd<T, N, 2><<<grid, NT, smem, st>>>(wb, se.src, se.alpha, se.src32, se.corr, se.rows, t.irr, t.line_start, tw, h->skip,
                                              0, 0);
     k_strided_coupled<T, N, 2><<<grid, NT, smem2, st>>>(wa, wb, N, 0, 0, cf, (size_t)total, tw, h->skip, Span{0, N},
                                                         Span{0, N});

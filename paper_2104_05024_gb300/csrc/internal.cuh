@@ -323,7 +323,18 @@ int setup_build(kfbi_handle* h, const kfbi_geometry* geom);
 //  corr    : optional compact corrections at the irregular nodes (float64)
 //  out_user: optional user-layout float64 output  out = beta*v + gamma*aux
 //  keep    : true = leave the solution in the padded work grid
+//  rows    : the same corrections not yet summed: the x transform takes each
+//            irregular node's CSR row of the density vector x itself (2-D
+//            Dirichlet box; corr must then be null)
+struct CorrRows {
+  const int32_t* ptr = nullptr;
+  const int32_t* pid = nullptr;
+  const double* w = nullptr;
+  const double* x = nullptr;      // null: no rows
+};
+inline CorrRows corr_rows(const Tables& t, const double* x) { return CorrRows{t.cr_ptr, t.cr_pid, t.cr_w, x}; }
 struct SolveArgs {
+  CorrRows rows;
   const double* src = nullptr;
   const float* src32 = nullptr;   // float32 source on the user layout (alpha not applied)
   double alpha = 1.0;

@@ -176,27 +176,33 @@ struct ResArgs {
   const float *sh, *sl;  // pair source (may be the outputs themselves)
   float *res, *res_lo;
 };
+// A thread takes one x and RES_ROWS rows of a plane, the rows above and below
+// in registers (one block per line of two nodes a thread was bound by its
+// index arithmetic and loads: 70 / 134 us for one round / PAIR at 256^3).
+constexpr int RES_T = 128, RES_ROWS = 8;
 template <bool NEUMANN, Src SRC, bool PAIR>
-__global__ void __launch_bounds__(128) k_residual_ff(GridParams gr, const float* __restrict__ u32, ResArgs A) {
+__global__ void __launch_bounds__(RES_T) k_residual_ff(GridParams gr, const float* __restrict__ u32, ResArgs A) {
   // n values per field row, P per work-grid row (Neumann box: the grid is
   // the field, a neighbour beyond the box its mirror image; Dirichlet box:
   // index 0 of the grid and what lies beyond its last index is zero)
   const int n = NEUMANN ? gr.N + 1 : gr.N - 1, P = NEUMANN ? gr.N + 1 : gr.N;
-  const int y = blockIdx.x, z = blockIdx.y;
+  const int x = blockIdx.x * RES_T + threadIdx.x, y0 = blockIdx.y * RES_ROWS, z = blockIdx.z;
+  if (x >= n) return;
+  const int y1 = min(n, y0 + RES_ROWS);
   const int64_t PP = (int64_t)P * P;
   const bool d3 = gr.dim == 3;
-  const int64_t gbase = NEUMANN ? (int64_t)z * PP + (int64_t)y * P : (d3 ? (z + 1) * PP : 0) + (int64_t)(y + 1) * P + 1;
-  const int64_t fbase = ((int64_t)z * n + y) * n;
-  const int64_t ym = NEUMANN && y == 0 ? P : -P, yp = NEUMANN && y == n - 1 ? -P : P;
+  const float* up = u32 + x + (NEUMANN ? (int64_t)z * PP + (int64_t)y0 * P
+                                       : (d3 ? (z + 1) * PP : 0) + (int64_t)(y0 + 1) * P + 1);
+  int64_t f = ((int64_t)z * n + y0) * n + x;
   const int64_t zm = NEUMANN && z == 0 ? PP : -PP, zp = NEUMANN && z == n - 1 ? -PP : PP;
-  const bool y_on = NEUMANN || y < n - 1, z_on = NEUMANN || z < n - 1;
+  const bool z_on = NEUMANN || z < n - 1;
+  const int xl = NEUMANN && x == 0 ? 1 : -1, xr = NEUMANN && x == n - 1 ? -1 : 1;
+  const bool x_on = NEUMANN || x < n - 1;
+  float um = up[NEUMANN && y0 == 0 ? P : -P], uc = up[0];
 #pragma unroll 2
-  for (int x = threadIdx.x; x < n; x += 128) {
-    const float* up = u32 + gbase + x;
-    const float uc = up[0];
-    const float xm = up[NEUMANN && x == 0 ? 1 : -1];
-    const float xp = NEUMANN ? up[x == n - 1 ? -1 : 1] : x < n - 1 ? up[1] : 0.0f;
-    const float um = up[ym], upl = y_on ? up[yp] : 0.0f;
+  for (int y = y0; y < y1; ++y, up += P, f += n) {
+    const float xm = up[xl], xp = x_on ? up[xr] : 0.0f;
+    const float upl = y < n - 1 ? up[P] : NEUMANN ? um : 0.0f;
     float wm = 0.0f, wp = 0.0f;
     if (d3) {
       wm = up[zm];
@@ -204,7 +210,7 @@ __global__ void __launch_bounds__(128) k_residual_ff(GridParams gr, const float*
     }
     float q = 0.0f, m = 0.0f, l = 0.0f;  // the source
     if (SRC == Src::field) {
-      double v = A.src[fbase + x];
+      double v = A.src[f];
       if (PAIR) {
         if (A.alpha != 1.0) v *= A.alpha;
         if (!ffl::split3(v, q, m, l)) {
@@ -219,8 +225,8 @@ __global__ void __launch_bounds__(128) k_residual_ff(GridParams gr, const float*
       }
     }
     if (SRC == Src::pair) {
-      q = A.sh[fbase + x];
-      m = A.sl[fbase + x];
+      q = A.sh[f];
+      m = A.sl[f];
     }
     float s, e, t;
     two_sum(xm, xp, s, e);
@@ -267,8 +273,10 @@ __global__ void __launch_bounds__(128) k_residual_ff(GridParams gr, const float*
       rl = t1 + (m - (e1 + e2 + t0));
     }
     const float r = rh + rl;
-    A.res[fbase + x] = r;
-    if (PAIR) A.res_lo[fbase + x] = rl - (r - rh);
+    A.res[f] = r;
+    if (PAIR) A.res_lo[f] = rl - (r - rh);
+    um = uc;
+    uc = upl;
   }
 }
 
@@ -433,34 +441,6 @@ struct SmallLayout {
   __host__ __device__ int total() const { return y() + m + 2; }
 };
 
-// column j of H from hcol and sqrt(nrm2); apply rotations; new rotation; |g_{j+1}|
-__device__ void givens_column(double* s, int m, int j) {
-  SmallLayout L{m};
-  double* H = s + L.H();
-  double* cs = s + L.cs();
-  double* sn = s + L.sn();
-  double* g = s + L.g();
-  const double* hc = s + L.hcol();
-  double col[MAX_RESTART + 2];
-  for (int i = 0; i <= j; ++i) col[i] = hc[i];
-  col[j + 1] = sqrt(s[L.nrm2()]);
-  for (int i = 0; i < j; ++i) {
-    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
-  }
-  const double den = hypot(col[j], col[j + 1]);
-  cs[j] = col[j] / den;
-  sn[j] = col[j + 1] / den;
-  col[j] = den;
-  col[j + 1] = 0.0;
-  g[j + 1] = -sn[j] * g[j];
-  g[j] = cs[j] * g[j];
-  for (int i = 0; i <= j + 1; ++i) H[(size_t)j * (m + 1) + i] = col[i];
-  s[L.res()] = fabs(g[j + 1]);
-}
-
-
 // ------------------------------------------------- single-launch reductions
 // Each thread owns a grid-stride set of rows; the last block to finish (a
 // ticket counter, reset by that block) reduces the per-block partial sums in
@@ -594,8 +574,8 @@ __device__ __forceinline__ void arn_dots(const ArnArgs& A, double (*red)[MAX_RES
 // w_i -= sum_k cs[k] V_k[i] over the block's rows; each chunk's loads are
 // independent, so a thread has ARN_CH of them in flight.  vn (optional)
 // receives the result times inv as well.
-__device__ __forceinline__ void arn_update(const ArnArgs& A, const double* cs, double* vn, double inv) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) {
+__device__ __forceinline__ void arn_update(const ArnArgs& A, const double* cs, double* vn, double inv, int nb) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += nb * blockDim.x) {
     double acc = 0.0;
     for (int k0 = 0; k0 < A.nv; k0 += ARN_CH) {
       double x[ARN_CH];
@@ -620,19 +600,41 @@ __device__ __forceinline__ double arn_norm2(const double* y, int nv) {
   return t > 0.0 ? t : 0.0;
 }
 
-// Givens update, estimate and stop flag (one thread; hcol and nrm2 are set)
-__device__ __forceinline__ void arn_finish(const ArnArgs& A) {
+// Column j of H (col: hcol, then sqrt(n2)), the earlier rotations (cs, sn in
+// shared memory like col: from global memory each step of the chain waits
+// for its loads), the new rotation, |g_{j+1}|, the stop flag (one thread)
+__device__ __forceinline__ void arn_finish(const ArnArgs& A, double* col, const double* cs, const double* sn,
+                                           double n2) {
   SmallLayout L{A.m};
   double* s = A.s;
-  givens_column(s, A.m, A.j);
-  const double rel = s[L.res()] / A.gnorm;
+  const int j = A.j;
+  double c0 = col[0];
+  const double last = sqrt(n2);
+  for (int i = 0; i < j; ++i) {
+    const double c1 = col[i + 1];
+    col[i] = cs[i] * c0 + sn[i] * c1;
+    c0 = -sn[i] * c0 + cs[i] * c1;
+  }
+  const double den = hypot(c0, last), c = c0 / den, sj = last / den;
+  const double gj = s[L.g() + j], g1 = -sj * gj;
+  const double res = fabs(g1), rel = res / A.gnorm;
   const int done = !(rel > A.tol) || !isfinite(rel);
   *A.stop = done;
   // the decision last: the host polls it
   volatile double* host = A.host;
-  host[0] = s[L.res()];
+  host[0] = res;
   __threadfence_system();
   host[1] = done ? 1.0 : 0.0;
+  s[L.cs() + j] = c;
+  s[L.sn() + j] = sj;
+  s[L.g() + j + 1] = g1;
+  s[L.g() + j] = c * gj;
+  s[L.res()] = res;
+  s[L.nrm2()] = n2;
+  double* H = s + L.H() + (size_t)j * (A.m + 1);
+  for (int i = 0; i < j; ++i) H[i] = col[i];
+  H[j] = den;
+  H[j + 1] = 0.0;
 }
 
 // [UPDATE: w -= sum_k coef[k] V_k;]  out[k] = V_k . w (k < nv), and with
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(256) k_arn_gs(ArnArgs A, const double* __restr
   if (UPDATE) {
     for (int k = threadIdx.x; k < A.nv; k += blockDim.x) cs[k] = coef[k];
     __syncthreads();
-    arn_update(A, cs, nullptr, 0.0);
+    arn_update(A, cs, nullptr, 0.0, gridDim.x);
   }
   // each thread reads back only the rows it updated itself
   arn_dots<UPDATE>(A, red);
@@ -663,22 +665,29 @@ __global__ void __launch_bounds__(256) k_arn_gs(ArnArgs A, const double* __restr
   if (threadIdx.x == 0) *A.counter = 0u;
 }
 
-// v_{j+1} = (w - sum_k y[k] V_k) / |.|; the first block also closes column j
+// v_{j+1} = (w - sum_k y[k] V_k) / |.|, and column j by one more block
 __global__ void __launch_bounds__(256) k_arn_close(ArnArgs A) {
   pdl_wait();
   pdl_launch_next();
   if (A.skip != nullptr && *A.skip) return;
   SmallLayout L{A.m};
-  __shared__ double y[MAX_RESTART + 2];
-  for (int k = threadIdx.x; k <= A.nv; k += blockDim.x) y[k] = A.s[L.y() + k];
+  const bool closing = blockIdx.x == gridDim.x - 1;  // closes column j while the others update
+  __shared__ double y[MAX_RESTART + 2], col[MAX_RESTART + 2], cs[MAX_RESTART], sn[MAX_RESTART];
+  for (int k = threadIdx.x; k <= A.nv; k += blockDim.x) {
+    y[k] = A.s[L.y() + k];
+    if (closing && k < A.nv) col[k] = A.s[L.hcol() + k] + y[k];
+    if (closing && k < A.j) {
+      cs[k] = A.s[L.cs() + k];
+      sn[k] = A.s[L.sn() + k];
+    }
+  }
   __syncthreads();
   const double n2 = arn_norm2(y, A.nv), norm = sqrt(n2);
-  arn_update(A, y, A.V + (size_t)(A.j + 1) * A.ld, norm > 0.0 ? 1.0 / norm : 0.0);
-  if (blockIdx.x != 0) return;
-  for (int k = threadIdx.x; k < A.nv; k += blockDim.x) A.s[L.hcol() + k] += y[k];
-  if (threadIdx.x == 0) A.s[L.nrm2()] = n2;
-  __syncthreads();
-  if (threadIdx.x == 0) arn_finish(A);
+  if (closing) {
+    if (threadIdx.x == 0) arn_finish(A, col, cs, sn, n2);
+    return;
+  }
+  arn_update(A, y, A.V + (size_t)(A.j + 1) * A.ld, norm > 0.0 ? 1.0 / norm : 0.0, gridDim.x - 1);
 }
 
 // the whole step by one block
@@ -687,8 +696,12 @@ __global__ void __launch_bounds__(ARN_ONE_T) k_arn_one(ArnArgs A) {
   pdl_launch_next();
   if (A.skip != nullptr && *A.skip) return;
   __shared__ double red[ARN_ONE_T / 32][MAX_RESTART + 2];
-  __shared__ double h[MAX_RESTART + 2], y[MAX_RESTART + 2];
+  __shared__ double h[MAX_RESTART + 2], y[MAX_RESTART + 2], cs[MAX_RESTART], sn[MAX_RESTART];
   SmallLayout L{A.m};
+  for (int k = threadIdx.x; k < A.j; k += ARN_ONE_T) {
+    cs[k] = A.s[L.cs() + k];
+    sn[k] = A.s[L.sn() + k];
+  }
   auto sum = [&](double* out, int nd) {
     for (int k = threadIdx.x; k < nd; k += ARN_ONE_T) {
       double t = 0.0;
@@ -700,15 +713,14 @@ __global__ void __launch_bounds__(ARN_ONE_T) k_arn_one(ArnArgs A) {
   };
   arn_dots<false>(A, red);
   sum(h, A.nv);
-  arn_update(A, h, nullptr, 0.0);
+  arn_update(A, h, nullptr, 0.0, 1);
   arn_dots<true>(A, red);
   sum(y, A.nv + 1);
   const double n2 = arn_norm2(y, A.nv), norm = sqrt(n2);
-  for (int k = threadIdx.x; k < A.nv; k += ARN_ONE_T) A.s[L.hcol() + k] = h[k] + y[k];
-  if (threadIdx.x == 0) A.s[L.nrm2()] = n2;
-  arn_update(A, y, A.V + (size_t)(A.j + 1) * A.ld, norm > 0.0 ? 1.0 / norm : 0.0);
+  for (int k = threadIdx.x; k < A.nv; k += ARN_ONE_T) h[k] += y[k];
+  arn_update(A, y, A.V + (size_t)(A.j + 1) * A.ld, norm > 0.0 ? 1.0 / norm : 0.0, 1);
   __syncthreads();
-  if (threadIdx.x == 0) arn_finish(A);
+  if (threadIdx.x == 0) arn_finish(A, h, cs, sn, n2);
 }
 
 // Normal equations of the density-history projection in one launch:
@@ -1094,11 +1106,11 @@ static FTrip ftrip(double v) {
 template <Src SRC, bool PAIR>
 static void residual_ff(kfbi_handle* h, const float* u32, const ResArgs& A) {
   const int n = field_n(h->grid);
-  const dim3 grid(n, h->grid.dim == 3 ? n : 1);
+  const dim3 grid((n + RES_T - 1) / RES_T, (n + RES_ROWS - 1) / RES_ROWS, h->grid.dim == 3 ? n : 1);
   if (h->grid.bc == KFBI_BOX_NEUMANN)
-    k_residual_ff<true, SRC, PAIR><<<grid, 128, 0, h->stream>>>(h->grid, u32, A);
+    k_residual_ff<true, SRC, PAIR><<<grid, RES_T, 0, h->stream>>>(h->grid, u32, A);
   else
-    k_residual_ff<false, SRC, PAIR><<<grid, 128, 0, h->stream>>>(h->grid, u32, A);
+    k_residual_ff<false, SRC, PAIR><<<grid, RES_T, 0, h->stream>>>(h->grid, u32, A);
 }
 
 int launch_residual_ff(kfbi_handle* h, const double* src, double alpha, const double* corr, const float* u32,
@@ -1521,7 +1533,7 @@ int arnoldi_step(kfbi_handle* h, double* V, int ld, double* wv, int j, int m, do
   if (launch_pdl(k_arn_gs<false>, dim3(nb), dim3(256), 0, st, A, (const double*)nullptr, s + L.hcol()) != cudaSuccess ||
       launch_pdl(k_arn_gs<true>, dim3(nb), dim3(256), 0, st, A, (const double*)(s + L.hcol()), s + L.y()) !=
           cudaSuccess ||
-      launch_pdl(k_arn_close, dim3(nb), dim3(256), 0, st, A) != cudaSuccess)
+      launch_pdl(k_arn_close, dim3(nb + 1), dim3(256), 0, st, A) != cudaSuccess)
     return launch_failed("Arnoldi step");
   KFBI_CHECK_LAUNCH_N(3);
   return KFBI_OK;

@@ -48,59 +48,57 @@ __device__ __forceinline__ float dsilu_f(float z) {
   return s * (1.0f + z * (1.0f - s));
 }
 
-// C[M x N] (=, or += by atomics for split-K) A[M x K] B[K x N]; bf16 operands,
-// float32 accumulation.  A row-major: A[m lda + k]; col-major: A[k lda + m].
-// B row-major: B[k ldb + n]; col-major: B[n ldb + k].  M, N, K multiples of 16.
-template <typename LA, typename LB, bool ATOMIC>
-__global__ void __launch_bounds__(128) k_gemm(const bf16* __restrict__ A, int lda, const bf16* __restrict__ B, int ldb,
-                                              float* __restrict__ C, int ldc, int M, int N, int K, int kchunk) {
+// Weight gradients dW_l += d_l^T A_{l-1} of the four hidden layers in one
+// launch (bf16 operands, float32 accumulation and atomics; A_{-1} = X).  A
+// block owns a 64 x 64 tile of one layer's product over `kch` rows: the row
+// sum is a serial chain of 16-row products, so it is split into about one
+// block per SM and layer (16 blocks of 1024 rows each took 107 us a layer at
+// 4096 rows).
+struct WeightGrad {
+  const bf16 *d[4], *A[4];  // delta [Bp][128], activation [Bp][lda]
+  float* g[4];              // [128][n]
+};
+__global__ void __launch_bounds__(128) k_weight_grad(WeightGrad P, int K, int kch, int splits) {
   using namespace nvcuda;
+  const int l = blockIdx.z / splits, split = blockIdx.z % splits;
+  const int lda = l == 0 ? KIN : WID, n = l == 0 ? NIN : WID, N = l == 0 ? KIN : WID;
   const int warp = threadIdx.x >> 5, wy = warp >> 1, wx = warp & 1;
   const int m0 = blockIdx.y * TILE + wy * 32, n0 = blockIdx.x * TILE + wx * 32;
-  const int k0 = blockIdx.z * kchunk;
-  const int k1 = min(K, k0 + kchunk);
+  if (n0 >= N) return;
+  const bf16 *D = P.d[l], *A = P.A[l];
+  const int k0 = split * kch, k1 = min(K, k0 + kch);
   wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc[2][2];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) wmma::fill_fragment(acc[i][j], 0.0f);
-  const bool a_row = std::is_same<LA, wmma::row_major>::value;
-  const bool b_row = std::is_same<LB, wmma::row_major>::value;
+#pragma unroll 2
   for (int k = k0; k < k1; k += 16) {
-    wmma::fragment<wmma::matrix_a, 16, 16, 16, bf16, LA> fa[2];
-    wmma::fragment<wmma::matrix_b, 16, 16, 16, bf16, LB> fb[2];
+    wmma::fragment<wmma::matrix_a, 16, 16, 16, bf16, wmma::col_major> fa[2];
+    wmma::fragment<wmma::matrix_b, 16, 16, 16, bf16, wmma::row_major> fb[2];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int m = m0 + i * 16;
-      if (m < M) wmma::load_matrix_sync(fa[i], a_row ? A + (size_t)m * lda + k : A + (size_t)k * lda + m, lda);
-    }
+    for (int i = 0; i < 2; ++i) wmma::load_matrix_sync(fa[i], D + (size_t)k * WID + m0 + i * 16, WID);
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int n = n0 + j * 16;
-      if (n < N) wmma::load_matrix_sync(fb[j], b_row ? B + (size_t)k * ldb + n : B + (size_t)n * ldb + k, ldb);
-    }
+    for (int j = 0; j < 2; ++j)
+      if (n0 + j * 16 < N) wmma::load_matrix_sync(fb[j], A + (size_t)k * lda + n0 + j * 16, lda);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 2; ++j)
-        if (m0 + i * 16 < M && n0 + j * 16 < N) wmma::mma_sync(acc[i][j], fa[i], fb[j], acc[i][j]);
+        if (n0 + j * 16 < N) wmma::mma_sync(acc[i][j], fa[i], fb[j], acc[i][j]);
   }
   __shared__ float stage[4][16 * 16];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int m = m0 + i * 16, n = n0 + j * 16;
-      if (m >= M || n >= N) continue;
-      if (!ATOMIC) {
-        wmma::store_matrix_sync(C + (size_t)m * ldc + n, acc[i][j], ldc, wmma::mem_row_major);
-      } else {
-        wmma::store_matrix_sync(stage[warp], acc[i][j], 16, wmma::mem_row_major);
-        __syncwarp();
-        for (int e = threadIdx.x & 31; e < 256; e += 32)
-          atomicAdd(C + (size_t)(m + e / 16) * ldc + n + (e % 16), stage[warp][e]);
-        __syncwarp();
-      }
+      const int mb = m0 + i * 16, nb = n0 + j * 16;
+      if (nb >= N) continue;
+      wmma::store_matrix_sync(stage[warp], acc[i][j], 16, wmma::mem_row_major);
+      __syncwarp();
+      for (int e = threadIdx.x & 31; e < 256; e += 32)
+        if (nb + (e % 16) < n) atomicAdd(P.g[l] + (size_t)(mb + e / 16) * n + nb + (e % 16), stage[warp][e]);
+      __syncwarp();
     }
 }
 
@@ -202,101 +200,6 @@ __global__ void __launch_bounds__(256) k_moments(const float* __restrict__ F, co
   }
 }
 
-__global__ void k_bias_act(float* __restrict__ Z, const float* __restrict__ bias, bf16* __restrict__ A, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float z = Z[i] + bias[i % WID];
-  Z[i] = z;
-  A[i] = __float2bfloat16_rn(silu_f(z));
-}
-
-// o_b = sum_j A3[b][j] w4[j] + b4 (one warp per row)
-__global__ void k_out(const bf16* __restrict__ A, const bf16* __restrict__ w4, const float* __restrict__ b4, float* o,
-                      int Bp) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= Bp) return;
-  float acc = 0.0f;
-  for (int j = lane; j < WID; j += 32) acc += __bfloat162float(A[(size_t)row * WID + j]) * __bfloat162float(w4[j]);
-  for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
-  if (lane == 0) o[row] = acc + b4[0];
-}
-
-// output-layer delta d4 = (o - t)/B and the loss partial sums; the raw
-// targets T are normalised first, t = (T - m_out) / s_out (norm[18], norm[19])
-__global__ void k_delta_out(const float* __restrict__ o, const float* __restrict__ T, const float* __restrict__ norm,
-                            int B, int Bp, float* d4, float* loss) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  float r = 0.0f;
-  if (b < B) r = o[b] - (T[b] - norm[2 * NIN]) / norm[2 * NIN + 1];
-  if (b < Bp) d4[b] = r / (float)B;
-  float sq = r * r;
-  for (int s = 16; s > 0; s >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, s);
-  if ((threadIdx.x & 31) == 0 && sq != 0.0f) atomicAdd(loss, sq);
-}
-
-// Row-wise backward kernels: a block of 256 threads owns BACK_ROWS rows (two
-// rows at a time, one thread per column), so that a column's sums over the
-// block's rows need one float32 atomic each: with one atomic per element the
-// 4096-row output layer took 22 us (4096 additions to each of 128 addresses)
-// and the bias sums were a pass of their own (17 us a layer); now 4-5 us with
-// the sums included.
-constexpr int BACK_ROWS = 16;
-
-// a column's value of the two row halves to one atomic addition
-__device__ __forceinline__ void column_add(float* g, float v, float* red) {
-  const int j = threadIdx.x & (WID - 1);
-  if (threadIdx.x >= WID) red[j] = v;
-  __syncthreads();
-  if (threadIdx.x < WID) atomicAdd(g + j, v + red[j]);
-  __syncthreads();
-}
-
-// gradients of the output layer, delta of the last hidden layer (d optional)
-// and its bias gradient
-__global__ void __launch_bounds__(256) k_back_out(const float* __restrict__ d4, const bf16* __restrict__ A3,
-                                                  const float* __restrict__ Z3, const bf16* __restrict__ w4, float* gw4,
-                                                  float* gb4, float* gb, float* d, bf16* db, int Bp) {
-  __shared__ float red[WID];
-  const int j = threadIdx.x & (WID - 1);
-  const float w = __bfloat162float(w4[j]);
-  const int b1 = min(Bp, (int)(blockIdx.x + 1) * BACK_ROWS);
-  float sw = 0.0f, sb = 0.0f, s4 = 0.0f;
-#pragma unroll 4
-  for (int b = blockIdx.x * BACK_ROWS + (threadIdx.x >> 7); b < b1; b += 2) {
-    const size_t i = (size_t)b * WID + j;
-    const float q = d4[b], dq = __bfloat162float(__float2bfloat16_rn(q));
-    sw += dq * __bfloat162float(A3[i]);
-    s4 += q;
-    const float v = dq * w * dsilu_f(Z3[i]);
-    sb += v;
-    if (d != nullptr) d[i] = v;
-    db[i] = __float2bfloat16_rn(v);
-  }
-  if (j == 0) atomicAdd(gb4, s4);
-  column_add(gw4, sw, red);
-  column_add(gb, sb, red);
-}
-
-// delta of a hidden layer from the delta's product with the weights, and its
-// bias gradient
-__global__ void __launch_bounds__(256) k_dsilu(const float* __restrict__ da, const float* __restrict__ Z, float* gb,
-                                               float* d, bf16* db, int Bp) {
-  __shared__ float red[WID];
-  const int j = threadIdx.x & (WID - 1);
-  const int b1 = min(Bp, (int)(blockIdx.x + 1) * BACK_ROWS);
-  float sb = 0.0f;
-#pragma unroll 4
-  for (int b = blockIdx.x * BACK_ROWS + (threadIdx.x >> 7); b < b1; b += 2) {
-    const size_t i = (size_t)b * WID + j;
-    const float v = da[i] * dsilu_f(Z[i]);
-    sb += v;
-    if (d != nullptr) d[i] = v;
-    db[i] = __float2bfloat16_rn(v);
-  }
-  column_add(gb, sb, red);
-}
-
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                        int n, float lr, float c1, float c2) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -322,12 +225,6 @@ __global__ void k_refresh(const float* __restrict__ p, Offsets off, bf16* W0, bf
     W3[i] = __float2bfloat16_rn(p[off.w[3] + i]);
   }
   if (i < WID) w4[i] = __float2bfloat16_rn(p[off.w[4] + i]);
-}
-
-// W0 gradient: columns 0..8 of the padded [128][16] product
-__global__ void k_unpad_w0(const float* __restrict__ g16, float* gw0) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < WID * NIN) gw0[i] += g16[(i / NIN) * KIN + i % NIN];
 }
 
 // psi_L = psi_F + 2 gamma r_F + rms(r_F) * (s_out o + m_out), the network
@@ -430,6 +327,186 @@ __global__ void __launch_bounds__(256, 1) k_mlp_infer(const bf16* __restrict__ X
   }
 }
 
+// Forward and backward pass of a training batch but for the weight products,
+// one launch: a block takes TR rows through the four hidden layers and, with
+// targets, back through their deltas (both are row-wise), with the bfloat16
+// weights and the current layer's operands in shared memory.  Pre-activations
+// and activations go to memory once (the backward pass and the weight
+// gradients read them); a column's sums over the block's rows (bias and
+// output gradients) take one float32 atomic each.  As one launch per product
+// and pointwise pass (22 launches of 3 to 22 us) the 4096-row gradient took
+// 200 us.  Same products and summation order per element as k_mlp_infer.
+constexpr int TR = 32;
+constexpr size_t STEP_SMEM = (size_t)3 * WID * LDW * 2 + (size_t)WID * LDX * 2 + (size_t)TR * LDW * 2 +
+                             (size_t)TR * LDX * 2 + (size_t)TR * LDS * 4 + (size_t)4 * WID * 4 + (size_t)2 * WID * 4 +
+                             (size_t)TR * 4;
+struct StepArgs {
+  const float *F, *T;  // raw rows [B][9], raw targets [B] (null: forward only)
+  const float* norm;
+  int B;
+  const bf16 *W0, *W[3], *w4;
+  const float* p;
+  Offsets off;
+  bf16* X;
+  float* Z[4];
+  bf16 *A[4], *db[4];
+  float *o, *d4, *g, *loss, *dump_d;
+};
+
+// a column's values of the two row halves to one atomic addition
+__device__ __forceinline__ void column_add(float* g, float v, float* red) {
+  const int j = threadIdx.x & (WID - 1);
+  if (threadIdx.x >= WID) red[j] = v;
+  __syncthreads();
+  if (threadIdx.x < WID) atomicAdd(g + j, v + red[j]);
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(256, 1) k_mlp_step(StepArgs P) {
+  using namespace nvcuda;
+  extern __shared__ __align__(128) unsigned char sm_step[];
+  bf16* sW = reinterpret_cast<bf16*>(sm_step);  // 3 x [WID][LDW], W[n][k]
+  bf16* sW0 = sW + 3 * WID * LDW;                // [WID][LDX]
+  bf16* sA = sW0 + WID * LDX;                    // [TR][LDW] activations, then deltas
+  bf16* sX = sA + TR * LDW;                      // [TR][LDX]
+  float* sZ = reinterpret_cast<float*>(sX + TR * LDX);  // [TR][LDS]
+  float* sB = sZ + TR * LDS;                     // [4][WID]
+  float* sw4 = sB + 4 * WID;                     // [WID]
+  float* red = sw4 + WID;                        // [WID]
+  float* sd4 = red + WID;                        // [TR]
+  const int tid = threadIdx.x, row0 = blockIdx.x * TR;
+  for (int l = 0; l < 3; ++l)
+    for (int i = tid; i < WID * WID / 8; i += blockDim.x) {
+      const int n = i / (WID / 8), q = i % (WID / 8);
+      *reinterpret_cast<uint4*>(sW + (size_t)l * WID * LDW + n * LDW + 8 * q) =
+          *reinterpret_cast<const uint4*>(P.W[l] + (size_t)n * WID + 8 * q);
+    }
+  for (int i = tid; i < WID * KIN / 8; i += blockDim.x) {
+    const int n = i / (KIN / 8), q = i % (KIN / 8);
+    *reinterpret_cast<uint4*>(sW0 + n * LDX + 8 * q) = *reinterpret_cast<const uint4*>(P.W0 + (size_t)n * KIN + 8 * q);
+  }
+  for (int i = tid; i < 4 * WID; i += blockDim.x) sB[i] = P.p[P.off.b[i / WID] + i % WID];
+  for (int i = tid; i < WID; i += blockDim.x) sw4[i] = __bfloat162float(P.w4[i]);
+  for (int i = tid; i < TR * KIN; i += blockDim.x) {
+    const int r = i / KIN, c = i % KIN, b = row0 + r;
+    float v = 0.0f;
+    if (b < P.B && c < NIN) v = (P.F[(size_t)b * NIN + c] - P.norm[c]) / P.norm[NIN + c];
+    const bf16 x = __float2bfloat16_rn(v);
+    sX[r * LDX + c] = x;
+    P.X[(size_t)b * KIN + c] = x;
+  }
+  const int warp = tid >> 5, lane = tid & 31;
+  const int rb = warp & 1, cb = (warp >> 1) * 2;  // 16-row block, two 16-column blocks
+  const int col = tid & (WID - 1), r0 = tid >> 7;  // the pointwise passes: one column, every other row
+  wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc[2];
+  auto store = [&]() {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      wmma::store_matrix_sync(sZ + rb * 16 * LDS + (cb + j) * 16, acc[j], LDS, wmma::mem_row_major);
+    __syncthreads();  // every warp has read its inputs and written its products
+  };
+  __syncthreads();
+  for (int l = 0; l < 4; ++l) {
+    const bf16* Ain = l == 0 ? sX : sA;
+    const int lda = l == 0 ? LDX : LDW, K = l == 0 ? KIN : WID;
+    const bf16* Bw = l == 0 ? sW0 : sW + (size_t)(l - 1) * WID * LDW;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) wmma::fill_fragment(acc[j], 0.0f);
+    for (int k0 = 0; k0 < K; k0 += 16) {
+      wmma::fragment<wmma::matrix_a, 16, 16, 16, bf16, wmma::row_major> fa;
+      wmma::load_matrix_sync(fa, Ain + rb * 16 * lda + k0, lda);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        wmma::fragment<wmma::matrix_b, 16, 16, 16, bf16, wmma::col_major> fb;
+        wmma::load_matrix_sync(fb, Bw + (cb + j) * 16 * lda + k0, lda);
+        wmma::mma_sync(acc[j], fa, fb, acc[j]);
+      }
+    }
+    store();
+    const float bias = sB[l * WID + col];
+    float* Z = P.Z[l] + (size_t)row0 * WID + col;
+    bf16* A = P.A[l] + (size_t)row0 * WID + col;
+#pragma unroll 4
+    for (int r = r0; r < TR; r += 2) {
+      const float z = sZ[r * LDS + col] + bias;
+      const bf16 a = __float2bfloat16_rn(silu_f(z));
+      Z[(size_t)r * WID] = z;
+      A[(size_t)r * WID] = a;
+      sA[r * LDW + col] = a;
+    }
+    __syncthreads();
+  }
+  // output, its delta and the loss
+  const float b4 = P.p[P.off.b[4]];
+  float sq = 0.0f;
+  for (int r = warp; r < TR; r += 8) {
+    float v = 0.0f;
+    for (int j = lane; j < WID; j += 32) v += __bfloat162float(sA[r * LDW + j]) * sw4[j];
+    for (int sft = 16; sft > 0; sft >>= 1) v += __shfl_xor_sync(0xffffffffu, v, sft);
+    const int b = row0 + r;
+    const float o = v + b4;
+    if (lane == 0) P.o[b] = o;
+    if (P.T != nullptr) {
+      const float e = b < P.B ? o - (P.T[b] - P.norm[2 * NIN]) / P.norm[2 * NIN + 1] : 0.0f;
+      sq += e * e;
+      if (lane == 0) {
+        sd4[r] = e / (float)P.B;
+        P.d4[b] = sd4[r];
+      }
+    }
+  }
+  if (P.T == nullptr) return;
+  if (lane == 0) atomicAdd(P.loss, sq);
+  __syncthreads();
+  if (warp == 0) {
+    float v = sd4[lane];
+    for (int sft = 16; sft > 0; sft >>= 1) v += __shfl_xor_sync(0xffffffffu, v, sft);
+    if (lane == 0) atomicAdd(P.g + P.off.b[4], v);
+  }
+  // deltas of the hidden layers, last first (a thread reads back the
+  // pre-activations it wrote)
+  for (int l = 3; l >= 0; --l) {
+    const float* Z = P.Z[l] + (size_t)row0 * WID + col;
+    bf16* db = P.db[l] + (size_t)row0 * WID + col;
+    float* dump = P.dump_d == nullptr ? nullptr : P.dump_d + ((size_t)(3 - l) * P.B + row0) * WID + col;
+    float sb = 0.0f, sw = 0.0f;
+#pragma unroll 4
+    for (int r = r0; r < TR; r += 2) {
+      float v;
+      if (l == 3) {
+        const float dq = __bfloat162float(__float2bfloat16_rn(sd4[r]));
+        sw += dq * __bfloat162float(sA[r * LDW + col]);
+        v = dq * sw4[col] * dsilu_f(Z[(size_t)r * WID]);
+      } else {
+        v = sZ[r * LDS + col] * dsilu_f(Z[(size_t)r * WID]);
+      }
+      sb += v;
+      if (dump != nullptr && row0 + r < P.B) dump[(size_t)r * WID] = v;
+      const bf16 q = __float2bfloat16_rn(v);
+      db[(size_t)r * WID] = q;
+      sA[r * LDW + col] = q;
+    }
+    if (l == 3) column_add(P.g + P.off.w[4], sw, red);
+    column_add(P.g + P.off.b[l], sb, red);
+    if (l == 0) break;
+    // d_l W_l: W_l's rows are its outputs, so it is the row-major right factor
+    const bf16* Bw = sW + (size_t)(l - 1) * WID * LDW;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) wmma::fill_fragment(acc[j], 0.0f);
+    for (int k0 = 0; k0 < WID; k0 += 16) {
+      wmma::fragment<wmma::matrix_a, 16, 16, 16, bf16, wmma::row_major> fa;
+      wmma::load_matrix_sync(fa, sA + rb * 16 * LDW + k0, LDW);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        wmma::fragment<wmma::matrix_b, 16, 16, 16, bf16, wmma::row_major> fb;
+        wmma::load_matrix_sync(fb, Bw + (size_t)k0 * LDW + (cb + j) * 16, LDW);
+        wmma::mma_sync(acc[j], fa, fb, acc[j]);
+      }
+    }
+    store();
+  }
+}
+
 }  // namespace
 }  // namespace kfbi
 
@@ -442,8 +519,8 @@ struct kfbi_mlp {
   bf16* X = nullptr;
   bf16* A[4] = {nullptr, nullptr, nullptr, nullptr};
   float* Z[4] = {nullptr, nullptr, nullptr, nullptr};
-  float *o = nullptr, *d4 = nullptr, *d = nullptr, *da = nullptr, *g16 = nullptr, *loss = nullptr;
-  bf16* db = nullptr;
+  float *o = nullptr, *d4 = nullptr, *loss = nullptr;  // loss: the element after g
+  bf16* db[4] = {nullptr, nullptr, nullptr, nullptr};
   float* dump_d = nullptr;   // kfbi_mlp_layers: per-layer deltas go here (else null)
   float* dump_d4 = nullptr;
   int step = 0;
@@ -464,23 +541,6 @@ int malloc_mlp(kfbi_mlp* m, T** p, size_t n) {
 }
 
 int blocks(size_t n, int bs) { return (int)((n + bs - 1) / bs); }
-
-// forward over rows already placed in m->X; leaves o, Z, A
-int mlp_forward_rows(kfbi_mlp* m, int Bp) {
-  using namespace nvcuda;
-  cudaStream_t st = m->stream;
-  const dim3 g(WID / TILE, Bp / TILE, 1);
-  k_gemm<wmma::row_major, wmma::col_major, false><<<g, 128, 0, st>>>(m->X, KIN, m->W0, KIN, m->Z[0], WID, Bp, WID, KIN, KIN);
-  k_bias_act<<<blocks((size_t)Bp * WID, 256), 256, 0, st>>>(m->Z[0], m->p + m->off.b[0], m->A[0], Bp * WID);
-  for (int l = 1; l < 4; ++l) {
-    k_gemm<wmma::row_major, wmma::col_major, false><<<g, 128, 0, st>>>(m->A[l - 1], WID, m->W[l - 1], WID, m->Z[l], WID,
-                                                                       Bp, WID, WID, WID);
-    k_bias_act<<<blocks((size_t)Bp * WID, 256), 256, 0, st>>>(m->Z[l], m->p + m->off.b[l], m->A[l], Bp * WID);
-  }
-  k_out<<<blocks((size_t)Bp * 32, 256), 256, 0, st>>>(m->A[3], m->w4, m->p + m->off.b[4], m->o, Bp);
-  KFBI_CHECK_LAUNCH_N(9);
-  return KFBI_OK;
-}
 
 // inference over rows already placed in m->X (Bp a multiple of 64): m->o
 int mlp_infer_rows(kfbi_mlp* m, int Bp) {
@@ -515,50 +575,58 @@ int mlp_prepare_raw(kfbi_mlp* m, const float* F, int B, int* Bp) {
   return KFBI_OK;
 }
 
-// gradients of 0.5 mean (o - t)^2 into m->g (rows already forwarded)
-int mlp_backward(kfbi_mlp* m, const float* t, int B, int Bp) {
-  using namespace nvcuda;
+// forward pass over raw rows F (leaves o, Z, A, X) and, with raw targets t,
+// the gradients of 0.5 mean (o - t)^2 into m->g and the squared error sum
+int mlp_step(kfbi_mlp* m, const float* F, const float* t, int B) {
+  if (B < 1 || B > m->bmax) {
+    set_error("batch %d outside 1..%d", B, m->bmax);
+    return KFBI_ERR_ARG;
+  }
+  static bool opted = false;
+  if (!opted) {
+    if (cudaFuncSetAttribute(k_mlp_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)STEP_SMEM) != cudaSuccess) {
+      set_error("cudaFuncSetAttribute failed for the training kernel");
+      return KFBI_ERR_CUDA;
+    }
+    opted = true;
+  }
   cudaStream_t st = m->stream;
   const Offsets& off = m->off;
-  KFBI_CUDA(cudaMemsetAsync(m->g, 0, sizeof(float) * off.total, st));
-  KFBI_CUDA(cudaMemsetAsync(m->loss, 0, sizeof(float), st));
-  KFBI_CUDA(cudaMemsetAsync(m->g16, 0, sizeof(float) * WID * KIN, st));
-  k_delta_out<<<blocks(Bp, 256), 256, 0, st>>>(m->o, t, m->norm, B, Bp, m->d4, m->loss);
-  float* d = m->dump_d ? m->d : nullptr;
-  const int nrow = blocks(Bp, BACK_ROWS);
-  k_back_out<<<nrow, 256, 0, st>>>(m->d4, m->A[3], m->Z[3], m->w4, m->g + off.w[4], m->g + off.b[4], m->g + off.b[3], d,
-                                   m->db, Bp);
-  int launched = 2;
-  if (m->dump_d4) KFBI_CUDA(cudaMemcpyAsync(m->dump_d4, m->d4, sizeof(float) * B, cudaMemcpyDeviceToDevice, st));
-  for (int l = 3; l >= 0; --l) {
-    if (m->dump_d)
-      KFBI_CUDA(cudaMemcpyAsync(m->dump_d + (size_t)(3 - l) * B * WID, m->d, sizeof(float) * B * WID,
-                                cudaMemcpyDeviceToDevice, st));
-    // weight gradient d^T A_{l-1}, split over rows (float32 atomics) into
-    // about one block per SM: the row sum is a serial chain of 16-row
-    // products (in 1024-row pieces, 16 blocks, 107 us a layer at 4096 rows)
-    const int tiles = (l == 0 ? 1 : WID / TILE) * (WID / TILE);
-    const int kch = std::max(TILE, blocks((size_t)Bp * tiles, 152 * TILE) * TILE);
-    const dim3 gg(l == 0 ? 1 : WID / TILE, WID / TILE, blocks(Bp, kch));
-    if (l > 0) {
-      k_gemm<wmma::col_major, wmma::row_major, true><<<gg, 128, 0, st>>>(m->db, WID, m->A[l - 1], WID, m->g + off.w[l],
-                                                                         WID, WID, WID, Bp, kch);
-    } else {
-      k_gemm<wmma::col_major, wmma::row_major, true><<<gg, 128, 0, st>>>(m->db, WID, m->X, KIN, m->g16, KIN, WID, KIN,
-                                                                         Bp, kch);
-      k_unpad_w0<<<blocks(WID * NIN, 256), 256, 0, st>>>(m->g16, m->g + off.w[0]);
-      ++launched;
-    }
-    ++launched;
-    if (l > 0) {
-      const dim3 g2(WID / TILE, Bp / TILE, 1);
-      k_gemm<wmma::row_major, wmma::row_major, false><<<g2, 128, 0, st>>>(m->db, WID, m->W[l - 1], WID, m->da, WID, Bp,
-                                                                          WID, WID, WID);
-      k_dsilu<<<nrow, 256, 0, st>>>(m->da, m->Z[l - 1], m->g + off.b[l - 1], d, m->db, Bp);
-      launched += 2;
-    }
+  const int Bp = (B + TILE - 1) / TILE * TILE;
+  StepArgs P;
+  P.F = F;
+  P.T = t;
+  P.norm = m->norm;
+  P.B = B;
+  P.W0 = m->W0;
+  P.w4 = m->w4;
+  P.p = m->p;
+  P.off = off;
+  P.X = m->X;
+  P.o = m->o;
+  P.d4 = m->d4;
+  P.g = m->g;
+  P.loss = m->loss;
+  P.dump_d = m->dump_d;
+  for (int l = 0; l < 3; ++l) P.W[l] = m->W[l];
+  WeightGrad G;
+  for (int l = 0; l < 4; ++l) {
+    P.Z[l] = m->Z[l];
+    P.A[l] = m->A[l];
+    P.db[l] = m->db[l];
+    G.d[l] = m->db[l];
+    G.A[l] = l == 0 ? m->X : m->A[l - 1];
+    G.g[l] = m->g + off.w[l];
   }
-  KFBI_CHECK_LAUNCH_N(launched);
+  if (t != nullptr) KFBI_CUDA(cudaMemsetAsync(m->g, 0, sizeof(float) * (off.total + 1), st));
+  k_mlp_step<<<Bp / TR, 256, STEP_SMEM, st>>>(P);
+  KFBI_CHECK_LAUNCH();
+  if (t == nullptr) return KFBI_OK;
+  if (m->dump_d4) KFBI_CUDA(cudaMemcpyAsync(m->dump_d4, m->d4, sizeof(float) * B, cudaMemcpyDeviceToDevice, st));
+  const int tiles = (WID / TILE) * (WID / TILE);
+  const int kch = std::max(TILE, blocks((size_t)Bp * tiles, 152 * TILE) * TILE), splits = blocks(Bp, kch);
+  k_weight_grad<<<dim3(WID / TILE, WID / TILE, 4 * splits), 128, 0, st>>>(G, Bp, kch, splits);
+  KFBI_CHECK_LAUNCH();
   return KFBI_OK;
 }
 
@@ -650,18 +718,18 @@ int kfbi_mlp_create(const float* params_host, const float* norm_host, int max_ba
     kfbi_mlp_destroy(m);
     return code;
   };
-  if ((rc = malloc_mlp(m, &m->p, P)) || (rc = malloc_mlp(m, &m->g, P)) || (rc = malloc_mlp(m, &m->m, P)) ||
+  if ((rc = malloc_mlp(m, &m->p, P)) || (rc = malloc_mlp(m, &m->g, P + 1)) || (rc = malloc_mlp(m, &m->m, P)) ||
       (rc = malloc_mlp(m, &m->v, P)) || (rc = malloc_mlp(m, &m->norm, 2 * NIN + 2)) ||
       (rc = malloc_mlp(m, &m->W0, WID * KIN)) || (rc = malloc_mlp(m, &m->w4, WID)) ||
-      (rc = malloc_mlp(m, &m->X, Bp * KIN)) || (rc = malloc_mlp(m, &m->o, Bp)) || (rc = malloc_mlp(m, &m->d4, Bp)) ||
-      (rc = malloc_mlp(m, &m->d, Bp * WID)) || (rc = malloc_mlp(m, &m->da, Bp * WID)) ||
-      (rc = malloc_mlp(m, &m->db, Bp * WID)) || (rc = malloc_mlp(m, &m->g16, WID * KIN)) ||
-      (rc = malloc_mlp(m, &m->loss, 1)))
+      (rc = malloc_mlp(m, &m->X, Bp * KIN)) || (rc = malloc_mlp(m, &m->o, Bp)) || (rc = malloc_mlp(m, &m->d4, Bp)))
     return fail(rc);
+  m->loss = m->g + P;
   for (int l = 0; l < 3; ++l)
     if ((rc = malloc_mlp(m, &m->W[l], WID * WID))) return fail(rc);
   for (int l = 0; l < 4; ++l)
-    if ((rc = malloc_mlp(m, &m->A[l], Bp * WID)) || (rc = malloc_mlp(m, &m->Z[l], Bp * WID))) return fail(rc);
+    if ((rc = malloc_mlp(m, &m->A[l], Bp * WID)) || (rc = malloc_mlp(m, &m->Z[l], Bp * WID)) ||
+        (rc = malloc_mlp(m, &m->db[l], Bp * WID)))
+      return fail(rc);
   cudaStream_t st = m->stream;
   if (cudaMemcpyAsync(m->p, params_host, sizeof(float) * P, cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(m->norm, norm_host, sizeof(float) * (2 * NIN + 2), cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -715,10 +783,7 @@ int kfbi_mlp_grad(kfbi_mlp* m, const float* F_dev, const float* t_dev, int B, fl
     set_error("null argument");
     return KFBI_ERR_ARG;
   }
-  int Bp, rc;
-  if ((rc = mlp_prepare_raw(m, F_dev, B, &Bp))) return rc;
-  if ((rc = mlp_forward_rows(m, Bp))) return rc;
-  if ((rc = mlp_backward(m, t_dev, B, Bp))) return rc;
+  if (int rc = mlp_step(m, F_dev, t_dev, B)) return rc;
   float l = 0.0f;
   KFBI_CUDA(cudaMemcpyAsync(&l, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
   if (grad_host)
@@ -734,22 +799,17 @@ int kfbi_mlp_layers(kfbi_mlp* m, const float* F_dev, const float* T_dev, int B, 
     set_error("null argument");
     return KFBI_ERR_ARG;
   }
-  int Bp, rc;
-  if ((rc = mlp_prepare_raw(m, F_dev, B, &Bp))) return rc;
-  if ((rc = mlp_forward_rows(m, Bp))) return rc;
   cudaStream_t st = m->stream;
+  m->dump_d = T_dev ? d_dev : nullptr;
+  m->dump_d4 = T_dev ? d4_dev : nullptr;
+  const int rc = mlp_step(m, F_dev, T_dev, B);
+  m->dump_d = m->dump_d4 = nullptr;
+  if (rc) return rc;
   if (z_dev)
     for (int l = 0; l < 4; ++l)
       KFBI_CUDA(cudaMemcpyAsync(z_dev + (size_t)l * B * WID, m->Z[l], sizeof(float) * B * WID,
                                 cudaMemcpyDeviceToDevice, st));
   if (o_dev) KFBI_CUDA(cudaMemcpyAsync(o_dev, m->o, sizeof(float) * B, cudaMemcpyDeviceToDevice, st));
-  if (T_dev) {
-    m->dump_d = d_dev;
-    m->dump_d4 = d4_dev;
-    rc = mlp_backward(m, T_dev, B, Bp);
-    m->dump_d = m->dump_d4 = nullptr;
-    if (rc) return rc;
-  }
   KFBI_CUDA(cudaStreamSynchronize(st));
   return KFBI_OK;
 }

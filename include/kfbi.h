@@ -316,9 +316,9 @@ int kfbi_export_tables(kfbi_handle* h, double* node_wn, int32_t* node_cnt, int32
 /* Box solve (Sections 5.2-5.3): v = L_h^{-1} r, 5/7-point operator with the
  * handle's box condition (zero Dirichlet data by sine transforms, or the
  * Neumann box's mirrored ghost rows by cosine transforms).  precision
- * KFBI_FP64 (float64 transforms), KFBI_MIXED / KFBI_MIXED_LEARNED (float32
- * transforms refined by one round of the float64 residual, two when the
- * handle's tolerance is below 1e-9: float64-accurate) or KFBI_FP32 (float32
+ * KFBI_FP64 (64-bit transforms), KFBI_MIXED / KFBI_MIXED_LEARNED (float32
+ * transforms refined by one round of an extended-precision residual, two when
+ * the handle's tolerance is below 1e-9: float64-accurate) or KFBI_FP32 (float32
  * transforms only).                                                         */
 int kfbi_box_solve(kfbi_handle* h, int precision, double lambda, const double* r_dev, double* v_dev);
 
@@ -436,8 +436,8 @@ int kfbi_training_rows(kfbi_handle* h, float* F_dev, float* T_dev);
 
 /* One pass of the box solver on the handle's padded work grid, for timing
  * the transform kernels in isolation: pass 0 = x forward (no right-hand
- * side), 1 = y forward, 2 = z solve (forward, spectral divide, inverse; the
- * y solve in 2-D), 3 = x inverse; with kfbi_info.xy_fused also 4 = fused x-y
+ * side), 1 = y forward, 2 = z solve (elimination, or forward, spectral divide,
+ * inverse for nearly Poisson lambda; the y solve in 2-D), 3 = x inverse; with kfbi_info.xy_fused also 4 = fused x-y
  * forward and 5 = fused x-y inverse (KFBI_MIXED).  precision KFBI_FP64 or
  * KFBI_MIXED.  The grid content is arbitrary afterwards.                     */
 int kfbi_transform_pass(kfbi_handle* h, int precision, int pass, double lambda);
@@ -456,8 +456,8 @@ int64_t kfbi_launch_count(void);
 
 /*
  * Box solve for callers that cannot allocate device memory (the paper has no
- * counterpart).  Same operation and result as kfbi_box_solve with precision
- * KFBI_FP64 -- v = L_h^{-1} r on the (N-1)^dim interior nodes of [lo, hi]^dim
+ * counterpart).  Same operation as kfbi_box_solve with precision KFBI_FP64,
+ * the same result to rounding -- v = L_h^{-1} r on the (N-1)^dim interior nodes of [lo, hi]^dim
  * with zero Dirichlet data -- but without a handle and without any device
  * allocation: some callers run where every byte of device memory belongs to a
  * pool or arena they do not control, or where allocation after start-up is

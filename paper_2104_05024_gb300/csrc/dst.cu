@@ -18,7 +18,8 @@
 //   x forward  : assembles r = alpha*src + corrections (irregular nodes) while
 //                loading, transforms along x;
 //   y forward  : strided rows, coalesced W-wide segments;
-//   z solve    : forward DST, spectral divide, inverse DST in one pass;
+//   z solve    : elimination per (x, y) mode, or forward DST, spectral divide,
+//                inverse DST in one pass;
 //   y forward  : (the DST-I is its own inverse up to the folded scale);
 //   x inverse  : transforms along x and writes the padded grid and/or a user
 //                layout output  beta*v + gamma*aux.
@@ -85,7 +86,7 @@ struct Tile {
   static constexpr size_t smem_elems = (size_t)N * RS + mem_elems;
   // resident blocks per SM the registers are budgeted for (shared memory
   // allows no more for long lines)
-  static constexpr int BLOCKS = FIX ? (N <= 256 ? 2 : 1) : REG ? (N <= 256 ? 3 : 2) : 1;
+  static constexpr int BLOCKS = FIX ? (N <= 256 ? 2 : 1) : REG ? (N <= 256 ? 4 : 2) : 1;
 };
 
 template <typename T, int N>
@@ -941,6 +942,169 @@ __global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const _
   if (threadIdx.x == 0) tma_wait_all();
 }
 
+// ------------------------------------- z solve by elimination (3-D, N >= 32)
+// After the x and y transforms every (p, q) mode leaves one symmetric Toeplitz
+// tridiagonal system along z,
+//   (2 + eps) v_k - v_{k-1} - v_{k+1} = R_k = -h^2 (2/N)^2 r_k,
+//   eps = -h^2 (mu1[p] + mu1[q] - lambda) > 0,
+// which elimination solves in about 5 operations per value, against two
+// transforms of 20 to 25 each and a division.  Eliminating from both ends to
+// the middle halves the serial chain and shares its pivots (they depend on
+// the distance from the end only); a tile of TW columns is two threads per
+// column.  The pivots d_k = 1 + s_k are kept as s_k = eps + s_{k-1} /
+// d_{k-1}, all terms positive, so that eps (as small as 1e-4) is never
+// rounded against 2; the middle row's pivot is eps + 2 s / d.  float32 forms
+// 1 / d as it goes; float64, whose divisions would be the whole cost, reads
+// it from a table built per lambda (N/2 values per mode, row 0 the inverse of
+// the middle pivot).
+// Measured at 256^3: float32 59 -> 40 us, float64 292 -> 192 us a pass (512^3
+// float32 515 -> 451 us): bound by the chain and the tile's load latency at
+// 8 warps per SM (48 KB of rows and pivots per 32 columns).
+template <typename T, int N>
+struct ZTri {
+  static constexpr int TW = sizeof(T) == 8 && N >= 384 ? 16 : 32;  // columns (64 KB of float64 at most)
+  static constexpr int NTH = 2 * TW, M = N / 2;
+  static constexpr bool INLINE_G = sizeof(T) == 4;
+  static constexpr size_t smem = ((size_t)N * TW + (INLINE_G ? (size_t)M * TW : 0) + NTH) * sizeof(T);
+};
+
+template <typename T, int N>
+__global__ void __launch_bounds__(ZTri<T, N>::NTH) k_ztri(T* __restrict__ a, const T* __restrict__ mu1, T lambda, T h2,
+                                                          T rs, const T* __restrict__ tab, const int* __restrict__ skip,
+                                                          Span in, Span out) {
+  using Z = ZTri<T, N>;
+  constexpr int TW = Z::TW, NTH = Z::NTH, M = Z::M, CH = 8;
+  constexpr int CPR = TW * (int)sizeof(T) / 16, RPS = NTH / CPR, EPC = 16 / (int)sizeof(T);  // 16-byte pieces of a row
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T* s = reinterpret_cast<T*>(smem_raw);
+  T* gs = s + N * TW;                                  // 1 / d_j (float32)
+  T* mid = gs + (Z::INLINE_G ? M * TW : 0);
+  pdl_wait();
+  if (skip != nullptr && *skip != 0) return;
+  const int x0 = blockIdx.x * TW, q = blockIdx.y + 1;
+  constexpr size_t rstride = (size_t)N * N;
+  T* base = a + (size_t)q * N + x0;
+  const int piece = EPC * (threadIdx.x % CPR), r0 = threadIdx.x / CPR;
+#pragma unroll 4
+  for (int k = in.lo + r0; k < in.hi; k += RPS) copy_async16(s + k * TW + piece, base + k * rstride + piece);
+  for (int i = threadIdx.x; i < in.lo * TW; i += NTH) s[i] = (T)0;
+  for (int i = in.hi * TW + threadIdx.x; i < N * TW; i += NTH) s[i] = (T)0;
+  const int half = threadIdx.x / TW, c = threadIdx.x % TW, p = x0 + c;
+  const T eps = -h2 * (mu1[p] + mu1[q] - lambda);
+  const T* tq = tab + (Z::INLINE_G ? 0 : (size_t)q * M * N + p);
+  copy_async_wait();
+  __syncthreads();
+  // rows j = 1 .. M - 1 from this half's end
+  T* sr = s + (half ? N * TW : 0) + c;
+  const int rstep = half ? -TW : TW;
+  auto pivot = [&](T sv) -> T {
+    const float d = 1.0f + (float)sv, r = __fdividef(1.0f, d);
+    return (T)fmaf(r, fmaf(-d, r, 1.0f), r);
+  };
+  T y = (T)0, g = (T)0, sv = (T)0;
+  // rows (and table pivots) in batches of CH; with the table the next batch
+  // is loaded before this one's chain (223 -> 192 us at 256^3; float32, whose
+  // batches come from shared memory, ran slower with it: 40 -> 47 us)
+  constexpr bool AHEAD = !Z::INLINE_G;
+  T r[CH], gg[CH];
+  auto fetch = [&](int j0) {
+#pragma unroll
+    for (int u = 0; u < CH; ++u) {
+      const bool on = j0 + u < M;
+      r[u] = on ? sr[(j0 + u) * rstep] : (T)0;
+      if constexpr (!Z::INLINE_G) gg[u] = on ? tq[(size_t)(j0 + u) * N] : (T)0;
+    }
+  };
+  if (AHEAD) fetch(1);
+#pragma unroll 1
+  for (int j0 = 1; j0 < M; j0 += CH) {
+    if (!AHEAD) fetch(j0);
+    T rc[CH], gc[CH];
+#pragma unroll
+    for (int u = 0; u < CH; ++u) {
+      rc[u] = r[u];
+      gc[u] = gg[u];
+    }
+    if (AHEAD) fetch(j0 + CH);
+#pragma unroll
+    for (int u = 0; u < CH; ++u) {
+      const int j = j0 + u;
+      if (j < M) {
+        y = g * y + rs * rc[u];
+        if constexpr (Z::INLINE_G) {
+          sv = j == 1 ? 1.0f + eps : sv * g + eps;
+          g = pivot(sv);
+          if (half == 0) gs[j * TW + c] = g;
+        } else {
+          g = gc[u];
+        }
+        sr[j * rstep] = y;
+      }
+    }
+  }
+  mid[threadIdx.x] = y * g;
+  const T rm = rs * s[M * TW + c];
+  __syncthreads();
+  const T num = rm + mid[c] + mid[TW + c];
+  T v;
+  if constexpr (Z::INLINE_G)
+    v = num / (eps + 2.0f * sv * g);
+  else
+    v = num * tq[0];
+  if (half == 0) s[M * TW + c] = v;
+  auto fetch_back = [&](int j0) {
+#pragma unroll
+    for (int u = 0; u < CH; ++u) {
+      const int j = j0 - u;
+      r[u] = j > 0 ? sr[j * rstep] : (T)0;
+      if constexpr (Z::INLINE_G)
+        gg[u] = j > 0 ? gs[j * TW + c] : (T)0;
+      else
+        gg[u] = j > 0 ? tq[(size_t)j * N] : (T)0;
+    }
+  };
+  if (AHEAD) fetch_back(M - 1);
+#pragma unroll 1
+  for (int j0 = M - 1; j0 > 0; j0 -= CH) {
+    if (!AHEAD) fetch_back(j0);
+    T rc[CH], gc[CH];
+#pragma unroll
+    for (int u = 0; u < CH; ++u) {
+      rc[u] = r[u];
+      gc[u] = gg[u];
+    }
+    if (AHEAD) fetch_back(j0 - CH);
+#pragma unroll
+    for (int u = 0; u < CH; ++u)
+      if (j0 - u > 0) {
+        v = (rc[u] + v) * gc[u];
+        sr[(j0 - u) * rstep] = v;
+      }
+  }
+  __syncthreads();
+  pdl_launch_next();
+#pragma unroll 4
+  for (int k = out.lo + r0; k < out.hi; k += RPS)
+    *reinterpret_cast<float4*>(base + k * rstride + piece) = *reinterpret_cast<const float4*>(s + k * TW + piece);
+}
+
+// 1 / d_j of every (q, p) mode at row j of its table, the inverse of the
+// middle pivot at row 0
+__global__ void k_ztab(const double* __restrict__ mu1, double lambda, double h2, int N, double* __restrict__ tab) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y, M = N / 2;
+  if (p >= N) return;
+  const double eps = -h2 * (mu1[p] + mu1[q] - lambda);
+  double* t = tab + (size_t)q * M * N + p;
+  double s = 1.0 + eps, g = 1.0 / (1.0 + s);
+  t[N] = g;
+  for (int j = 2; j < M; ++j) {
+    s = fma(s, g, eps);
+    g = 1.0 / (1.0 + s);
+    t[(size_t)j * N] = g;
+  }
+  t[0] = 1.0 / (eps + 2.0 * s * g);
+}
+
 // ------------------------------- fused x and y passes (thread-block clusters)
 // One z-plane of the padded float32 grid is transformed along x and then y
 // by a cluster of N / 32 blocks (N <= 256) that exchange the plane through
@@ -1304,6 +1468,70 @@ SolveSpans solve_spans(const kfbi_handle* h, bool in, bool out) {
   return s;
 }
 
+// Whether the z systems of this lambda are solved by elimination.  Its error
+// grows with the number of rows 1 / sqrt(eps) over which the slowest mode (p
+// = q = 1) remembers its roundings; up to 48 rows it is below the two
+// transforms' (float32, z stage alone, against 80 bits: 4e-7 at 256 rows and
+// 5e-7 at 512 for lambda = 60, where the transforms leave 9e-7 and 1.7e-6;
+// at 110 rows 3e-6).  The time-step problems (lambda = 40, 60, ...) are well
+// inside; Poisson and nearly Poisson problems on fine grids keep the
+// transforms.
+template <int N>
+bool z_by_elimination(const kfbi_handle* h, double lambda) {
+  if (N < 32 || h->grid.dim != 3) return false;
+  const double s = std::sin(3.14159265358979323846 / (2.0 * N));
+  const double eps = h->grid.h * h->grid.h * lambda + 8.0 * s * s;  // -h^2 (2 mu1[1] - lambda)
+  return eps * (48.0 * 48.0) >= 1.0;
+}
+
+// the float64 pivot table for this lambda (N^3 / 2 values, built once per
+// lambda), nullptr where the handle has none
+inline const double* z_table(kfbi_handle* h, double lambda, int N) {
+  if (!h->rinv_ok) return nullptr;
+  if (h->ztab == nullptr) {
+    if (dalloc(h, &h->ztab, (size_t)N * N * (N / 2)) != KFBI_OK) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    h->ztab_lambda = std::nan("");
+  }
+  if (!(h->ztab_lambda == lambda)) {
+    k_ztab<<<dim3((N + 127) / 128, N), 128, 0, h->stream>>>(h->t.mu, lambda, h->grid.h * h->grid.h, N, h->ztab);
+    KFBI_COUNT(1);
+    h->ztab_lambda = lambda;
+  }
+  return h->ztab;
+}
+
+// the z pass of a 3-D solve: elimination where z_by_elimination allows it,
+// else forward transform, spectral divide, inverse transform
+template <typename T, int N>
+const T* mode_factors(kfbi_handle* h, double lambda, double scale);
+template <typename T, int N>
+int launch_zsolve(kfbi_handle* h, double lambda, T* work, const T* mu1, T scale, const T* tw, const PassSpan& ps) {
+  if constexpr (N >= 32) {
+    using Z = ZTri<T, N>;
+    bool tri = z_by_elimination<N>(h, lambda);
+    const T* tab = nullptr;
+    if constexpr (sizeof(T) == 8) {
+      if (tri) tab = z_table(h, lambda, N);
+      tri = tri && tab != nullptr;
+    }
+    if (tri) {
+      int rc;
+      if ((rc = prep(k_ztri<T, N>, Z::smem))) return rc;
+      const double h2 = h->grid.h * h->grid.h;
+      const T rs = (T)(-h2 * (2.0 / N) * (2.0 / N));
+      if (launch_pdl(k_ztri<T, N>, dim3(N / Z::TW, N - 1), dim3(Z::NTH), Z::smem, h->stream, work, mu1, (T)lambda,
+                     (T)h2, rs, tab, (const int*)h->skip, ps.in, ps.out) != cudaSuccess)
+        return launch_failed("z elimination pass");
+      return KFBI_OK;
+    }
+  }
+  return launch_strided3<T, N>(h, 1, true, work, mu1, (T)lambda, scale, tw,
+                               mode_factors<T, N>(h, lambda, (double)scale), ps);
+}
+
 // scale / mu_p over the mode grid (q, k, p) of the float64 middle pass,
 // mu_p = (mu1[k] + mu1[p]) + mu1[q] (3-D) - lambda, in the pass's own order;
 // n modes per axis, mode 0 absent (sine modes) or present (cosine modes)
@@ -1369,7 +1597,7 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
         cudaError_t e = launch_cluster(k_xy_fwd<N>, N / 32, grid, sxy, st, false, work, sa.src, sa.alpha, sa.src32, sa.corr,
                                        (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, h->skip);
         if (e == cudaSuccess) {
-          if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, nullptr, whole<N>()))) return rc;
+          if ((rc = launch_zsolve<T, N>(h, sa.lambda, work, mu1, scale, tw, whole<N>()))) return rc;
           e = launch_cluster(k_xy_inv<N>, N / 32, grid, sxy, st, false, work, sa.keep || sa.out_user == nullptr,
                              sa.out_user, sa.aux, sa.beta, sa.gamma, tw, h->skip, sa.aux32);
           if (e != cudaSuccess) {
@@ -1384,7 +1612,6 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
         h->xy_fused = false;
       }
     }
-    const T* rinv = mode_factors<T, N>(h, sa.lambda, (double)scale);
     if ((rc = prep(k_xfwd<T, N, 3>, smem))) return rc;
     if ((rc = prep(k_xinv<T, N, 3>, smem))) return rc;
     // the five passes chained by programmatic dependent launch
@@ -1395,7 +1622,7 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
                     (const int32_t*)t.line_start, tw, (const int*)h->skip, sp.xf_y.lo, sp.xf_z.lo) != cudaSuccess)
       return launch_failed("x forward pass");
     if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, sp.yf))) return rc;
-    if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, rinv, sp.z))) return rc;
+    if ((rc = launch_zsolve<T, N>(h, sa.lambda, work, mu1, scale, tw, sp.z))) return rc;
     if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, sp.yi))) return rc;
     if (launch_pass(h, k_xinv<T, N, 3>, gi, smem, work, sa.keep || sa.out_user == nullptr, sa.out_user,
                     (const double*)sa.aux, sa.beta, sa.gamma, tw, (const int*)h->skip, sa.aux32, sp.xi_y.lo,
@@ -1455,8 +1682,7 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
     } else if (pass == 1) {
       if ((rc = launch_strided3<T, N>(h, 0, false, work, mu1, lam, scale, tw, nullptr, whole<N>()))) return rc;
     } else if (pass == 2) {
-      const T* rinv = mode_factors<T, N>(h, lambda, (double)scale);
-      if ((rc = launch_strided3<T, N>(h, 1, true, work, mu1, lam, scale, tw, rinv, whole<N>()))) return rc;
+      if ((rc = launch_zsolve<T, N>(h, lambda, work, mu1, scale, tw, whole<N>()))) return rc;
     } else if (pass == 3) {
       if ((rc = prep(k_xinv<T, N, 3>, smem))) return rc;
       k_xinv<T, N, 3><<<grid, NT, smem, st>>>(work, true, nullptr, nullptr, 1.0, 0.0, tw, nullptr, nullptr, 0, 1);
@@ -1738,6 +1964,11 @@ int dispatch_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1
 // with the same mu_p as the sine solve (p = 0..N).  Work and user grids share
 // the layout (N+1)^d, x fastest.  A tile holds N+1 transform rows by W lines.
 
+// (float64 lines take the shared-memory FFT, whose long tiles stay at 16 lines)
+template <typename T, int N>
+struct NCfg : Tile<T, N, (sizeof(T) == 8 && N >= 384 ? 16 : WSel<T, N>::W),
+                   (sizeof(T) == 8 && N >= 384 ? 16 : WSel<T, N>::W) + 1> {};
+
 template <typename C>
 constexpr size_t dct_smem_elems() {
   // tile, scan totals, twiddles, X_1 per column, sines (register path)
@@ -1884,7 +2115,7 @@ __global__ void __launch_bounds__(NT) k_nxfwd(T* __restrict__ a, const double* _
                                               const double* __restrict__ corr, const int32_t* __restrict__ irr,
                                               const int32_t* __restrict__ line_start, const T* __restrict__ tw_g,
                                               const int* __restrict__ skip) {
-  using C = Cfg<T, N>;
+  using C = NCfg<T, N>;
   constexpr int W = C::W, RS = C::RS, P = N + 1, n1 = N - 1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
@@ -1935,7 +2166,7 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
                                               const double* __restrict__ aux, double beta, double gamma,
                                               const T* __restrict__ tw_g, const int* __restrict__ skip,
                                               const float* __restrict__ aux32) {
-  using C = Cfg<T, N>;
+  using C = NCfg<T, N>;
   constexpr int W = C::W, RS = C::RS, P = N + 1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
@@ -1992,7 +2223,7 @@ __global__ void __launch_bounds__(NT) k_nstrided(T* __restrict__ a, size_t row_s
                                                  const T* __restrict__ mu1, T lambda, T scale,
                                                  const T* __restrict__ tw_g, const int* __restrict__ skip,
                                                  const T* __restrict__ rinv = nullptr) {
-  using C = Cfg<T, N>;
+  using C = NCfg<T, N>;
   constexpr int W = C::W, RS = C::RS, P = N + 1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
@@ -2034,7 +2265,7 @@ __global__ void __launch_bounds__(NT) k_nstrided(T* __restrict__ a, size_t row_s
 
 template <typename T, int N>
 int run_solve_neumann(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const T* tw) {
-  using C = Cfg<T, N>;
+  using C = NCfg<T, N>;
   constexpr int W = C::W, P = N + 1;
   const size_t smem = dct_smem_elems<C>() * sizeof(T);
   const int dim = h->grid.dim;

@@ -285,6 +285,9 @@ struct kfbi_handle {
   double* rinv64 = nullptr;
   double rinv_lambda = 0.0;
   bool rinv_ok = false;
+  // float64 z elimination: the pivots for the lambda they were built for
+  double* ztab = nullptr;
+  double ztab_lambda = 0.0;
   // coupled solves: the per-mode 2 x 2 solve factors for the kappa they were
   // built for, one table per element type (3 N^dim values each)
   double* cpl64 = nullptr;

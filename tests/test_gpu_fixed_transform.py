@@ -63,6 +63,32 @@ def test_box_solve_matches_dense_products(dim, N, kind):
     h.close()
 
 
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("N,lams", [(32, (0.0, 1e5)), (64, (0.0, 60.0)), (256, (0.0, 2.0, 60.0, 1e5)), (384, (5.0, 60.0))])
+def test_z_elimination_and_transforms_match_dense_products(N, lams, precision):
+    """Both sides of the rule that picks the z solve: elimination (lambda
+    large against the mode spacing), transforms (Poisson and nearly so on
+    fine grids)."""
+    import torch
+    from kfbi_workloads import configs as C, geometry as G
+    from paper_2104_05024_gb300 import kfbi as K
+    grid = C.Grid(3, N)
+    h = K.KFBI(G.sphere3(0.5, max(4, N // 4)), grid)
+    dev = torch.device("cuda:0")
+    for kind in ("smooth", "sparse"):
+        r = field(kind, grid.shape, N, dev)
+        v = torch.empty_like(r)
+        for lam in lams:
+            h.box_solve(r, v, lam, precision=K.FP64 if precision == "fp64" else K.FP32)
+            ref = dense_solve(r, N, lam)
+            err = float((v - ref).norm() / ref.norm())
+            # float64: six transforms' bound as above; float32: the same
+            # roundings at 2^-24 instead of 2^-53
+            bound = 6 * 3e-15 * math.sqrt(N / 512.0) + 1e-15
+            assert err < (bound if precision == "fp64" else bound * 2.0 ** 29), (kind, lam, err)
+    h.close()
+
+
 def test_non_finite_sources_reach_the_solution():
     import torch
     from kfbi_workloads import configs as C, geometry as G

@@ -1743,6 +1743,21 @@ int run_pass(kfbi_handle* h, int pass, double lambda, T* work, const T* mu1, con
 // scaled by (2/N)^d, then the inverse DST of both tiles.  The solve takes
 // its three factors per mode (v_i = f0 r_i + f1 r_e, v_e = f1 r_i + f2 r_e)
 // from a table built once per kappa in float64 (k_cpl_factors).
+//
+// Two tiles per block where they fit in shared memory.  They do not for
+// float64 lines of 512 (284 672 bytes): there one tile takes the fields in
+// turn, and field a's modes wait in its work grid (every element read back by
+// the thread that wrote it, from L2); the values are the same.
+constexpr size_t SMEM_MAX = 232448;  // shared memory a block can have
+template <typename T, int N>
+struct CoupledTiles {
+  using C = Cfg<T, N>;
+  static constexpr size_t one = (size_t)N * C::RS, max_elems = SMEM_MAX / sizeof(T);
+  static constexpr bool TWO = 2 * one + C::mem_elems <= max_elems;
+  static constexpr size_t smem = ((TWO ? 2 : 1) * one + C::mem_elems) * sizeof(T);
+  static_assert(smem <= SMEM_MAX, "tiles of the coupled pass");
+};
+
 template <typename T, int N, int DIM>
 __global__ void __launch_bounds__(NT, N <= 128 ? 2 : 1) k_strided_coupled(T* __restrict__ a, T* __restrict__ b, size_t row_stride,
                                                         size_t plane_stride, int qoff, const T* __restrict__ cf,
@@ -1750,9 +1765,10 @@ __global__ void __launch_bounds__(NT, N <= 128 ? 2 : 1) k_strided_coupled(T* __r
                                                         const int* __restrict__ skip, Span in, Span out) {
   using C = Cfg<T, N>;
   constexpr int W = C::W, RS = C::RS;
+  constexpr bool TWO = CoupledTiles<T, N>::TWO;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* sa = reinterpret_cast<T*>(smem_raw);
-  T* sb = sa + N * RS;
+  T* sb = TWO ? sa + N * RS : sa;
   T* mem = sb + N * RS;
   load_tables<C>(mem, tw_g);
   pdl_wait();
@@ -1761,37 +1777,72 @@ __global__ void __launch_bounds__(NT, N <= 128 ? 2 : 1) k_strided_coupled(T* __r
   const int q = blockIdx.y + qoff;
   T* ba = a + (size_t)q * plane_stride + x0;
   T* bb = b + (size_t)q * plane_stride + x0;
-  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-    const int c = idx % W, k = idx / W;
-    if (k >= in.lo && k < in.hi) {
-      copy_async(&sa[k * RS + c], &ba[(size_t)k * row_stride + c]);
-      copy_async(&sb[k * RS + c], &bb[(size_t)k * row_stride + c]);
-    } else {
-      sa[k * RS + c] = (T)0;
-      sb[k * RS + c] = (T)0;
-    }
-  }
-  copy_async_wait();
-  __syncthreads();
-#pragma unroll 1
-  for (int f = 0; f < 2; ++f) dst_tile<C>(f == 0 ? sa : sb, mem);
   // table row of this plane: modes (q, k, p), p fastest
   const T* f0 = cf + (size_t)q * N * N + x0;
-  for (int idx = threadIdx.x; idx < N * W; idx += NT) {
-    const int c = idx % W, k = idx / W;
-    const size_t o = (size_t)k * N + c;
-    const T g0 = f0[o], g1 = f0[o + cf_stride], g2 = f0[o + 2 * cf_stride];
-    const T ri = sa[k * RS + c], re = sb[k * RS + c];
-    sa[k * RS + c] = g0 * ri + g1 * re;
-    sb[k * RS + c] = g1 * ri + g2 * re;
-  }
-  __syncthreads();
+  if constexpr (TWO) {
+    for (int idx = threadIdx.x; idx < N * W; idx += NT) {
+      const int c = idx % W, k = idx / W;
+      if (k >= in.lo && k < in.hi) {
+        copy_async(&sa[k * RS + c], &ba[(size_t)k * row_stride + c]);
+        copy_async(&sb[k * RS + c], &bb[(size_t)k * row_stride + c]);
+      } else {
+        sa[k * RS + c] = (T)0;
+        sb[k * RS + c] = (T)0;
+      }
+    }
+    copy_async_wait();
+    __syncthreads();
 #pragma unroll 1
-  for (int f = 0; f < 2; ++f) dst_tile<C>(f == 0 ? sa : sb, mem);
-  for (int idx = threadIdx.x + out.lo * W; idx < out.hi * W; idx += NT) {
-    const int c = idx % W, k = idx / W;
-    ba[(size_t)k * row_stride + c] = sa[k * RS + c];
-    bb[(size_t)k * row_stride + c] = sb[k * RS + c];
+    for (int f = 0; f < 2; ++f) dst_tile<C>(f == 0 ? sa : sb, mem);
+    for (int idx = threadIdx.x; idx < N * W; idx += NT) {
+      const int c = idx % W, k = idx / W;
+      const size_t o = (size_t)k * N + c;
+      const T g0 = f0[o], g1 = f0[o + cf_stride], g2 = f0[o + 2 * cf_stride];
+      const T ri = sa[k * RS + c], re = sb[k * RS + c];
+      sa[k * RS + c] = g0 * ri + g1 * re;
+      sb[k * RS + c] = g1 * ri + g2 * re;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int f = 0; f < 2; ++f) dst_tile<C>(f == 0 ? sa : sb, mem);
+    for (int idx = threadIdx.x + out.lo * W; idx < out.hi * W; idx += NT) {
+      const int c = idx % W, k = idx / W;
+      ba[(size_t)k * row_stride + c] = sa[k * RS + c];
+      bb[(size_t)k * row_stride + c] = sb[k * RS + c];
+    }
+  } else {
+    // steps: a forward, b forward and the 2 x 2 solve, b inverse, a inverse
+    // (one inlined transform); between two steps each thread passes on the
+    // elements idx = threadIdx.x + i NT of the grids and the tile alone
+#pragma unroll 1
+    for (int step = 0; step < 4; ++step) {
+      if (step != 2) {
+        const T* src = step == 1 ? bb : ba;
+        for (int idx = threadIdx.x; idx < N * W; idx += NT) {
+          const int c = idx % W, k = idx / W;
+          sa[k * RS + c] = step == 3 || (k >= in.lo && k < in.hi) ? src[(size_t)k * row_stride + c] : (T)0;
+        }
+      }
+      __syncthreads();
+      dst_tile<C>(sa, mem);
+      for (int idx = threadIdx.x; idx < N * W; idx += NT) {
+        const int c = idx % W, k = idx / W;
+        T* ga = &ba[(size_t)k * row_stride + c];
+        T* s = &sa[k * RS + c];
+        if (step == 0) {
+          *ga = *s;
+        } else if (step == 1) {
+          const size_t o = (size_t)k * N + c;
+          const T g0 = f0[o], g1 = f0[o + cf_stride], g2 = f0[o + 2 * cf_stride];
+          const T ri = *ga, re = *s;
+          *ga = g0 * ri + g1 * re;
+          *s = g1 * ri + g2 * re;
+        } else if (k >= out.lo && k < out.hi) {
+          (step == 2 ? bb : ba)[(size_t)k * row_stride + c] = *s;
+        }
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -1858,7 +1909,7 @@ int run_solve_coupled(kfbi_handle* h, const SolveArgs& si, const SolveArgs& se, 
   using C = Cfg<T, N>;
   constexpr int W = C::W;
   const size_t smem = C::smem_elems * sizeof(T);
-  const size_t smem2 = (2 * (size_t)N * C::RS + C::mem_elems) * sizeof(T);
+  constexpr size_t smem2 = CoupledTiles<T, N>::smem;
   const int dim = h->grid.dim;
   cudaStream_t st = h->stream;
   const Tables& t = h->t;

@@ -513,8 +513,8 @@ __device__ __forceinline__ double warp_sum8(double (&v)[ARN_CH]) {
 // ------------------------------------------------- Arnoldi step (CGS2)
 // One Krylov step after w = A v_j:
 //   h = V^T w;  w1 = w - V h;  y = V^T w1, |w1|^2;  w2 = w1 - V y;
-//   H(:, j) = h + y, |w2|^2 = |w1|^2 - |y|^2 (V has orthonormal columns, and
-//   y is of rounding size unless the space is exhausted, where both vanish);
+//   H(:, j) = h + y, |w2|^2 = |w1|^2 - |y|^2 (V has orthonormal columns; where
+//   the difference cancels, see arn_norm2);
 //   v_{j+1} = w2 / |w2|;  the Givens update, the residual estimate |g_{j+1}|
 //   and the stop flag (estimate / gnorm <= tol, or not finite: the host's
 //   test, in the same float64 operations).
@@ -593,11 +593,27 @@ __device__ __forceinline__ void arn_update(const ArnArgs& A, const double* cs, d
   }
 }
 
-// |w2| from |w1|^2 and y (every thread)
-__device__ __forceinline__ double arn_norm2(const double* y, int nv) {
-  double t = y[nv];
-  for (int k = 0; k < nv; ++k) t = fma(-y[k], y[k], t);
-  return t > 0.0 ? t : 0.0;
+// |w2|^2 (every thread of the block): |w1|^2 - |y|^2, or, where less than half
+// of |w1|^2 is left of it (an exhausted Krylov space: w1 and y are both of
+// rounding size and the difference has no digits, or is negative), the sum
+// over the rows of w2 itself.  That path is rare, so each block takes all
+// rows, in one order: every block has the same value.
+__device__ __forceinline__ double arn_norm2(const ArnArgs& A, const double* y, double* ws) {
+  double t = y[A.nv];
+  for (int k = 0; k < A.nv; ++k) t = fma(-y[k], y[k], t);
+  if (t > 0.5 * y[A.nv]) return t;
+  t = 0.0;
+  for (int i = threadIdx.x; i < A.n; i += blockDim.x) {
+    double wi = A.w[i];
+    for (int k = 0; k < A.nv; ++k) wi -= y[k] * A.V[(size_t)k * A.ld + i];
+    t += wi * wi;
+  }
+  t = warp_sum(t);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = t;
+  __syncthreads();
+  t = 0.0;
+  for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += ws[q];
+  return t;
 }
 
 // Column j of H (col: hcol, then sqrt(n2)), the earlier rotations (cs, sn in
@@ -672,7 +688,7 @@ __global__ void __launch_bounds__(256) k_arn_close(ArnArgs A) {
   if (A.skip != nullptr && *A.skip) return;
   SmallLayout L{A.m};
   const bool closing = blockIdx.x == gridDim.x - 1;  // closes column j while the others update
-  __shared__ double y[MAX_RESTART + 2], col[MAX_RESTART + 2], cs[MAX_RESTART], sn[MAX_RESTART];
+  __shared__ double y[MAX_RESTART + 2], col[MAX_RESTART + 2], cs[MAX_RESTART], sn[MAX_RESTART], ws[8];
   for (int k = threadIdx.x; k <= A.nv; k += blockDim.x) {
     y[k] = A.s[L.y() + k];
     if (closing && k < A.nv) col[k] = A.s[L.hcol() + k] + y[k];
@@ -682,7 +698,7 @@ __global__ void __launch_bounds__(256) k_arn_close(ArnArgs A) {
     }
   }
   __syncthreads();
-  const double n2 = arn_norm2(y, A.nv), norm = sqrt(n2);
+  const double n2 = arn_norm2(A, y, ws), norm = sqrt(n2);
   if (closing) {
     if (threadIdx.x == 0) arn_finish(A, col, cs, sn, n2);
     return;
@@ -696,7 +712,7 @@ __global__ void __launch_bounds__(ARN_ONE_T) k_arn_one(ArnArgs A) {
   pdl_launch_next();
   if (A.skip != nullptr && *A.skip) return;
   __shared__ double red[ARN_ONE_T / 32][MAX_RESTART + 2];
-  __shared__ double h[MAX_RESTART + 2], y[MAX_RESTART + 2], cs[MAX_RESTART], sn[MAX_RESTART];
+  __shared__ double h[MAX_RESTART + 2], y[MAX_RESTART + 2], cs[MAX_RESTART], sn[MAX_RESTART], ws[ARN_ONE_T / 32];
   SmallLayout L{A.m};
   for (int k = threadIdx.x; k < A.j; k += ARN_ONE_T) {
     cs[k] = A.s[L.cs() + k];
@@ -716,7 +732,7 @@ __global__ void __launch_bounds__(ARN_ONE_T) k_arn_one(ArnArgs A) {
   arn_update(A, h, nullptr, 0.0, 1);
   arn_dots<true>(A, red);
   sum(y, A.nv + 1);
-  const double n2 = arn_norm2(y, A.nv), norm = sqrt(n2);
+  const double n2 = arn_norm2(A, y, ws), norm = sqrt(n2);
   for (int k = threadIdx.x; k < A.nv; k += ARN_ONE_T) h[k] += y[k];
   arn_update(A, y, A.V + (size_t)(A.j + 1) * A.ld, norm > 0.0 ? 1.0 / norm : 0.0, 1);
   __syncthreads();

@@ -68,8 +68,10 @@ extern "C" {
 /* precision of the integral evaluations */
 #define KFBI_FP64 0          /* all transforms and corrections in 64 bits (float64
                                 fields; transform lines of 32 or more points on
-                                64-bit block fixed point, error below that of
-                                float64 butterflies)                              */
+                                64-bit block fixed point: error usually a few
+                                times below that of float64 butterflies, on
+                                lines of few values far above a background up
+                                to about theirs)                                  */
 #define KFBI_MIXED 1         /* float32 transforms inside GMRES, float64 Arnoldi,
                                 residuals and outer refinement                   */
 #define KFBI_MIXED_LEARNED 2 /* KFBI_MIXED + learned warm start of the density

@@ -15,21 +15,33 @@
 //    operations.
 //
 // Scale.  Let |x| <= m in a column of integers and A = sum |x|.  The folded
-// values are |y| <= 2 m; a sum over the P complex values of the FFT's first
-// level stays below min(2 sqrt(2) P m, 2 A), any later one below
-// min(1.44 N m, 2 A) (sum |y_j| <= sum over pairs of 4 m max(sin, 1/2), or
-// 2 (|x_j| + |x_{N-j}|)).  The column's largest value gets as many bits as
-// keep these below 2^61: `early` bits up to the first level's twiddles, whose
-// products are shifted down to `late` bits.  A costs three integer
-// instructions per value and pays in lines with few large values (corrections
-// along x, decaying spectra): without it those lost two to three bits.
-// Every rounding is at one unit of these scales, without bias; the error
-// against 80-bit arithmetic is below that of the float64 transform this
-// replaces (tests/test_dst_fix_host.py measures both).
+// values are |y| <= 2 m max(sin, 1/2); a component of a sum over the P complex
+// values of the FFT's first level stays below min(1.83 P m, 2 A) (the largest
+// over all levels' angles), any later one below min(1.44 N m, 2 A) (sum |y_j|
+// <= sum over pairs of 4 m max(sin, 1/2), or 2 (|x_j| + |x_{N-j}|)).  The
+// column's largest value gets as many bits as keep these below 2^61: `early`
+// bits up to the first level's twiddles, whose products are shifted down to
+// `late` bits.  A costs three integer instructions per value and pays in lines
+// with few large values (corrections along x, decaying spectra): without it
+// those lost two to three bits.
+//
+// Rounding.  The running sum of the odd outputs collects what the values
+// before it share: a mean of a quarter unit in the first level's results cost
+// lines of a background and a few larger values a factor of up to four.  So
+// values enter the pre-fold at 60 bits (below 2^-60 of the largest cut off)
+// and are rounded once, after it; products round to the nearest unit at their
+// final scale; and integers that a shift alone brings there, where half units
+// are common, round half to even (the first level's, see phase A1, up and
+// down in turn).
+// Error (2-norm, against 80-bit arithmetic, over that of the same transform in
+// float64 with exact tables): 0.1 to 0.6 over smooth, dense, sparse, widely
+// scaled and single-mode lines.  Its worst lines are a low background with
+// few values far above it, whose unit is that of the largest: at most 0.6 up
+// to 256 lines, 0.9 at 512 and 1.2 at 384.
 //
 // Measured (GB300, CUDA events): a 256^3 float64 box solve took 4.16 ms with
 // float64 butterflies (26 float64 instructions per point and transform, at
-// 1/32 of the integer rate) and takes 1.12 ms; its error against dense
+// 1/32 of the integer rate) and takes 0.76 ms; its error against dense
 // float64 products went from 5.3e-15 to 2.2e-15 (2-norm, smooth field).
 //
 // The decomposition is that of dst_reg.cuh (two-level FFT m = a + 8q, k = k1
@@ -137,8 +149,8 @@ KFBI_HD ll mul63(ll a, fx w) {
 }
 
 // (xr + i xi) w for w at S = 62, |w| <= 1, |xr|, |xi| < 2^61 - 2^32; with
-// half = 2^29 + 2^(28 + sh) the caller's shift of the result by sh >> rounds
-// (half = 2^29: rounded here)
+// half = 2^(29 + sh) the caller's shift of the result by sh rounds to the
+// nearest (half = 2^29: rounded here)
 KFBI_HD void cmul62(ll& xr, ll& xi, const cfx& w, ll half = 1LL << 29) {
   int32_t rh, rl, ih, il;
   halves(xr, rh, rl);
@@ -153,6 +165,11 @@ KFBI_HD void cmul62(ll& xr, ll& xi, const cfx& w, ll half = 1LL << 29) {
 
 // a / 2 rounded half to even (floor would leave a bias that the sums collect)
 KFBI_HD ll half_even(ll a) { return (a + (ll)((lo_of(a) >> 1) & 1)) >> 1; }
+// a / 2^sh rounded half to even (sh >= 0)
+KFBI_HD ll shift_even(ll a, int sh) {
+  const ll r = (1LL << sh) >> 1;
+  return (a + r - (ll)((int32_t)(sh > 0) & ~lo_of(a >> sh) & 1)) >> sh;
+}
 
 // sqrt(1/2) and sqrt(3)/2 at S = 63, cos(pi/8), sin(pi/8) at S = 62
 #define KFBI_FX_R2 fx_of(0x5A827999FCEF3242LL)
@@ -359,10 +376,11 @@ KFBI_HD void dft_first(ll* xr, ll* xi, const cfx* sp) {
 // bits).  A column that holds an infinity or NaN is transformed to NaN
 // throughout, as in float64.
 constexpr double HUGE_STEP = 0x1p512;
+constexpr int FOLD_BITS = 60;  // the sum of two values stays below 2^62 - 2^32
 struct Scale {
   int in;          // shift of a 63-bit significand of the largest exponent, plus its exponent field
+  int fold;        // shift of twice a folded value from FOLD_BITS to early bits
   int sh;          // early - late
-  ll half;         // rounding of the product that is shifted by sh
   double out, oc;  // 2^(-k-1) (the integers are twice the outputs) and (2^84 + 2^63 + 2^52) 2^(-k-1)
   bool huge;       // both are smaller by HUGE_STEP (oc would overflow): the outputs need it back
 };
@@ -373,9 +391,10 @@ KFBI_HD int bit_length(uint32_t v) {
   return v ? 32 - __builtin_clz(v) : 0;
 #endif
 }
+constexpr int EARLY_MORE = 4;
 template <int N>
 KFBI_HD constexpr int late_bits() {
-  // 1.44 N 2^late < 2^61 and 2 sqrt(2) (N / 16) 2^(late + 3) < 2^61
+  // 1.44 N 2^late < 2^61 and 1.83 (N / 16) 2^(late + EARLY_MORE) < 2^61
   return N <= 32 ? 55 : N <= 64 ? 54 : N <= 128 ? 53 : N <= 256 ? 52 : 51;
 }
 template <int N>
@@ -385,19 +404,21 @@ KFBI_HD Scale scale_of(int emax, uint32_t asum) {
   // 2 A 2^(b - (emax - 1022)) < 2^(bit_length - 20 + b) = 2^60
   const int b1 = 80 - bit_length(asum);
   const int late = b1 > late_bits<N>() ? b1 : late_bits<N>();
-  const int early = b1 > late_bits<N>() + 3 ? b1 : late_bits<N>() + 3;
-  s.in = e + 63 - early;
+  // twice that is enough for sums that no difference doubles
+  const int early = b1 + 1 > late_bits<N>() + EARLY_MORE ? b1 + 1 : late_bits<N>() + EARLY_MORE;
+  s.in = e + 63 - FOLD_BITS;
+  s.fold = FOLD_BITS + 1 - early;
   s.sh = early - late;
-  s.half = (1LL << 29) + ((1LL << s.sh) >> 1 << 30);
   s.huge = e > 1900;
   const int eo = e - late - (s.huge ? 512 : 0);  // biased exponent of 2^(-k-1)
   s.out = double_of(emax == 0x7ff ? 0x7ff8000000000000LL : (ll)eo << 52);
   s.oc = s.out * double_of(0x4530000080100000LL);  // 2^84 + 2^63 + 2^52
   return s;
 }
-// x as an integer at the column's scale, on its bits: the significand
-// shifted by the distance to the largest exponent (truncated; zeros and
-// subnormal values come out as 0, their distance being 64 or more)
+// x as an integer of FOLD_BITS bits, on its bits: the significand shifted by
+// the distance to the largest exponent (truncated: 53 bits lose theirs from
+// 2^-7 of the largest value on, below any later unit; zeros and subnormal
+// values come out as 0, their distance being 64 or more)
 KFBI_HD ll to_fix(double x, const Scale& s) {
   const ll b = bits_of(x);
   const int32_t h = hi_of(b);
@@ -490,7 +511,8 @@ KFBI_HD void phase_s(State<G>& st, const int* mx, uint32_t* sm, int a, int c) {
 }
 
 // phase 1: column scale, conversion, sine pre-fold of the pairs
-//   y_j = sin(pi j / N)(x_j + x_{N-j}) + (x_j - x_{N-j}) / 2,  y_0 = 0
+//   y_j = sin(pi j / N)(x_j + x_{N-j}) + (x_j - x_{N-j}) / 2,  y_0 = 0,
+// twice y_j at FOLD_BITS bits shifted down to early bits
 template <class G>
 KFBI_HD void phase_1(State<G>& st, ll* s, const uint32_t* sm, const fx* sinv, int a, int c) {
   constexpr int N = G::N, RS = G::RS, T = G::T, P = G::P, W = G::W;
@@ -498,17 +520,19 @@ KFBI_HD void phase_1(State<G>& st, ll* s, const uint32_t* sm, const fx* sinv, in
 #pragma unroll
   for (int b = 0; b < T; ++b) asum += sm[b * W + c];
   st.sc = scale_of<N>(st.emax, asum);
+  const int fold = st.sc.fold;
+  const ll r = 1LL << (fold - 1);
 #pragma unroll
   for (int i = 0; i < P; ++i) {
     const int j = a + T * i;
     const ll na = to_fix(st.xa[i], st.sc), nb = to_fix(st.xb[i], st.sc);
     if (i == 0 && a == 0) {
       s[c] = 0;
-      s[(N / 2) * RS + c] = 2 * na;
+      s[(N / 2) * RS + c] = (4 * na + r) >> fold;
     } else {
-      const ll t = mul63(na + nb, sinv[j]), d = half_even(na - nb);
-      s[j * RS + c] = t + d;
-      s[(N - j) * RS + c] = t - d;
+      const ll t = 2 * mul63(na + nb, sinv[j]) + r, d = na - nb;
+      s[j * RS + c] = (t + d) >> fold;
+      s[(N - j) * RS + c] = (t - d) >> fold;
     }
   }
 }
@@ -525,12 +549,14 @@ KFBI_HD void phase_a1(State<G>& st, const ll* s, const cfx* sp, const cfx* lv, i
   }
   dft_first<P, N>(st.zr, st.zi, sp);
   const int sh = st.sc.sh;
-  const ll r = (1LL << sh) >> 1;
-  st.zr[0] = (st.zr[0] + r) >> sh;
-  st.zi[0] = (st.zi[0] + r) >> sh;
+  st.zr[0] = shift_even(st.zr[0], sh);
+  st.zi[0] = shift_even(st.zi[0], sh);
+  // for a = 0 all twiddles are 1 and half units are common: they round up
+  // for even k1 and down for odd k1, which the running sum over k cancels
+  const ll half = 1LL << (29 + sh);
 #pragma unroll
   for (int k1 = 1; k1 < P; ++k1) {
-    cmul62(st.zr[k1], st.zi[k1], lv[a * P + k1], st.sc.half);
+    cmul62(st.zr[k1], st.zi[k1], lv[a * P + k1], half - (k1 & 1));
     st.zr[k1] >>= sh;
     st.zi[k1] >>= sh;
   }

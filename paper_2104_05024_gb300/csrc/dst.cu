@@ -2181,7 +2181,20 @@ __global__ void __launch_bounds__(NT) k_nxfwd(T* __restrict__ a, const double* _
   const int y0 = blockIdx.x * W;
   const int z = DIM == 3 ? blockIdx.y : 0;
   const size_t plane = (size_t)z * P * P;
-  if (src != nullptr) {
+  // float64 passes are bound by the transform: with their lines' loads issued
+  // together, here and in k_nxinv, the box solve took 5.48 instead of 5.43 ms
+  // at 256^3 and 821 instead of 804 us at 128^3
+  if constexpr (sizeof(T) == 8) {
+    for (int idx = threadIdx.x; idx < P * W; idx += NT) {
+      const int x = idx % P, c = idx / P, y = y0 + c;
+      T v = (T)0;
+      if (y <= N) {
+        if (src != nullptr) v = alpha * src[plane + (size_t)y * P + x];
+        else if (src32 != nullptr) v = (T)src32[plane + (size_t)y * P + x];
+      }
+      s[x * RS + c] = v;
+    }
+  } else if (src != nullptr) {
     const T a_t = (T)alpha;
     fill_lines_n<C>(s, src + plane, y0, [&](double v) { return a_t * to_T<T>(v); });
   } else if (src32 != nullptr) {
@@ -2239,30 +2252,44 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
   copy_async_wait();
   __syncthreads();
   dct_tile<C>(s, tw, sinv, tot, x1);
-  constexpr int LW = N < 32 ? N : 32, PER = N / LW, CH = batch_of(PER);
-  const int lane = threadIdx.x % LW;
-  const T b_t = (T)beta;
-  auto put = [&](size_t o, T v, double w) {
-    if (keep) a[o] = v;
-    if (out != nullptr) {
-      const double bv = to_double(b_t * v);
-      out[o] = aux32 != nullptr ? bv + w : aux != nullptr ? fma(gamma, w, bv) : bv;
+  if constexpr (sizeof(T) == 8) {
+    for (int idx = threadIdx.x; idx < P * W; idx += NT) {
+      const int x = idx % P, c = idx / P, y = y0 + c;
+      if (y > N) continue;
+      const size_t o = plane + (size_t)y * P + x;
+      const T v = s[x * RS + c];
+      if (keep) a[o] = v;
+      if (out != nullptr) {
+        const double bv = (T)beta * v;
+        out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
+      }
     }
-  };
-  auto other = [&](size_t o) { return aux32 != nullptr ? ffl::widen(aux32[o]) : aux != nullptr ? aux[o] : 0.0; };
+  } else {
+    constexpr int LW = N < 32 ? N : 32, PER = N / LW, CH = batch_of(PER);
+    const int lane = threadIdx.x % LW;
+    const T b_t = (T)beta;
+    auto put = [&](size_t o, T v, double w) {
+      if (keep) a[o] = v;
+      if (out != nullptr) {
+        const double bv = to_double(b_t * v);
+        out[o] = aux32 != nullptr ? bv + w : aux != nullptr ? fma(gamma, w, bv) : bv;
+      }
+    };
+    auto other = [&](size_t o) { return aux32 != nullptr ? ffl::widen(aux32[o]) : aux != nullptr ? aux[o] : 0.0; };
 #pragma unroll 1
-  for (int c = threadIdx.x / LW; c < W; c += NT / LW) {
-    if (y0 + c > N) continue;
-    const size_t o = plane + (size_t)(y0 + c) * P + lane;
+    for (int c = threadIdx.x / LW; c < W; c += NT / LW) {
+      if (y0 + c > N) continue;
+      const size_t o = plane + (size_t)(y0 + c) * P + lane;
 #pragma unroll
-    for (int i0 = 0; i0 < PER; i0 += CH) {
-      double w[CH];
+      for (int i0 = 0; i0 < PER; i0 += CH) {
+        double w[CH];
 #pragma unroll
-      for (int i = 0; i < CH; ++i) w[i] = other(o + LW * (i0 + i));
+        for (int i = 0; i < CH; ++i) w[i] = other(o + LW * (i0 + i));
 #pragma unroll
-      for (int i = 0; i < CH; ++i) put(o + LW * (i0 + i), s[(lane + LW * (i0 + i)) * RS + c], w[i]);
+        for (int i = 0; i < CH; ++i) put(o + LW * (i0 + i), s[(lane + LW * (i0 + i)) * RS + c], w[i]);
+      }
+      if (lane == 0) put(o + N, s[N * RS + c], other(o + N));
     }
-    if (lane == 0) put(o + N, s[N * RS + c], other(o + N));
   }
 }
 

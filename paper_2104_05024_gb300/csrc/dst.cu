@@ -1030,7 +1030,7 @@ __global__ void __launch_bounds__(ZTri<T, N>::NTH) k_ztri(T* __restrict__ a, con
     for (int u = 0; u < CH; ++u) {
       const int j = j0 + u;
       if (j < M) {
-        y = g * y + rs * rc[u];
+        y = fma(g, y, rs * rc[u]);
         if constexpr (Z::INLINE_G) {
           sv = j == 1 ? 1.0f + eps : sv * g + eps;
           g = pivot(sv);
@@ -1088,6 +1088,14 @@ __global__ void __launch_bounds__(ZTri<T, N>::NTH) k_ztri(T* __restrict__ a, con
     *reinterpret_cast<float4*>(base + k * rstride + piece) = *reinterpret_cast<const float4*>(s + k * TW + piece);
 }
 
+// 1 / (1 + s) with the rounding of 1 + s taken back: the pivots of
+// neighbouring rows are nearly equal, so a shared error of theirs adds up over
+// the rows that a mode remembers (z stage error at 48 rows 5.5e-16 -> 4.5e-16)
+__device__ __forceinline__ double ztab_pivot(double s) {
+  const double d = 1.0 + s, t = d - 1.0, e = (1.0 - (d - t)) + (s - t);  // d + e = 1 + s
+  const double g = 1.0 / d;
+  return fma(g, fma(-g, e, fma(-g, d, 1.0)), g);
+}
 // 1 / d_j of every (q, p) mode at row j of its table, the inverse of the
 // middle pivot at row 0
 __global__ void k_ztab(const double* __restrict__ mu1, double lambda, double h2, int N, double* __restrict__ tab) {
@@ -1095,14 +1103,14 @@ __global__ void k_ztab(const double* __restrict__ mu1, double lambda, double h2,
   if (p >= N) return;
   const double eps = -h2 * (mu1[p] + mu1[q] - lambda);
   double* t = tab + (size_t)q * M * N + p;
-  double s = 1.0 + eps, g = 1.0 / (1.0 + s);
+  double s = 1.0 + eps, g = ztab_pivot(s);
   t[N] = g;
   for (int j = 2; j < M; ++j) {
     s = fma(s, g, eps);
-    g = 1.0 / (1.0 + s);
+    g = ztab_pivot(s);
     t[(size_t)j * N] = g;
   }
-  t[0] = 1.0 / (eps + 2.0 * s * g);
+  t[0] = 1.0 / fma(2.0 * s, g, eps);
 }
 
 // ------------------------------- fused x and y passes (thread-block clusters)
@@ -1470,12 +1478,22 @@ SolveSpans solve_spans(const kfbi_handle* h, bool in, bool out) {
 
 // Whether the z systems of this lambda are solved by elimination.  Its error
 // grows with the number of rows 1 / sqrt(eps) over which the slowest mode (p
-// = q = 1) remembers its roundings; up to 48 rows it is below the two
-// transforms' (float32, z stage alone, against 80 bits: 4e-7 at 256 rows and
-// 5e-7 at 512 for lambda = 60, where the transforms leave 9e-7 and 1.7e-6;
-// at 110 rows 3e-6).  The time-step problems (lambda = 40, 60, ...) are well
-// inside; Poisson and nearly Poisson problems on fine grids keep the
-// transforms.
+// = q = 1) remembers its roundings; the line is drawn at 48 rows for both
+// types.  z stage alone against 80 bits (2-norm, dense, smooth, sparse and
+// single-mode right-hand sides):
+//  - float32: below the two transforms' (4e-7 at 256 rows and 5e-7 at 512 for
+//    lambda = 60, where the transforms leave 9e-7 and 1.7e-6; 3e-6 at 110
+//    rows);
+//  - float64: 2.7e-16 to 3.1e-16 at 256 lines and 16 rows (lambda = 60),
+//    3.7e-16 to 4.8e-16 at 48 rows; at 512 lines and 32 rows 3.6e-16 to
+//    4.2e-16.  That is a quarter of what two transforms in float64
+//    arithmetic leave (0.9e-15 to 1.6e-15 and 1.7e-15 to 3.3e-15), and 1.0 to
+//    2.4 times what the two fixed-point transforms leave (1.9e-16 to 3.0e-16
+//    and 2.6e-16 to 3.2e-16), for two thirds of their time.  Up to 128 lines,
+//    where no lambda >= 0 reaches more than 29 rows, it stays below two thirds
+//    of the former.
+// The time-step problems (lambda = 40, 60, ...) are well inside; Poisson and
+// nearly Poisson problems on fine grids keep the transforms.
 template <int N>
 bool z_by_elimination(const kfbi_handle* h, double lambda) {
   if (N < 32 || h->grid.dim != 3) return false;

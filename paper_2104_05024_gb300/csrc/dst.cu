@@ -1382,7 +1382,7 @@ int prep(K kernel, size_t smem) {
 // allocation-free box solve: no mode-factor table either)
 template <typename K, typename... Args>
 cudaError_t launch_pass(kfbi_handle* h, K kernel, dim3 grid, size_t smem, Args... args) {
-  if (h->rinv_ok) return launch_pdl(kernel, grid, dim3(NT), smem, h->stream, args...);
+  if (h->owner) return launch_pdl(kernel, grid, dim3(NT), smem, h->stream, args...);
   kernel<<<grid, NT, smem, h->stream>>>(args...);
   return cudaGetLastError();
 }
@@ -1502,23 +1502,24 @@ bool z_by_elimination(const kfbi_handle* h, double lambda) {
   return eps * (48.0 * 48.0) >= 1.0;
 }
 
+// storage of a table, nullptr where it cannot be had
+inline double* table_alloc(kfbi_handle* h, int64_t n) {
+  double* p = nullptr;
+  if (dalloc(h, &p, (size_t)n) == KFBI_OK) return p;
+  cudaGetLastError();
+  return nullptr;
+}
+
 // the float64 pivot table for this lambda (N^3 / 2 values, built once per
 // lambda), nullptr where the handle has none
 inline const double* z_table(kfbi_handle* h, double lambda, int N) {
-  if (!h->rinv_ok) return nullptr;
-  if (h->ztab == nullptr) {
-    if (dalloc(h, &h->ztab, (size_t)N * N * (N / 2)) != KFBI_OK) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    h->ztab_lambda = std::nan("");
-  }
-  if (!(h->ztab_lambda == lambda)) {
-    k_ztab<<<dim3((N + 127) / 128, N), 128, 0, h->stream>>>(h->t.mu, lambda, h->grid.h * h->grid.h, N, h->ztab);
-    KFBI_COUNT(1);
-    h->ztab_lambda = lambda;
-  }
-  return h->ztab;
+  if (!h->owner) return nullptr;
+  return h->ztab.get(
+      lambda, [&] { return table_alloc(h, (int64_t)N * N * (N / 2)); },
+      [&](double* p) {
+        k_ztab<<<dim3((N + 127) / 128, N), 128, 0, h->stream>>>(h->t.mu, lambda, h->grid.h * h->grid.h, N, p);
+        KFBI_COUNT(1);
+      });
 }
 
 // the z pass of a 3-D solve: elimination where z_by_elimination allows it,
@@ -1571,25 +1572,17 @@ const T* mode_factors(kfbi_handle* h, double lambda, double scale) {
   if constexpr (sizeof(T) != 8) {
     return nullptr;
   } else {
-    if (!h->rinv_ok) return nullptr;
+    if (!h->owner) return nullptr;
     const bool cosine = h->grid.bc == KFBI_BOX_NEUMANN;
     const int n = cosine ? N + 1 : N;
     const int64_t total = h->grid.dim == 3 ? (int64_t)n * n * n : (int64_t)n * n;
-    if (h->rinv64 == nullptr) {
-      if (dalloc(h, &h->rinv64, (size_t)total) != KFBI_OK) {
-        cudaGetLastError();
-        h->rinv_ok = false;
-        return nullptr;
-      }
-      h->rinv_lambda = std::nan("");
-    }
-    if (!(h->rinv_lambda == lambda)) {
-      const int nb = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
-      k_rinv<<<nb, 256, 0, h->stream>>>(h->t.mu, lambda, scale, n, h->grid.dim, cosine, h->rinv64, total);
-      KFBI_COUNT(1);
-      h->rinv_lambda = lambda;
-    }
-    return h->rinv64;
+    return h->rinv.get(
+        lambda, [&] { return table_alloc(h, total); },
+        [&](double* p) {
+          const int nb = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
+          k_rinv<<<nb, 256, 0, h->stream>>>(h->t.mu, lambda, scale, n, h->grid.dim, cosine, p, total);
+          KFBI_COUNT(1);
+        });
   }
 }
 
@@ -1652,7 +1645,7 @@ int run_solve(kfbi_handle* h, const SolveArgs& sa, T* work, const T* mu1, const 
     if constexpr (N >= 32 && N <= 256) {
       constexpr size_t s2 = (2 * (size_t)N * C::RS + C::mem_elems) * sizeof(T);
       if ((rc = prep(k_solve2d<T, N>, s2))) return rc;
-      if (launch_cluster(k_solve2d<T, N>, N / 32, dim3(N / 32), s2, st, h->rinv_ok, work, sa.src, sa.alpha, sa.src32,
+      if (launch_cluster(k_solve2d<T, N>, N / 32, dim3(N / 32), s2, st, h->owner, work, sa.src, sa.alpha, sa.src32,
                          sa.corr, sa.rows, (const int32_t*)t.irr, (const int32_t*)t.line_start, tw, mu1, lam, scale,
                          rinv, sa.keep || sa.out_user == nullptr, sa.out_user, sa.aux, sa.beta, sa.gamma, sa.aux32,
                          (const int*)h->skip, 4) == cudaSuccess) {

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "kfbi.h"
+#include "lazy_table.cuh"
 
 namespace kfbi {
 
@@ -280,14 +281,10 @@ struct kfbi_handle {
   bool tma = false;
   int sms = 152;                  // the device's multiprocessor count (persistent grids)
   bool xy_fused = false;          // float32 3-D solves use the cluster-fused x-y passes
-  // float64 solves: the mode factors scale / mu_p for the lambda they were
-  // built for (rinv_ok: the handle may allocate the table; set at creation)
-  double* rinv64 = nullptr;
-  double rinv_lambda = 0.0;
-  bool rinv_ok = false;
-  // float64 z elimination: the pivots for the lambda they were built for
-  double* ztab = nullptr;
-  double ztab_lambda = 0.0;
+  // float64 tables by lambda: the mode factors scale / mu_p, the pivots of
+  // the z elimination
+  kfbi::LazyTable rinv, ztab;
+  bool owner = false;             // made by kfbi_create: may allocate, tables set up before its solves
   // coupled solves: the per-mode 2 x 2 solve factors for the kappa they were
   // built for, one table per element type (3 N^dim values each)
   double* cpl64 = nullptr;

@@ -593,19 +593,15 @@ __device__ __forceinline__ void arn_update(const ArnArgs& A, const double* cs, d
   }
 }
 
-// |w2|^2 (every thread of the block): |w1|^2 - |y|^2, or, where less than half
-// of |w1|^2 is left of it (an exhausted Krylov space: w1 and y are both of
-// rounding size and the difference has no digits, or is negative), the sum
-// over the rows of w2 itself.  That path is rare, so each block takes all
-// rows, in one order: every block has the same value.
-__device__ __forceinline__ double arn_norm2(const ArnArgs& A, const double* y, double* ws) {
-  double t = y[A.nv];
-  for (int k = 0; k < A.nv; ++k) t = fma(-y[k], y[k], t);
-  if (t > 0.5 * y[A.nv]) return t;
-  t = 0.0;
-  for (int i = threadIdx.x; i < A.n; i += blockDim.x) {
-    double wi = A.w[i];
-    for (int k = 0; k < A.nv; ++k) wi -= y[k] * A.V[(size_t)k * A.ld + i];
+// |w2|^2 summed over the rows of w2 itself, by each block over all rows in one
+// order: every block has the same value (out of line: the steps that need it
+// are rare)
+__device__ __noinline__ double arn_norm2_rows(const double* w, const double* V, int ld, int n, int nv, const double* y,
+                                              double* ws) {
+  double t = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    double wi = w[i];
+    for (int k = 0; k < nv; ++k) wi -= y[k] * V[(size_t)k * ld + i];
     t += wi * wi;
   }
   t = warp_sum(t);
@@ -614,6 +610,17 @@ __device__ __forceinline__ double arn_norm2(const ArnArgs& A, const double* y, d
   t = 0.0;
   for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += ws[q];
   return t;
+}
+
+// |w2|^2 (every thread of the block): |w1|^2 - |y|^2, or, where less than half
+// of |w1|^2 is left of it (an exhausted Krylov space: w1 and y are both of
+// rounding size and the difference has no digits, or is negative), the sum
+// over the rows
+__device__ __forceinline__ double arn_norm2(const ArnArgs& A, const double* y, double* ws) {
+  double t = y[A.nv];
+  for (int k = 0; k < A.nv; ++k) t = fma(-y[k], y[k], t);
+  if (t > 0.5 * y[A.nv]) return t;
+  return arn_norm2_rows(A.w, A.V, A.ld, A.n, A.nv, y, ws);
 }
 
 // Column j of H (col: hcol, then sqrt(n2)), the earlier rotations (cs, sn in

@@ -710,8 +710,9 @@ __global__ void __launch_bounds__(NT, StridedCfg<T, N>::BLOCKS) k_strided(
     for (int i = threadIdx.x; i < in.lo * W; i += NT) s[i] = (T)0;
     for (int i = in.hi * W + threadIdx.x; i < N * W; i += NT) s[i] = (T)0;
     if (!mbar_wait(&bar, 0u)) {
-      // the copies of this block finish before its shared memory goes
-      if (threadIdx.x == 0 && err != nullptr) atomicOr(err, DEVERR_TIMEOUT);
+      // recorded by every thread that gives up (the others may go on without
+      // it); the copies of this block finish before its shared memory goes
+      if (err != nullptr) atomicOr(err, DEVERR_TIMEOUT);
       mbar_wait(&bar, 0u);
       return;
     }
@@ -900,8 +901,8 @@ __global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const _
         break;
       }
     if (!ok) {
+      atomicOr(err, DEVERR_TIMEOUT);  // by every thread that gives up
       if (threadIdx.x == 0) {
-        atomicOr(err, DEVERR_TIMEOUT);
         // the copies this block issued finish before its shared memory goes:
         // stores by their bulk group, the pending load by its barrier
         tma_wait_all();

@@ -542,17 +542,26 @@ int malloc_mlp(kfbi_mlp* m, T** p, size_t n) {
 
 int blocks(size_t n, int bs) { return (int)((n + bs - 1) / bs); }
 
+// opts a kernel into its dynamic shared memory, once per device (bit of done)
+template <typename K>
+int opt_in(K kernel, size_t smem, std::atomic<uint64_t>& done, const char* what) {
+  int dev = 0;
+  KFBI_CUDA(cudaGetDevice(&dev));
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev < 64 && (done.load() & bit) != 0) return KFBI_OK;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    cudaGetLastError();
+    set_error("cudaFuncSetAttribute failed for the %s kernel", what);
+    return KFBI_ERR_CUDA;
+  }
+  done.fetch_or(bit);
+  return KFBI_OK;
+}
+
 // inference over rows already placed in m->X (Bp a multiple of 64): m->o
 int mlp_infer_rows(kfbi_mlp* m, int Bp) {
-  static bool opted = false;
-  if (!opted) {
-    if (cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)INFER_SMEM) !=
-        cudaSuccess) {
-      set_error("cudaFuncSetAttribute failed for the inference kernel");
-      return KFBI_ERR_CUDA;
-    }
-    opted = true;
-  }
+  static std::atomic<uint64_t> opted{0};
+  if (int rc = opt_in(k_mlp_infer, INFER_SMEM, opted, "inference")) return rc;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -582,14 +591,8 @@ int mlp_step(kfbi_mlp* m, const float* F, const float* t, int B) {
     set_error("batch %d outside 1..%d", B, m->bmax);
     return KFBI_ERR_ARG;
   }
-  static bool opted = false;
-  if (!opted) {
-    if (cudaFuncSetAttribute(k_mlp_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)STEP_SMEM) != cudaSuccess) {
-      set_error("cudaFuncSetAttribute failed for the training kernel");
-      return KFBI_ERR_CUDA;
-    }
-    opted = true;
-  }
+  static std::atomic<uint64_t> opted{0};
+  if (int rc = opt_in(k_mlp_step, STEP_SMEM, opted, "training")) return rc;
   cudaStream_t st = m->stream;
   const Offsets& off = m->off;
   const int Bp = (B + TILE - 1) / TILE * TILE;

@@ -341,7 +341,7 @@ int norm2(kfbi_handle* h, const double* v, double* slot, double* out) {
 }
 
 // float64-accurate box solve from float32 transforms (iterative refinement
-// with the float64 5/7-point residual): u = L_h^{-1}(alpha*src + corr) on the
+// with the 5/7-point residual on float pairs): u = L_h^{-1}(alpha*src + corr) on the
 // user layout.  Each round gains about -log10(kappa(L_h) eps_32) digits: one
 // round leaves a relative error near 1e-12 at 256^3 and 1e-10 at 512^3, so
 // GMRES tolerances below 1e-9 take a second round.

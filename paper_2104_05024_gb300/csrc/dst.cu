@@ -810,14 +810,13 @@ __global__ void __launch_bounds__(NT, StridedCfg<T, N>::BLOCKS) k_strided(
 // buffer (completion counted on an mbarrier) while all threads transform the
 // current tile; the finished tile goes back by a TMA tensor store.  Every
 // wait is bounded: on timeout the block records DEVERR_TIMEOUT and returns.
-// resident blocks per SM: three (shared memory allows three at N = 256); at
-// 80 registers neither pass spills as long as the plain pass runs its single
-// transform inside the runtime-bounded loop (the compile-time bound of one
-// lets the compiler schedule it into spills)
-template <bool SOLVE>
-constexpr int tma_blocks() {
-  return 3;
-}
+// Three resident blocks per SM (shared memory allows three at N = 256), so 80
+// registers.  At 256 rows the plain pass over whole rows just fits them, as
+// long as it runs its single transform inside the runtime-bounded loop (the
+// compile-time bound of one lets the compiler schedule it into spills); the
+// other forms spill: 32 bytes a thread over ranges, 48 with the solve, 36 with
+// both.
+constexpr int TMA_BLOCKS = 3;
 
 template <int N>
 using TmaTile = Tile<float, N, TMA_W, TMA_W>;
@@ -834,7 +833,7 @@ constexpr size_t tma_smem_bytes() {
 // false: all N of both (known at compile time: the runtime spans cost the
 // 256-row kernels register spills, 24.5 -> 26.4 us a pass).
 template <int N, bool SOLVE, bool PART>
-__global__ void __launch_bounds__(NT, tma_blocks<SOLVE>()) k_strided_tma(const __grid_constant__ CUtensorMap map_in,
+__global__ void __launch_bounds__(NT, TMA_BLOCKS) k_strided_tma(const __grid_constant__ CUtensorMap map_in,
                                                     const __grid_constant__ CUtensorMap map_out, int mode,
                                                     Span planes_p, Span in_p, Span out_p,
                                                     const float* __restrict__ mu1, float lambda, float scale,
@@ -1412,7 +1411,7 @@ int launch_strided3(kfbi_handle* h, int mode, bool solve, T* work, const T* mu1,
       const CUtensorMap& min = h->tmap[second][ps.in.hi - ps.in.lo < N][mode];
       const CUtensorMap& mout = h->tmap[second][ps.out.hi - ps.out.lo < N][mode];
       const int tiles = (N / TMA_W) * (ps.planes.hi - ps.planes.lo);
-      const int nb = (solve ? tma_blocks<true>() : tma_blocks<false>()) * h->sms;
+      const int nb = TMA_BLOCKS * h->sms;
       const int grid = tiles < nb ? tiles : nb;
       const bool part = ps.planes.hi - ps.planes.lo < N - 1 || ps.in.hi - ps.in.lo < N || ps.out.hi - ps.out.lo < N;
       auto go = [&](auto kernel, int reps) -> int {

@@ -239,14 +239,13 @@ __global__ void k_predict(const double* __restrict__ psiF, const double* __restr
   }
 }
 
-// Inference of the whole network in one persistent kernel (the training
-// path keeps the layer-by-layer kernels, whose activations the backward pass
-// needs).  The bfloat16 weights are staged in shared memory once per block;
-// per tile of 64 rows each layer runs on the tensor cores from the tile's
-// activations in shared memory, the float32 products go to a shared staging
-// tile, and the epilogue adds the bias, applies SiLU and rounds to bfloat16
-// in place; the output layer is one warp dot product per row.  Same
-// operations and summation order per element as the layer-by-layer path.
+// Inference of the whole network in one persistent kernel (training has
+// k_mlp_step, which also keeps what the backward pass needs).  The bfloat16
+// weights are staged in shared memory once per block; per tile of 64 rows
+// each layer runs on the tensor cores from the tile's activations in shared
+// memory, the float32 products go to a shared staging tile, and the epilogue
+// adds the bias, applies SiLU and rounds to bfloat16 in place; the output
+// layer is one warp dot product per row.
 constexpr int IR = 64;                      // rows per tile
 constexpr int LDW = WID + 8, LDX = KIN + 8;  // padded bf16 leading dimensions
 constexpr int LDS = WID + 4;                 // padded float32 staging

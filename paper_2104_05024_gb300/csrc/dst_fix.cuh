@@ -42,7 +42,7 @@
 // Measured (GB300, CUDA events): a 256^3 float64 box solve took 4.16 ms with
 // float64 butterflies (26 float64 instructions per point and transform, at
 // 1/32 of the integer rate) and takes 0.76 ms; its error against dense
-// float64 products went from 5.3e-15 to 2.2e-15 (2-norm, smooth field).
+// float64 products went from 5.3e-15 to 1.9e-15 (2-norm, smooth field).
 //
 // The decomposition is that of dst_reg.cuh (two-level FFT m = a + 8q, k = k1
 // + P k2, one exchange, split pairs in registers, segmented scan); here the

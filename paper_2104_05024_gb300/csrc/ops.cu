@@ -176,19 +176,22 @@ struct ResArgs {
   const float *sh, *sl;  // pair source (may be the outputs themselves)
   float *res, *res_lo;
 };
-// A thread takes one x and RES_ROWS rows of a plane, the rows above and below
+// A thread takes one x and `rows` rows of a plane, the rows above and below
 // in registers (one block per line of two nodes a thread was bound by its
-// index arithmetic and loads: 70 / 134 us for one round / PAIR at 256^3).
+// index arithmetic and loads: 70 / 134 us for one round / PAIR at 256^3): up
+// to RES_ROWS, fewer on grids that would leave the chip short of blocks, where
+// the rows are a serial chain (residual_rows).
 constexpr int RES_T = 128, RES_ROWS = 8;
 template <bool NEUMANN, Src SRC, bool PAIR>
-__global__ void __launch_bounds__(RES_T) k_residual_ff(GridParams gr, const float* __restrict__ u32, ResArgs A) {
+__global__ void __launch_bounds__(RES_T) k_residual_ff(GridParams gr, const float* __restrict__ u32, ResArgs A,
+                                                       int rows) {
   // n values per field row, P per work-grid row (Neumann box: the grid is
   // the field, a neighbour beyond the box its mirror image; Dirichlet box:
   // index 0 of the grid and what lies beyond its last index is zero)
   const int n = NEUMANN ? gr.N + 1 : gr.N - 1, P = NEUMANN ? gr.N + 1 : gr.N;
-  const int x = blockIdx.x * RES_T + threadIdx.x, y0 = blockIdx.y * RES_ROWS, z = blockIdx.z;
+  const int x = blockIdx.x * RES_T + threadIdx.x, y0 = blockIdx.y * rows, z = blockIdx.z;
   if (x >= n) return;
-  const int y1 = min(n, y0 + RES_ROWS);
+  const int y1 = min(n, y0 + rows);
   const int64_t PP = (int64_t)P * P;
   const bool d3 = gr.dim == 3;
   const float* up = u32 + x + (NEUMANN ? (int64_t)z * PP + (int64_t)y0 * P
@@ -1126,14 +1129,23 @@ static FTrip ftrip(double v) {
   return {a, b, (float)(r - (double)b)};
 }
 
+// rows per thread: doubled while the blocks exceed what the chip holds at once
+// (16 of RES_T threads per SM)
+static int residual_rows(const kfbi_handle* h, int n) {
+  const int64_t lines = (int64_t)((n + RES_T - 1) / RES_T) * (h->grid.dim == 3 ? n : 1);
+  int rows = 1;
+  while (rows < RES_ROWS && lines * ((n + rows - 1) / rows) > 16 * (int64_t)h->sms) rows *= 2;
+  return rows;
+}
+
 template <Src SRC, bool PAIR>
 static void residual_ff(kfbi_handle* h, const float* u32, const ResArgs& A) {
-  const int n = field_n(h->grid);
-  const dim3 grid((n + RES_T - 1) / RES_T, (n + RES_ROWS - 1) / RES_ROWS, h->grid.dim == 3 ? n : 1);
+  const int n = field_n(h->grid), rows = residual_rows(h, n);
+  const dim3 grid((n + RES_T - 1) / RES_T, (n + rows - 1) / rows, h->grid.dim == 3 ? n : 1);
   if (h->grid.bc == KFBI_BOX_NEUMANN)
-    k_residual_ff<true, SRC, PAIR><<<grid, RES_T, 0, h->stream>>>(h->grid, u32, A);
+    k_residual_ff<true, SRC, PAIR><<<grid, RES_T, 0, h->stream>>>(h->grid, u32, A, rows);
   else
-    k_residual_ff<false, SRC, PAIR><<<grid, RES_T, 0, h->stream>>>(h->grid, u32, A);
+    k_residual_ff<false, SRC, PAIR><<<grid, RES_T, 0, h->stream>>>(h->grid, u32, A, rows);
 }
 
 int launch_residual_ff(kfbi_handle* h, const double* src, double alpha, const double* corr, const float* u32,

@@ -2149,9 +2149,20 @@ __device__ __forceinline__ void dct_tile(typename C::T* s, const typename C::T* 
   }
 }
 
+// Whether the Neumann box's x passes take a line's values together (on; plain:
+// but not on the way out where nothing is loaded there).  Not in float64,
+// whose passes are bound by the transform (box solve 5.48 instead of 5.43 ms
+// at 256^3, 821 instead of 804 us at 128^3), nor for lines so short that a
+// warp has too few values to batch (float32 solve at 64^3 38.9 instead of 36.9
+// us with the results batched too).
+template <typename T, int N>
+struct NBatch {
+  static constexpr bool on = sizeof(T) == 4 && N >= 64, plain = N < 128;
+};
+
 // The W x-lines y0 .. y0 + W - 1 (zero beyond y = N) of a plane of the
 // Neumann layout to the tile s[x][line], mapped by f; a line's loads are
-// issued together (as in fill_lines).
+// issued together (as in fill_lines; N >= 32).
 template <typename C, typename S, typename F>
 __device__ __forceinline__ void fill_lines_n(typename C::T* s, const S* __restrict__ src, int y0, const F& f) {
   constexpr int N = C::N, W = C::W, RS = C::RS, P = N + 1;
@@ -2198,15 +2209,12 @@ __global__ void __launch_bounds__(NT) k_nxfwd(T* __restrict__ a, const double* _
   const int y0 = blockIdx.x * W;
   const int z = DIM == 3 ? blockIdx.y : 0;
   const size_t plane = (size_t)z * P * P;
-  // float64 passes are bound by the transform: with their lines' loads issued
-  // together, here and in k_nxinv, the box solve took 5.48 instead of 5.43 ms
-  // at 256^3 and 821 instead of 804 us at 128^3
-  if constexpr (sizeof(T) == 8) {
+  if constexpr (!NBatch<T, N>::on) {
     for (int idx = threadIdx.x; idx < P * W; idx += NT) {
       const int x = idx % P, c = idx / P, y = y0 + c;
       T v = (T)0;
       if (y <= N) {
-        if (src != nullptr) v = alpha * src[plane + (size_t)y * P + x];
+        if (src != nullptr) v = (T)alpha * to_T<T>(src[plane + (size_t)y * P + x]);
         else if (src32 != nullptr) v = (T)src32[plane + (size_t)y * P + x];
       }
       s[x * RS + c] = v;
@@ -2269,7 +2277,8 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
   copy_async_wait();
   __syncthreads();
   dct_tile<C>(s, tw, sinv, tot, x1);
-  if constexpr (sizeof(T) == 8) {
+  const bool batch = NBatch<T, N>::on && (!NBatch<T, N>::plain || aux32 != nullptr || aux != nullptr);
+  if (!NBatch<T, N>::on || !batch) {
     for (int idx = threadIdx.x; idx < P * W; idx += NT) {
       const int x = idx % P, c = idx / P, y = y0 + c;
       if (y > N) continue;
@@ -2277,13 +2286,16 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
       const T v = s[x * RS + c];
       if (keep) a[o] = v;
       if (out != nullptr) {
-        const double bv = (T)beta * v;
-        out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
+        const double bv = to_double((T)beta * v);
+        if (sizeof(T) == 4 && aux32 != nullptr)
+          out[o] = bv + ffl::widen(aux32[o]);
+        else
+          out[o] = aux != nullptr ? fma(gamma, aux[o], bv) : bv;
       }
     }
-  } else {
-    constexpr int LW = N < 32 ? N : 32, PER = N / LW, CH = batch_of(PER);
-    const int lane = threadIdx.x % LW;
+  } else if constexpr (NBatch<T, N>::on) {
+    constexpr int PER = N / 32, CH = batch_of(PER);
+    const int lane = threadIdx.x & 31;
     const T b_t = (T)beta;
     auto put = [&](size_t o, T v, double w) {
       if (keep) a[o] = v;
@@ -2294,16 +2306,16 @@ __global__ void __launch_bounds__(NT) k_nxinv(T* __restrict__ a, bool keep, doub
     };
     auto other = [&](size_t o) { return aux32 != nullptr ? ffl::widen(aux32[o]) : aux != nullptr ? aux[o] : 0.0; };
 #pragma unroll 1
-    for (int c = threadIdx.x / LW; c < W; c += NT / LW) {
+    for (int c = threadIdx.x / 32; c < W; c += NT / 32) {
       if (y0 + c > N) continue;
       const size_t o = plane + (size_t)(y0 + c) * P + lane;
 #pragma unroll
       for (int i0 = 0; i0 < PER; i0 += CH) {
         double w[CH];
 #pragma unroll
-        for (int i = 0; i < CH; ++i) w[i] = other(o + LW * (i0 + i));
+        for (int i = 0; i < CH; ++i) w[i] = other(o + 32 * (i0 + i));
 #pragma unroll
-        for (int i = 0; i < CH; ++i) put(o + LW * (i0 + i), s[(lane + LW * (i0 + i)) * RS + c], w[i]);
+        for (int i = 0; i < CH; ++i) put(o + 32 * (i0 + i), s[(lane + 32 * (i0 + i)) * RS + c], w[i]);
       }
       if (lane == 0) put(o + N, s[N * RS + c], other(o + N));
     }

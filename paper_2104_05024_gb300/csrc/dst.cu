@@ -1092,7 +1092,7 @@ __global__ void __launch_bounds__(ZTri<T, N>::NTH) k_ztri(T* __restrict__ a, con
 // neighbouring rows are nearly equal, so a shared error of theirs adds up over
 // the rows that a mode remembers (z stage error at 48 rows 5.5e-16 ->
 // 4.5e-16).  Two Newton steps from the float reciprocal, the second on the
-// pair d + e = 1 + s (a table of 256^3 / 2 values in 0.16 ms, 0.27 ms by a
+// pair d + e = 1 + s (a table of 256^3 / 2 values in 0.13 ms, 0.27 ms by a
 // division and a correction after it, 0.12 ms by the division alone).
 __device__ __forceinline__ double ztab_pivot(double s) {
   const double d = 1.0 + s;
@@ -1111,11 +1111,15 @@ __global__ void k_ztab(const double* __restrict__ mu1, double lambda, double h2,
   double* t = tab + (size_t)q * M * N + p;
   double s = 1.0 + eps, g = ztab_pivot(s);
   t[N] = g;
-  for (int j = 2; j < M; ++j) {
-    s = fma(s, g, eps);
+  int j = 2;
+  for (; j < M; ++j) {
+    const double next = fma(s, g, eps);
+    if (next == s) break;  // the pivots have converged: most modes, within a few rows
+    s = next;
     g = ztab_pivot(s);
     t[(size_t)j * N] = g;
   }
+  for (; j < M; ++j) t[(size_t)j * N] = g;
   t[0] = 1.0 / fma(2.0 * s, g, eps);
 }
 
